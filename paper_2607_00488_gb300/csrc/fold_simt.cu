@@ -31,12 +31,68 @@
 namespace srw {
 namespace {
 
-constexpr int BM = 64;    // points per block
-constexpr int BN = 128;   // rec bins per block
-constexpr int BK = 16;
-constexpr int THR = 256;  // 16 x 16 threads
-constexpr int TM = 4;     // points per thread
-constexpr int TN = 8;     // rec bins per thread
+constexpr int kTile = 128;  // rec bins per tile of the transposed response copy
+constexpr int BK = 16;      // true bins per K tile (and per FMA chain)
+constexpr int THR = 128;
+constexpr int kRing = 4;    // K tiles of R in flight or in use
+constexpr int kNC = kNB - 1;  // monomials of a point's deviation (the constant one is always in the reference)
+
+// Thread block: MI x NI groups of 4 points x 4 rec bins a thread, a warp 8 x 4
+// lanes of them, four warps side by side along the bins.
+//   <2, 2>: 64 points x 128 bins.  A thread's 8 x 8 outputs take four 128-bit
+//           shared loads per 64 FMAs, half of the 4 x 8 outputs' six, which
+//           kept the kernel at the shared-memory limit (26 % of the FP32 rate);
+//           with 240 registers two blocks of four warps share an SM, and the
+//           one's epilogue and W production run beside the other's FMAs.
+//   <1, 1>: 32 points x 64 bins, for grids of fewer large tiles than SMs.
+template <int MI, int NI>
+struct SimtShape {
+  static constexpr int BM = MI * 32, BN = NI * 64;
+  static constexpr int kRow = BN + 16;  // floats per true bin of a ring slot: R, then the 14 spectra values (16)
+  static constexpr int kWPer = BM * BK / THR;  // W elements a thread forms per K tile
+};
+
+// Packed pairs of FP32: each half is the IEEE operation, so values are those of the scalar forms.
+__device__ __forceinline__ uint64_t pk(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpk(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
 // Coupling monomials c_b(theta) (see srw_internal.h) in double-float
 // arithmetic, returned as hi + lo float pairs so that W carries no per-theta
@@ -49,206 +105,327 @@ __device__ __forceinline__ void coefficients(const float* th, dfloat s, const Co
                          df_mul(grt, grt), {-y.hi, -y.lo}, {1.f, 0.f}, two_prod(th[4], th[4])};
 #pragma unroll
   for (int b = 0; b < kNB; ++b) {
+    if (b == 6) continue;
     const dfloat d = df_add(c[b], dfloat{-ref.hi[b], -ref.lo[b]});  // deviation from the reference point
-    hi[b] = d.hi;
-    lo[b] = d.lo;
+    hi[b < 6 ? b : 6] = d.hi;
+    lo[b < 6 ? b : 6] = d.lo;
   }
 }
 
-__global__ void __launch_bounds__(THR, 2)
-fold_simt_kernel(const float* __restrict__ theta, int P, dfloat sin2w, CoefRef cref, const float* __restrict__ shat,
-                 const float* __restrict__ shat_lo, int k_pad, const float* __restrict__ R, int n_rec, int ld,
-                 const double* __restrict__ n64, const double* __restrict__ b64,
-                 const unsigned char* __restrict__ mask, double* __restrict__ parts,
-                 float* __restrict__ musig_out, unsigned* __restrict__ status, const int2* __restrict__ krange) {
-  __shared__ float cs[BM][2 * kNB + 1];
+// R is read from a copy laid out for this kernel at create, Rt[tile of 128
+// bins][true bin][bin], and the spectra from shk[true bin][16] (seven hi, pad,
+// seven lo, pad): a K tile is then rows of contiguous floats that asynchronous
+// 16-byte copies bring in three K tiles ahead (the row-major R went through
+// registers and was transposed by four 4-byte stores per load).  order: {first
+// and end K tile holding nonzero response, rec tile, 0}, longest range first,
+// so that the last wave holds the short ones.
+template <int MI, int NI>
+__global__ void __launch_bounds__(THR, MI * NI == 4 ? 2 : 4)
+fold_simt_kernel(const float* __restrict__ theta, int P, dfloat sin2w, CoefRef cref, const float* __restrict__ shk,
+                 int k_pad, const float* __restrict__ Rt, int n_rec, const float4* __restrict__ consts,
+                 double* __restrict__ parts, float* __restrict__ musig_out, const float* __restrict__ muref,
+                 unsigned* __restrict__ status, const int4* __restrict__ order) {
+  using S = SimtShape<MI, NI>;
+  constexpr int BM = S::BM, BN = S::BN;
+  __shared__ __align__(16) float ring[kRing][BK][S::kRow];
   __shared__ __align__(16) float Ws[2][BK][BM];
-  __shared__ __align__(16) float Rs[2][BK][BN + 4];
+  __shared__ float cs[2 * kNC][BM];
 
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.x * BM, j0 = blockIdx.y * BN;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, lm = lane >> 2, ln = lane & 3;
+  const int m0 = blockIdx.x * BM;
+  const int4 od = order[blockIdx.y];
+  const int2 kr = make_int2(od.x, od.y);
+  const int j0 = od.z * BN;  // first rec bin
 
-  if (tid < BM) {
-    float hi[kNB], lo[kNB];
-    const int p = m0 + tid;
-    if (p < P) {
-      coefficients(theta + (size_t)p * 5, sin2w, cref, hi, lo);
+  for (int r = tid; r < BM; r += THR) {
+    float hi[kNC], lo[kNC];
+    if (m0 + r < P) {
+      coefficients(theta + (size_t)(m0 + r) * 5, sin2w, cref, hi, lo);
     } else {
 #pragma unroll
-      for (int b = 0; b < kNB; ++b) hi[b] = lo[b] = 0.f;
+      for (int b = 0; b < kNC; ++b) hi[b] = lo[b] = 0.f;
     }
 #pragma unroll
-    for (int b = 0; b < kNB; ++b) {
-      cs[tid][b] = hi[b];
-      cs[tid][kNB + b] = lo[b];
+    for (int b = 0; b < kNC; ++b) {
+      cs[b][r] = hi[b];
+      cs[kNC + b][r] = lo[b];
     }
   }
 
-  float acc[TM][TN], sum[TM][TN], comp[TM][TN];
-#pragma unroll
-  for (int r = 0; r < TM; ++r)
-#pragma unroll
-    for (int c = 0; c < TN; ++c) acc[r][c] = sum[r][c] = comp[r][c] = 0.f;
-
-  // K tiles of this rec tile that hold nonzero response; outside them every
-  // product is an exact zero
-  const int2 kr = krange ? krange[blockIdx.y] : make_int2(0, k_pad / BK);
-  // register staging of the next tile's R (two float4 a thread); the shat
-  // values are loaded when the tile's W is formed (kept live across the FMA
-  // loop they spilled registers at two blocks per SM)
-  const int wk = tid & (BK - 1), mg = (tid >> 4) * TM;
-  float4 rv[2];
+  const float* Rtile = Rt + (size_t)(j0 / kTile) * k_pad * kTile + (j0 % kTile);
   auto load_tile = [&](int kt) {
-    const int k0 = kt * BK;
+    if (kt < kr.y) {
+      SRW_CHECK(status, kt >= 0 && (kt + 1) * BK <= k_pad);
+      float(*dst)[S::kRow] = ring[(kt - kr.x) % kRing];
 #pragma unroll
-    for (int rr = 0; rr < 2; ++rr) {
-      const int f = tid + rr * THR, row = f >> 2, c4 = f & 3, j = j0 + row;
-      SRW_CHECK(status, k0 + c4 * 4 + 4 <= ld);
-      rv[rr] = j < n_rec ? __ldg(reinterpret_cast<const float4*>(R + (size_t)j * ld + k0 + c4 * 4))
-                         : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int q = tid; q < BK * BN / 4; q += THR) {
+        const int k = q / (BN / 4), c = (q % (BN / 4)) * 4;
+        cp_async16(&dst[k][c], Rtile + (size_t)(kt * BK + k) * kTile + c);
+      }
+      if (tid < BK * 4)
+        cp_async16(&dst[tid >> 2][BN + (tid & 3) * 4], shk + (size_t)(kt * BK + (tid >> 2)) * 16 + (tid & 3) * 4);
     }
+    cp_async_commit();  // one group per K tile, empty past the end
   };
-  auto store_tile = [&](int buf, int kt) {
-    // W^T tile: W[p][k] = sum_b c_b(p) shat_b[k], (c_hi + c_lo)(s_hi + s_lo) without lo*lo
-    float sh[kNB], sl[kNB];
+  // W^T tile: W[p][k] = sum_b c_b(p) shat_b[k], (c_hi + c_lo)(s_hi + s_lo) without lo*lo
+  auto make_w = [&](int kt) {
+    const float(*src)[S::kRow] = ring[(kt - kr.x) % kRing];
+    float(*dst)[BM] = Ws[(kt - kr.x) & 1];
+    const int p = tid % BM, kb = tid / BM * S::kWPer;
+    float ch[kNC], cl[kNC];
 #pragma unroll
-    for (int b = 0; b < kNB; ++b) {
-      sh[b] = __ldg(shat + (size_t)b * k_pad + kt * BK + wk);
-      sl[b] = __ldg(shat_lo + (size_t)b * k_pad + kt * BK + wk);
+    for (int b = 0; b < kNC; ++b) {
+      ch[b] = cs[b][p];
+      cl[b] = cs[kNC + b][p];
     }
-    float v[TM];
-#pragma unroll
-    for (int r = 0; r < TM; ++r) {
+#pragma unroll 2
+    for (int k = kb; k < kb + S::kWPer; ++k) {
+      const float4* q = reinterpret_cast<const float4*>(&src[k][BN]);
+      const float4 h0 = q[0], h1 = q[1], l0 = q[2], l1 = q[3];
+      const float sh[kNC] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z};
+      const float sl[kNC] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z};
       float s = 0.f, t = 0.f;
 #pragma unroll
-      for (int b = 0; b < kNB; ++b) {
-        s = fmaf(cs[mg + r][b], sh[b], s);
-        t = fmaf(cs[mg + r][kNB + b], sh[b], fmaf(cs[mg + r][b], sl[b], t));
+      for (int b = 0; b < kNC; ++b) {
+        s = fmaf(ch[b], sh[b], s);
+        t = fmaf(cl[b], sh[b], fmaf(ch[b], sl[b], t));
       }
-      v[r] = s + t;
-    }
-    *reinterpret_cast<float4*>(&Ws[buf][wk][mg]) = make_float4(v[0], v[1], v[2], v[3]);
-#pragma unroll
-    for (int rr = 0; rr < 2; ++rr) {  // R tile, transposed into Rs[k][j]
-      const int f = tid + rr * THR, row = f >> 2, c4 = f & 3;
-      Rs[buf][c4 * 4 + 0][row] = rv[rr].x;
-      Rs[buf][c4 * 4 + 1][row] = rv[rr].y;
-      Rs[buf][c4 * 4 + 2][row] = rv[rr].z;
-      Rs[buf][c4 * 4 + 3][row] = rv[rr].w;
+      dst[k][p] = s + t;
     }
   };
 
-  __syncthreads();  // the block's coefficients are in shared memory
-  if (kr.x < kr.y) load_tile(kr.x);
+  // packed along the bins: pair c of point row r holds bins 2c, 2c + 1 of the thread's 4 NI
+  uint64_t sum[4 * MI][2 * NI], comp[4 * MI][2 * NI];
+#pragma unroll
+  for (int r = 0; r < 4 * MI; ++r)
+#pragma unroll
+    for (int c = 0; c < 2 * NI; ++c) sum[r][c] = comp[r][c] = 0ull;
+
+#pragma unroll
+  for (int q = 0; q < kRing - 1; ++q) load_tile(kr.x + q);
+  cp_async_wait<kRing - 2>();
+  __syncthreads();  // the first K tile and the coefficients
+  if (kr.x < kr.y) make_w(kr.x);
   for (int kt = kr.x; kt < kr.y; ++kt) {
-    const int buf = (kt - kr.x) & 1;
-    // the other buffer was last read before the previous iteration's barrier
-    store_tile(buf, kt);
-    __syncthreads();
-    if (kt + 1 < kr.y) load_tile(kt + 1);  // in flight during the FMAs below
+    cp_async_wait<kRing - 3>();  // this thread's copies of K tile kt + 1
+    __syncthreads();             // everybody's, W of kt, and the end of kt - 1
+    load_tile(kt + kRing - 1);   // into the slot of kt - 1
+    const float(*rs)[S::kRow] = ring[(kt - kr.x) % kRing];
+    const float(*ws)[BM] = Ws[(kt - kr.x) & 1];
+    uint64_t acc[4 * MI][2 * NI];
 #pragma unroll
     for (int k = 0; k < BK; ++k) {
-      const float4 a = *reinterpret_cast<const float4*>(&Ws[buf][k][ty * TM]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Rs[buf][k][tx * TN]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Rs[buf][k][tx * TN + 4]);
-      const float av[TM] = {a.x, a.y, a.z, a.w};
-      const float bv[TN] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+      float a[4 * MI];
+      uint64_t b[2 * NI];
 #pragma unroll
-      for (int r = 0; r < TM; ++r)
+      for (int i = 0; i < MI; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(&ws[k][i * 32 + lm * 4]);
+        a[4 * i] = v.x; a[4 * i + 1] = v.y; a[4 * i + 2] = v.z; a[4 * i + 3] = v.w;
+      }
 #pragma unroll
-        for (int c = 0; c < TN; ++c) acc[r][c] = fmaf(av[r], bv[c], acc[r][c]);
+      for (int i = 0; i < NI; ++i) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&rs[k][warp * (16 * NI) + i * 16 + ln * 4]);
+        b[2 * i] = v.x;
+        b[2 * i + 1] = v.y;
+      }
+#pragma unroll
+      for (int r = 0; r < 4 * MI; ++r) {
+        const uint64_t aa = pk(a[r], a[r]);
+#pragma unroll
+        for (int c = 0; c < 2 * NI; ++c) acc[r][c] = k == 0 ? mul2(aa, b[c]) : fma2(aa, b[c], acc[r][c]);
+      }
     }
     // each 16-term chain is added to the running sum with Kahan compensation
 #pragma unroll
-    for (int r = 0; r < TM; ++r)
+    for (int r = 0; r < 4 * MI; ++r)
 #pragma unroll
-      for (int c = 0; c < TN; ++c) {
-        const float y = acc[r][c] - comp[r][c];
-        const float t = sum[r][c] + y;
-        comp[r][c] = (t - sum[r][c]) - y;
+      for (int c = 0; c < 2 * NI; ++c) {
+        const uint64_t y = sub2(acc[r][c], comp[r][c]);
+        const uint64_t t = add2(sum[r][c], y);
+        comp[r][c] = sub2(sub2(t, sum[r][c]), y);
         sum[r][c] = t;
-        acc[r][c] = 0.f;
       }
+    if (kt + 1 < kr.y) make_w(kt + 1);
   }
+  cp_async_wait<0>();
 
-  if (musig_out != nullptr) {  // batched folded spectra
+  const int jw = j0 + warp * (16 * NI) + ln * 4;  // bins jw + 16 i + 0..3
+  if (musig_out != nullptr) {  // batched folded spectra: deviation + reference fold
 #pragma unroll
-    for (int r = 0; r < TM; ++r) {
-      const int p = m0 + ty * TM + r;
-      if (p >= P) continue;
+    for (int i = 0; i < NI; ++i)
 #pragma unroll
-      for (int c = 0; c < TN; ++c) {
-        const int j = j0 + tx * TN + c;
-        if (j < n_rec) musig_out[(size_t)p * n_rec + j] = sum[r][c] - comp[r][c];
+      for (int c = 0; c < 4; ++c) {
+        const int j = jw + 16 * i + c;
+        if (j >= n_rec) continue;
+        const float ref = __ldg(muref + j);
+#pragma unroll
+        for (int r = 0; r < 4 * MI; ++r) {
+          const int p = m0 + (r / 4) * 32 + lm * 4 + (r & 3);
+          const float2 s2 = unpk(sum[r][2 * i + c / 2]), c2 = unpk(comp[r][2 * i + c / 2]);
+          const float v = (c & 1) ? s2.y - c2.y : s2.x - c2.x;
+          if (p < P) musig_out[(size_t)p * n_rec + j] = v + ref;
+        }
       }
-    }
   }
   if (parts == nullptr) return;
-  // Epilogue: Poisson terms (FP64) over this block's rec bins, per point.
-  double nj[TN], bj[TN];
-  bool on[TN];
+  // Epilogue: Poisson terms over this block's rec bins per point, in double-
+  // float: FP64 (a warp's instruction takes the SM's unit 16 cycles) spent
+  // 0.7 ms of a 4096-point call's 2.7 ms on the logarithms here.
+  dfloat d[4 * MI];
+  bool inf[4 * MI];
 #pragma unroll
-  for (int c = 0; c < TN; ++c) {
-    const int j = j0 + tx * TN + c;
-    on[c] = j < n_rec && (mask == nullptr || mask[j] != 0);
-    nj[c] = on[c] ? n64[j] : 0.0;
-    bj[c] = on[c] ? b64[j] : 0.0;
+  for (int r = 0; r < 4 * MI; ++r) {
+    d[r] = {0.f, 0.f};
+    inf[r] = false;
   }
 #pragma unroll
-  for (int r = 0; r < TM; ++r) {
-    double d = 0.0;
+  for (int c = 0; c < 4 * NI; ++c) {
+    const int j = jw + 16 * (c / 4) + (c & 3);
+    if (j >= n_rec) continue;
+    const float4 nb = __ldg(consts + 2 * j), mk = __ldg(consts + 2 * j + 1);  // {n, n lo, b, b lo}, {mask, ...}
+    if (mk.x == 0.f) continue;
 #pragma unroll
-    for (int c = 0; c < TN; ++c) {
-      if (on[c]) d += poisson_term_f64(((double)sum[r][c] - (double)comp[r][c]) + bj[c], nj[c]);
+    for (int r = 0; r < 4 * MI; ++r) {
+      const float2 s2 = unpk(sum[r][c / 2]), c2 = unpk(comp[r][c / 2]);
+      const dfloat dev = two_sum((c & 1) ? s2.y : s2.x, (c & 1) ? -c2.y : -c2.x);
+      const dfloat t = poisson_term_df(df_add(dev, dfloat{nb.z, nb.w}), dfloat{nb.x, nb.y});
+      if (isinf(t.hi)) inf[r] = true;
+      else d[r] = df_add(d[r], t);
     }
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-    const int p = m0 + ty * TM + r;
-    if (tx == 0 && p < P) parts[(size_t)blockIdx.y * P + p] = d;
   }
+  // the ring is free (its last copies landed above): the warps' sums per point
+  float2(*psum)[BM] = reinterpret_cast<float2(*)[BM]>(&ring[0][0][0]);
+  int(*pinf)[BM] = reinterpret_cast<int(*)[BM]>(&ring[1][0][0]);
+  static_assert(sizeof(float2) * 4 * BM <= sizeof(ring[0]), "sums of four warps in a ring slot");
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < 4 * MI; ++r) {
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+      d[r] = df_add(d[r], df_shfl_xor(d[r], o));
+      inf[r] = __shfl_xor_sync(0xffffffffu, (int)inf[r], o) || inf[r];
+    }
+    if (ln == 0) {
+      const int q = (r / 4) * 32 + lm * 4 + (r & 3);
+      psum[warp][q] = make_float2(d[r].hi, d[r].lo);
+      pinf[warp][q] = inf[r];
+    }
+  }
+  __syncthreads();
+  for (int q = tid; q < BM; q += THR)
+    if (m0 + q < P) {
+      double s = 0.0;
+      bool any = false;
+      for (int w = 0; w < 4; ++w) {
+        s += (double)psum[w][q].x + (double)psum[w][q].y;
+        any |= pinf[w][q] != 0;
+      }
+      parts[(size_t)od.z * P + m0 + q] = any ? __longlong_as_double(0x7ff0000000000000LL) : s;
+    }
+}
+
+// Rt[tile][k][128] from the row-major R (zero beyond n_rec), and shk[k][16].
+__global__ void simt_layout_kernel(const float* __restrict__ R, int n_rec, int ld, int k_pad,
+                                   float* __restrict__ Rt) {
+  __shared__ float s[32][33];
+  const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;  // 32 true bins x 32 rec bins
+  for (int i = threadIdx.y; i < 32; i += 8) {
+    const int j = r0 + i, k = k0 + threadIdx.x;
+    s[i][threadIdx.x] = j < n_rec && k < ld ? R[(size_t)j * ld + k] : 0.f;
+  }
+  __syncthreads();
+  const int t = r0 / kTile;
+  for (int i = threadIdx.y; i < 32; i += 8)
+    Rt[((size_t)t * k_pad + k0 + i) * kTile + r0 % kTile + threadIdx.x] = s[threadIdx.x][i];
+}
+__global__ void simt_spectra_kernel(const float* __restrict__ shat, const float* __restrict__ shat_lo, int k_pad,
+                                    float* __restrict__ shk) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= k_pad) return;
+#pragma unroll
+  for (int b = 0; b < kNC; ++b) {
+    const int src = b < 6 ? b : 7;
+    shk[(size_t)k * 16 + b] = shat[(size_t)src * k_pad + k];
+    shk[(size_t)k * 16 + 8 + b] = shat_lo[(size_t)src * k_pad + k];
+  }
+  shk[(size_t)k * 16 + 7] = shk[(size_t)k * 16 + 15] = 0.f;
+}
+
+template <int MI, int NI>
+void launch_shape(const srw_ctx* h, const float* theta, int P, double* parts, cudaStream_t s, float* musig_out,
+                  const int4* order) {
+  using S = SimtShape<MI, NI>;
+  const dim3 grid((P + S::BM - 1) / S::BM, (h->n_rec + S::BN - 1) / S::BN);
+  fold_simt_kernel<MI, NI><<<grid, THR, 0, s>>>(theta, P, df_from_double(h->sin2w), h->cref, h->d_simt_sh, h->k_pad,
+                                                h->d_simt_r, h->n_rec, h->d_simt_c, parts, musig_out, h->d_muref32,
+                                                h->d_status, order);
+}
+
+// The small tile where the large ones do not give every SM a block.
+bool small_tile(const srw_ctx* h, int P) {
+  const long long blocks = ((P + 63LL) / 64) * ((h->n_rec + 127) / 128);
+  return blocks < h->sm_count;
 }
 
 }  // namespace
 
-int fold_simt_parts(int n_rec) { return (n_rec + BN - 1) / BN; }
+int fold_simt_parts(const srw_ctx* h, int P) {
+  const int bn = small_tile(h, P) ? 64 : 128;
+  return (h->n_rec + bn - 1) / bn;
+}
 
 cudaError_t launch_fold_simt(const srw_ctx* h, const float* theta, int P, double* parts, cudaStream_t s,
                              int* n_parts, float* musig_out) {
-  const dim3 grid((P + BM - 1) / BM, (h->n_rec + BN - 1) / BN);
-  fold_simt_kernel<<<grid, THR, 0, s>>>(theta, P, df_from_double(h->sin2w), h->cref, h->d_shat, h->d_shat_lo, h->k_pad, h->d_R, h->n_rec,
-                                        h->ld_r, h->d_n64, h->d_bref64, h->d_mask, parts, musig_out, h->d_status,
-                                        h->d_simt_kr);
-  if (n_parts) *n_parts = (int)grid.y;
+  if (small_tile(h, P)) launch_shape<1, 1>(h, theta, P, parts, s, musig_out, h->d_simt_kr + (h->n_rec + 127) / 128);
+  else launch_shape<2, 2>(h, theta, P, parts, s, musig_out, h->d_simt_kr);
+  if (n_parts) *n_parts = fold_simt_parts(h, P);
   return launch_result();
 }
 
-// Per rec tile of BN bins the K tiles [first, end) between its first and last
-// nonzero column of R (FP32, exact zeros outside; a tile without any nonzero
-// element gets an empty range).
-cudaError_t simt_prepare(srw_ctx* h, const std::vector<float>& R) {
-  const int nt = fold_simt_parts(h->n_rec), n_kt = h->k_pad / BK, cols = std::min(h->ld_r, h->k_pad);
-  std::vector<int2> kr(nt);
-  for (int t = 0; t < nt; ++t) {
-    int first = cols, last = -1;
-    for (int j = t * BN; j < std::min(h->n_rec, (t + 1) * BN); ++j) {
-      const float* row = R.data() + (size_t)j * h->ld_r;
-      for (int k = 0; k < first; ++k)
-        if (row[k] != 0.f) {
-          first = k;
-          break;
-        }
-      for (int k = cols - 1; k > last; --k)
-        if (row[k] != 0.f) {
-          last = k;
-          break;
-        }
+// Per rec tile of 128 and of 64 bins the K tiles [first, end) between its
+// first and last nonzero column of R (FP32, exact zeros outside; a tile
+// without any nonzero element gets an empty range), longest first; and the
+// kernel's copies of R and of the coefficient spectra.
+cudaError_t simt_prepare(srw_ctx* h, const std::vector<float>& R, cudaStream_t s) {
+  const int n_kt = h->k_pad / BK, cols = std::min(h->ld_r, h->k_pad);
+  std::vector<int4> kr;
+  for (int bn = 128; bn >= 64; bn -= 64) {
+    const size_t first_of = kr.size();
+    for (int t = 0; t * bn < h->n_rec; ++t) {
+      int first = cols, last = -1;
+      for (int j = t * bn; j < std::min(h->n_rec, (t + 1) * bn); ++j) {
+        const float* row = R.data() + (size_t)j * h->ld_r;
+        for (int k = 0; k < first; ++k)
+          if (row[k] != 0.f) {
+            first = k;
+            break;
+          }
+        for (int k = cols - 1; k > last; --k)
+          if (row[k] != 0.f) {
+            last = k;
+            break;
+          }
+      }
+      kr.push_back(last < 0 ? make_int4(0, 0, t, 0) : make_int4(first / BK, std::min(n_kt, last / BK + 1), t, 0));
     }
-    kr[t] = last < 0 ? make_int2(0, 0) : make_int2(first / BK, std::min(n_kt, last / BK + 1));
+    std::stable_sort(kr.begin() + first_of, kr.end(),
+                     [](const int4& a, const int4& b) { return a.y - a.x > b.y - b.x; });
   }
+  const int nt = (h->n_rec + kTile - 1) / kTile;
+  const size_t bytes[3] = {sizeof(int4) * kr.size(), sizeof(float) * (size_t)nt * kTile * h->k_pad,
+                           sizeof(float) * 16 * (size_t)h->k_pad};
   cudaError_t e = cudaSuccess;
-  if (!h->d_simt_kr && (e = dev_malloc(&h->d_simt_kr, sizeof(int2) * (size_t)nt)) != cudaSuccess) return e;
-  h->device_bytes += sizeof(int2) * (size_t)nt;
-  return cudaMemcpy(h->d_simt_kr, kr.data(), sizeof(int2) * (size_t)nt, cudaMemcpyHostToDevice);
+  if (!h->d_simt_kr && (e = dev_malloc(&h->d_simt_kr, bytes[0])) != cudaSuccess) return e;
+  if (!h->d_simt_r && (e = dev_malloc(&h->d_simt_r, bytes[1])) != cudaSuccess) return e;
+  if (!h->d_simt_sh && (e = dev_malloc(&h->d_simt_sh, bytes[2])) != cudaSuccess) return e;
+  h->device_bytes += bytes[0] + bytes[1] + bytes[2];
+  simt_layout_kernel<<<dim3(h->k_pad / 32, nt * (kTile / 32)), dim3(32, 8), 0, s>>>(h->d_R, h->n_rec, h->ld_r,
+                                                                                    h->k_pad, h->d_simt_r);
+  simt_spectra_kernel<<<(h->k_pad + 255) / 256, 256, 0, s>>>(h->d_shat, h->d_shat_lo, h->k_pad, h->d_simt_sh);
+  if ((e = launch_result()) != cudaSuccess) return e;
+  return cudaMemcpyAsync(h->d_simt_kr, kr.data(), bytes[0], cudaMemcpyHostToDevice, s) == cudaSuccess
+             ? cudaStreamSynchronize(s)
+             : cudaErrorUnknown;
 }
 
 }  // namespace srw

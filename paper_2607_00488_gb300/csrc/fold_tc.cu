@@ -450,20 +450,30 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
             // {n_j (0 where masked), b_j + R W_ref - n_j, mask, 1/r_j}; padding columns add nothing
             dj[k] = j < n_rec ? __ldg(G.nb4 + j) : make_float4(0.f, 1.f, 0.f, 0.f);
           }
-        } else {  // folded spectra only (no data needed): just the row scales
+        } else {  // folded spectra only (no data needed): the row scales and the reference fold
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
             const int j = n0 + c0 + k;
-            dj[k] = make_float4(0.f, 0.f, 0.f, F16 && j < n_rec ? __ldg(G.rinv + j) : 0.f);
+            dj[k] = j < n_rec ? make_float4(0.f, 0.f, __ldg(G.muref + j), F16 ? __ldg(G.rinv + j) : 0.f)
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
           }
         }
         float v[16];
         tmem_ld16(tbase + (uint32_t)c0, v);
         if (musig_out != nullptr && p < P) {  // batched folded spectra (row p)
-          float* row = musig_out + (size_t)(G.p_off + p) * n_rec;
+          float* row = musig_out + (size_t)(G.p_off + p) * n_rec + n0 + c0;
+          // scaled, rounded, then the reference fold added
 #pragma unroll
-          for (int k = 0; k < 16; ++k)
-            if (n0 + c0 + k < n_rec) row[n0 + c0 + k] = F16 ? v[k] * (sinv * dj[k].w) : v[k];
+          for (int k = 0; k < 16; ++k) v[k] = __fadd_rn(F16 ? __fmul_rn(v[k], sinv * dj[k].w) : v[k], dj[k].z);
+          if ((n_rec & 3) == 0 && n0 + c0 + 16 <= n_rec && (reinterpret_cast<uint64_t>(musig_out) & 15u) == 0) {
+#pragma unroll
+            for (int k = 0; k < 16; k += 4)  // rows of 16-byte multiples: a thread's 64 bytes in four stores
+              *reinterpret_cast<float4*>(row + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+          } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+              if (n0 + c0 + k < n_rec) row[k] = v[k];
+          }
         }
         if (parts != nullptr) {
           float ts = 0.f;
@@ -991,6 +1001,7 @@ TcGroup tc_group_of(const srw_ctx* h, int bn, bool f16) {
   G.sin2w_lo = s2w.lo;
   G.cref = h->cref;
   G.rinv = h->d_rinv;
+  G.muref = h->d_muref32;
   for (int b = 0; b < kNB; ++b) G.wmax[b] = h->wmax[b];
   return G;
 }

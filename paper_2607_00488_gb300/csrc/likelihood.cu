@@ -322,14 +322,16 @@ __global__ void data_prepare_kernel(const double* __restrict__ bkg, int n_bkg, i
 // in FP64 (SIMT fold) and as floats with the count and the mask (tensor fold).
 __global__ void data_ref_kernel(const double* __restrict__ n64, const double* __restrict__ b64,
                                 const double* __restrict__ muref, const unsigned char* __restrict__ mask, int n_rec,
-                                const float* __restrict__ rinv, double* __restrict__ bref64, float4* __restrict__ nbm,
+                                const float* __restrict__ rinv, double* __restrict__ bref64, float4* __restrict__ simt_c,
                                 float2* __restrict__ nb2, float4* __restrict__ nb4) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n_rec) return;
   const double br = b64[j] + muref[j];
   bref64[j] = br;
   const bool on = mask == nullptr || mask[j] != 0;
-  nbm[j] = make_float4((float)n64[j], (float)br, on ? 1.f : 0.f, 0.f);
+  const dfloat nd = df_from_double(n64[j]), bd = df_from_double(br);
+  simt_c[2 * j] = make_float4(nd.hi, nd.lo, bd.hi, bd.lo);
+  simt_c[2 * j + 1] = make_float4(on ? 1.f : 0.f, 0.f, 0.f, 0.f);
   nb2[j] = make_float2(on ? (float)n64[j] : -1.f, (float)br);
   // tensor-core epilogue: mu - n is formed from b + R W_ref - n, rounded once from FP64
   if (nb4) nb4[j] = make_float4(on ? (float)n64[j] : 0.f, (float)(on ? br - n64[j] : br), on ? 1.f : 0.f,
@@ -527,23 +529,10 @@ cudaError_t launch_set_data(srw_ctx* h, const double* d_bkg, int n_bkg, cudaStre
 cudaError_t launch_data_ref(srw_ctx* h, cudaStream_t s) {
   const int thr = 256;
   data_ref_kernel<<<(h->n_rec + thr - 1) / thr, thr, 0, s>>>(h->d_n64, h->d_b64, h->d_muref64, h->d_mask, h->n_rec,
-                                                             h->d_rinv, h->d_bref64, h->d_nbm, h->d_nb2, h->d_nb4);
+                                                             h->d_rinv, h->d_bref64, h->d_simt_c, h->d_nb2, h->d_nb4);
   cudaError_t e = launch_result();
   if (e == cudaSuccess && h->d_lin) e = launch_linear_consts(h, s);
   return e;
-}
-
-// out[p][j] += mu_ref[j]: folded spectra of the batched path from deviations.
-__global__ void add_ref_kernel(float* __restrict__ out, const double* __restrict__ muref, int P, int n_rec) {
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)P * n_rec) return;
-  out[idx] += (float)muref[idx % n_rec];
-}
-
-cudaError_t launch_add_ref(const srw_ctx* h, float* out, int P, cudaStream_t s) {
-  const size_t n = (size_t)P * h->n_rec;
-  add_ref_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(out, h->d_muref64, P, h->n_rec);
-  return launch_result();
 }
 
 }  // namespace srw

@@ -10,6 +10,8 @@
 
 #include <cuda_runtime.h>
 
+#include "dfloat.cuh"
+
 namespace srw {
 
 // FP64 term (single-point path).  mu < 0, or mu == 0 with n > 0, gives +inf.
@@ -18,6 +20,49 @@ __device__ __forceinline__ double poisson_term_f64(double mu, double n) {
   if (n == 0.0) return mu;
   if (mu == 0.0) return __longlong_as_double(0x7ff0000000000000LL);
   return mu - n + n * log(n / mu);
+}
+
+// The same term in double-float on the FP32 pipes, about 1e-13 relative to n
+// and mu.  With k the power of two that brings n' = n 2^-k within a factor
+// ~sqrt(2) of mu and v = (n' - mu)/(n' + mu),
+//   ln(n/mu) = k ln 2 + 2 atanh(v) = k ln 2 + 2 v (1 + v^2 (1/3 + v^2 q(v^2))),
+// |v| < 0.18; q in FP32 (its part of the bracket is below 0.007, so its
+// rounding is below 1e-9 v^3), the rest in double-float.  Same domain rules as
+// poisson_term_f64; a mu too small for FP32 quotients takes that function.
+__device__ __forceinline__ dfloat poisson_term_df(dfloat mu, dfloat n) {
+  if (n.hi == 0.f && !(mu.hi < 0.f)) return mu;
+  if (!(mu.hi > 1e-30f)) {
+    const double t = poisson_term_f64((double)mu.hi + (double)mu.lo, (double)n.hi + (double)n.lo);
+    return isfinite(t) ? df_from_double(t) : dfloat{(float)t, 0.f};
+  }
+  const float r = __fdividef(n.hi, mu.hi) * 1.41421356f;
+  int k = (__float_as_int(r) >> 23) - 127;  // r > 0: n / mu in 2^k [0.707, 1.415)
+  k = max(-100, min(100, k));
+  const float p2 = __int_as_float((127 - k) << 23);
+  const dfloat ns = {n.hi * p2, n.lo * p2};
+  const dfloat d = df_add(ns, dfloat{-mu.hi, -mu.lo}), s = df_add(ns, mu);
+  const float q0 = __fdividef(d.hi, s.hi);  // v to FP32, then one correction step
+  const dfloat q0s = two_prod(q0, s.hi);
+  const dfloat rem = df_add(d, dfloat{-q0s.hi, -fmaf(q0, s.lo, q0s.lo)});
+  const dfloat v = fast_two_sum(q0, __fdividef(rem.hi, s.hi));
+  const dfloat v2 = df_mul(v, v);
+  float q = fmaf(v2.hi, 1.f / 19.f, 1.f / 17.f);
+  q = fmaf(v2.hi, q, 1.f / 15.f);
+  q = fmaf(v2.hi, q, 1.f / 13.f);
+  q = fmaf(v2.hi, q, 1.f / 11.f);
+  q = fmaf(v2.hi, q, 1.f / 9.f);
+  q = fmaf(v2.hi, q, 1.f / 7.f);
+  q = fmaf(v2.hi, q, 1.f / 5.f);
+  const dfloat third = {0.33333334f, -9.9341072e-9f};
+  const dfloat w = df_mul(v2, df_add(third, q * v2.hi));
+  dfloat l = df_add(v, df_mul(v, w));
+  l = {2.f * l.hi, 2.f * l.lo};
+  const float kf = (float)k;
+  const dfloat ln2 = {0.69314718f, -1.9046542e-9f};
+  dfloat kl = two_prod(kf, ln2.hi);
+  kl = fast_two_sum(kl.hi, fmaf(kf, ln2.lo, kl.lo));
+  l = df_add(kl, l);
+  return df_add(df_add(mu, dfloat{-n.hi, -n.lo}), df_mul(n, l));
 }
 
 // FP32 term of the tensor-core epilogue, branch-free and without per-element

@@ -404,7 +404,7 @@ __global__ void wref_kernel(const double* __restrict__ basis, const double* __re
 }
 
 __global__ void muref_kernel(const float* __restrict__ R, int ld, int n_t, const double* __restrict__ wref,
-                             double* __restrict__ muref) {
+                             double* __restrict__ muref, float* __restrict__ muref32) {
   __shared__ double red[32];
   const int j = blockIdx.x;
   double s = 0.0;
@@ -416,6 +416,7 @@ __global__ void muref_kernel(const float* __restrict__ R, int ld, int n_t, const
     double t = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
     muref[j] = t;
+    muref32[j] = (float)t;
   }
 }
 
@@ -426,7 +427,7 @@ cudaError_t launch_reference_fold(srw_ctx* h, cudaStream_t s) {
   cudaError_t e = dev_malloc_async(&d_w, sizeof(double) * h->n_t, s);
   if (e != cudaSuccess) return e;
   wref_kernel<<<(h->n_t + 255) / 256, 256, 0, s>>>(h->d_basis, h->d_ssm64, h->d_esm64, h->n_t, h->cref, d_w);
-  muref_kernel<<<h->n_rec, 256, 0, s>>>(h->d_R, h->ld_r, h->n_t, d_w, h->d_muref64);
+  muref_kernel<<<h->n_rec, 256, 0, s>>>(h->d_R, h->ld_r, h->n_t, d_w, h->d_muref64, h->d_muref32);
   if ((e = launch_result()) != cudaSuccess) return e;
   return cudaFreeAsync(d_w, s);
 }

@@ -58,7 +58,6 @@ DataView data_view(const srw_ctx* h) {
   d.n_rec = h->n_rec;
   d.n64 = h->d_n64;
   d.b64 = h->d_b64;
-  d.nbm = h->d_nbm;
   d.mask = h->d_mask;
   d.c_data = h->d_cdata;
   return d;
@@ -137,9 +136,9 @@ static void release(srw_ctx* h) {
   for (int f = 0; f < 2; ++f)
     for (int b = 0; b < 2; ++b) dfree(h->d_kbr[f][b]);
   dfree(h->d_ssm32); dfree(h->d_esm32); dfree(h->d_shat); dfree(h->d_R); dfree(h->d_rhi); dfree(h->d_rlo); dfree(h->d_rhi16); dfree(h->d_rlo16); dfree(h->d_rinv); dfree(h->d_coef); dfree(h->d_linM); dfree(h->d_lin); dfree(h->d_linp);
-  dfree(h->d_n64); dfree(h->d_b64); dfree(h->d_muref64); dfree(h->d_bref64); dfree(h->d_nbm); dfree(h->d_nb2); dfree(h->d_nb4); dfree(h->d_mask); dfree(h->d_cdata);
+  dfree(h->d_n64); dfree(h->d_b64); dfree(h->d_muref64); dfree(h->d_bref64); dfree(h->d_simt_c); dfree(h->d_muref32); dfree(h->d_nb2); dfree(h->d_nb4); dfree(h->d_mask); dfree(h->d_cdata);
   dfree(h->d_W); dfree(h->d_S); dfree(h->d_musig); dfree(h->d_mu); dfree(h->d_part); dfree(h->d_ticket);
-  dfree(h->d_status); dfree(h->d_gv_seg); dfree(h->d_simt_kr); dfree(h->d_gv_segs); dfree(h->d_gv_rows); dfree(h->d_bpart); dfree(h->d_theta); dfree(h->d_out); dfree(h->d_theta0);
+  dfree(h->d_status); dfree(h->d_gv_seg); dfree(h->d_simt_kr); dfree(h->d_simt_r); dfree(h->d_simt_sh); dfree(h->d_gv_segs); dfree(h->d_gv_rows); dfree(h->d_bpart); dfree(h->d_theta); dfree(h->d_out); dfree(h->d_theta0);
   if (h->own_stream) cudaStreamDestroy(h->own_stream);
   h->own_stream = nullptr;
   for (auto& ev : h->ev_fold)
@@ -416,6 +415,7 @@ static cudaError_t alloc_axis(srw_ctx* h, cudaStream_t s) {
   AX(dalloc(h, &h->d_S, n_t));
   AX(dalloc(h, &h->d_musig, n_rec));
   AX(dalloc(h, &h->d_muref64, n_rec));
+  AX(dalloc(h, &h->d_muref32, n_rec));
   AX(dalloc(h, &h->d_mu, n_rec));
   h->part_cap = fold_point_grid(h);
   AX(dalloc(h, &h->d_part, h->part_cap));
@@ -741,7 +741,7 @@ static srw_status create_impl(const srw_binning* bin, const srw_source* sources,
   std::vector<float> Rh((size_t)n_rec * h->ld_r);
   CREATE_CUDA(cudaMemcpy(Rh.data(), h->d_R, sizeof(float) * Rh.size(), cudaMemcpyDeviceToHost), "read R");
   CREATE_CUDA(gemv_prepare(h, Rh), "GEMV bands");
-  CREATE_CUDA(simt_prepare(h, Rh), "FP32 fold K ranges");
+  CREATE_CUDA(simt_prepare(h, Rh, s), "FP32 fold layout");
   // ---- tensor-core path: BF16 hi/lo split of R and TMA descriptors
   if (tc_supported(h)) {
     CREATE_CUDA(dalloc(h, &h->d_rhi, (size_t)h->rec_pad * h->k_pad), "alloc R hi");
@@ -839,7 +839,7 @@ srw_status srw_set_data(srw_handle h, const double* counts, const double* bkg, i
   // call allocates the ones still missing
   if (!h->d_n64) SRW_CUDA(h, dalloc(h, &h->d_n64, n_rec), "alloc data");
   if (!h->d_b64) SRW_CUDA(h, dalloc(h, &h->d_b64, n_rec), "alloc data");
-  if (!h->d_nbm) SRW_CUDA(h, dalloc(h, &h->d_nbm, n_rec), "alloc data");
+  if (!h->d_simt_c) SRW_CUDA(h, dalloc(h, &h->d_simt_c, 2 * (size_t)n_rec), "alloc data");
   if (!h->d_nb2) SRW_CUDA(h, dalloc(h, &h->d_nb2, n_rec), "alloc data");
   if (!h->d_nb4) SRW_CUDA(h, dalloc(h, &h->d_nb4, n_rec), "alloc data");
   if (!h->d_cdata) SRW_CUDA(h, dalloc(h, &h->d_cdata, 1), "alloc data");
@@ -962,7 +962,7 @@ static srw_status loglik_impl(srw_handle h, const float* theta, int P, double* o
       if (e == cudaSuccess) e = cudaEventRecord(h->ev_fold[1], s);
       if (e != cudaSuccess) return cuda_fail(h, e, "profiled single-point fold");
     } else {
-      const int n_parts_max = precision == SRW_FP32 ? fold_simt_parts(h->n_rec) : (h->rec_pad / 128);
+      const int n_parts_max = precision == SRW_FP32 ? fold_simt_parts(h, P) : (h->rec_pad / 128);
       st = ensure_bparts(h, (size_t)n_parts_max * P);
       if (st == SRW_OK && precision != SRW_FP32) st = ensure_coef(h, P);
       if (st != SRW_OK) return st;
@@ -989,7 +989,7 @@ static srw_status loglik_impl(srw_handle h, const float* theta, int P, double* o
       return launch_fold_point_after(h, h->d_W, o, cs);
     });
   } else {
-    const int n_parts_max = precision == SRW_FP32 ? fold_simt_parts(h->n_rec) : (h->rec_pad / 128);
+    const int n_parts_max = precision == SRW_FP32 ? fold_simt_parts(h, P) : (h->rec_pad / 128);
     st = ensure_bparts(h, (size_t)n_parts_max * P);
     if (st == SRW_OK && precision != SRW_FP32) st = ensure_coef(h, P);
     if (st != SRW_OK) return st;
@@ -1155,7 +1155,6 @@ srw_status srw_spectrum_batch(srw_handle h, const float* theta, int P, float* ou
   cudaError_t e = precision == SRW_FP32
                       ? launch_fold_simt(h, th, P, nullptr, s, &n_parts, o)
                       : launch_fold_tc(h, th, P, (int)precision, h->cfg[precision], nullptr, s, &n_parts, o);
-  if (e == cudaSuccess) e = launch_add_ref(h, o, P, s);
   if (e != cudaSuccess) {
     if (d_tmp) cudaFreeAsync(d_tmp, s);
     return cuda_fail(h, e, "batched fold");

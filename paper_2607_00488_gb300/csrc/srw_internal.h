@@ -80,7 +80,6 @@ struct DataView {
   int n_rec;
   const double* n64;     // counts
   const double* b64;     // summed background
-  const float4* nbm;     // {n_j, b_j, mask_j, 0} as floats for the batched epilogue
   const unsigned char* mask;
   const double* c_data;  // device scalar: 2 sum [n - n ln n + lnGamma(n+1)]
 };
@@ -115,6 +114,7 @@ struct TcGroup {
   float sin2w_hi, sin2w_lo;
   CoefRef cref;
   const float* rinv;           // SRW_FP16X3: [n_rec] inverse power-of-two row scales of R
+  const float* muref;          // [n_rec] R W_ref (folded spectra)
   const int2* kbr;             // [n_tiles] K-block walk {first block, +-count} over the tile's nonzero response
   float wmax[kNB];             // SRW_FP16X3: max_i |shat_b,i| (bound of the weighted-spectrum deviations)
 };
@@ -188,7 +188,7 @@ struct srw_ctx {
   // data
   double* d_n64 = nullptr;
   double* d_b64 = nullptr;
-  float4* d_nbm = nullptr;
+  float4* d_simt_c = nullptr;  // [2 n_rec] FP32 fold epilogue: {n, n lo, b + R W_ref, lo}, {mask, 0, 0, 0}
   float2* d_nb2 = nullptr;     // {n_j or -1 where masked, b_j + R W_ref} (surrogate epilogue)
   float4* d_nb4 = nullptr;     // {n_j (0 where masked), b_j + R W_ref - n_j, mask 1/0, 1/r_j} (tensor-core epilogue)
   unsigned char* d_mask = nullptr;
@@ -206,7 +206,9 @@ struct srw_ctx {
   int4* d_gv_seg = nullptr;    // single-point GEMV: stream segments of every block (rows' nonzero bands)
   int* d_gv_segs = nullptr;    // [gv_blocks + 1] first segment of each GEMV block
   int* d_gv_rows = nullptr;    // [gv_blocks + 1] first row of each GEMV block (band-balanced split)
-  int2* d_simt_kr = nullptr;   // FP32 batched fold: K-tile range [first, end) of each 128-bin rec tile
+  int4* d_simt_kr = nullptr;   // FP32 batched fold: {K-tile range [first, end), rec tile, 0} of its 128-bin, then 64-bin tiles
+  float* d_simt_r = nullptr;   // R in tiles of 128 bins, [tile][k_pad][128]
+  float* d_simt_sh = nullptr;  // [k_pad][16] coefficient spectra hi (7) and lo (7), k-major
   int gv_blocks = 0, gv_max_rows = 0, gv_max_segs = 0;
   long long gv_bytes = 0;      // bytes of R the GEMV streams (the bands)
   double* d_bpart = nullptr;   // batched partials [n_tiles][P]
@@ -228,6 +230,7 @@ struct srw_ctx {
   float theta_ref[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
   srw::CoefRef cref{};          // monomials of theta_ref (zeros when use_ref == 0)
   float gref[2][10] = {};       // coupling products of theta_ref for the spectrum kernel (hi, lo)
+  float* d_muref32 = nullptr;   // [n_rec] the same, rounded
   double* d_muref64 = nullptr;  // [n_rec] R W_ref in FP64
   double* d_bref64 = nullptr;   // [n_rec] R W_ref + background (FP64)
   cudaEvent_t ev_fold[2] = {nullptr, nullptr};
@@ -297,7 +300,6 @@ cudaError_t launch_basis_eval(const srw_ctx* h, const float* theta, int mode, fl
 // likelihood.cu
 cudaError_t launch_set_data(srw_ctx* h, const double* d_bkg, int n_bkg, cudaStream_t s);
 cudaError_t launch_data_ref(srw_ctx* h, cudaStream_t s);
-cudaError_t launch_add_ref(const srw_ctx* h, float* out, int P, cudaStream_t s);
 int fold_point_grid(const srw_ctx* h);
 // Nonzero bands of R's rows and the band-balanced row split of the GEMV
 // (R: the device R copied to the host, n_rec x ld_r).
@@ -315,9 +317,9 @@ inline bool all_finite(const float* x, size_t n) {
 }
 
 cudaError_t gemv_prepare(srw_ctx* h, const std::vector<float>& R);
-cudaError_t simt_prepare(srw_ctx* h, const std::vector<float>& R);
+cudaError_t simt_prepare(srw_ctx* h, const std::vector<float>& R, cudaStream_t s);
 void fold_point_init();
-int fold_simt_parts(int n_rec);
+int fold_simt_parts(const srw_ctx* h, int P);  // partial sums per point of a P-point call
 cudaError_t launch_fold_point(const srw_ctx* h, const float* W, float* musig_out, float* mu_out, double* out,
                               cudaStream_t s, bool delta = false);
 // The single-point fold (delta mode) as a programmatic dependent of the
