@@ -1,0 +1,97 @@
+"""Sizes at the edges of the kernels' tiles, chunks and rounds, against the oracle.
+
+Every size here sits on one side or the other of a tile, a K tile, a round of
+reconstructed bins, a chunk of constants or a dispatch threshold."""
+
+import numpy as np
+import pytest
+
+import oracle as O
+import workloads
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def srw():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2607_00488_gb300 as pkg
+    return pkg
+
+
+def line_workload(n_t, n_rec, exposure=2.0e4):
+    """One 7Be line on [0, 1] MeV with a few empty-data bins at the top."""
+    t_edges, rec_edges = np.linspace(0.0, 1.0, n_t + 1), np.linspace(0.0, 1.3, n_rec + 1)
+    r = workloads.solar.response_matrix(t_edges, rec_edges, res=0.06, tail_frac=1e-3)
+    return {"name": "line", "t_edges": t_edges, "rec_edges": rec_edges, "sources": workloads.solar.be7_sources(), "R": r,
+            "bkg": np.full((1, n_rec), 0.1 * exposure / n_rec), "exposure": exposure, "t_min": 1e-3, "sin2w": 0.23121,
+            "f_tau": 0.5}
+
+
+def model_and_counts(wl, mask=None):
+    m = O.OracleModel.from_workload(wl)
+    m.set_data(np.zeros(wl["R"].shape[0]), wl["bkg"])
+    counts = workloads.poisson_counts(m.mu(np.zeros(5)), 3)
+    m.set_data(counts, wl["bkg"], mask)
+    return m, counts
+
+
+def oracle_matrix(m):
+    """The folded signal per coupling monomial, [8, n_rec] (FP64): many points without many spectra."""
+    basis = O.coefficient_spectra(m.sources, m.t_edges, m.t_min)
+    safe = np.where(m.s_sm != 0, m.s_sm, 1.0)
+    shat = np.where(m.s_sm != 0, basis * (m.e_sm / safe), 0.0)
+    shat[6] = np.where(m.s_sm != 0, shat[6], m.e_sm)
+    return shat @ m.r.T
+
+
+def values(m, M, theta):
+    from scipy.special import gammaln, xlogy
+    c = np.array([O.coupling_coefficients(t) for t in theta.astype(np.float64)])
+    mu = c @ M + m.bkg_sum
+    t = 2.0 * (mu - xlogy(m.counts, mu) + gammaln(m.counts + 1.0))
+    return (t * (1.0 if m.mask is None else (m.mask != 0))).sum(1), mu
+
+
+# FP32 products: |d(-2 ln L)| <= 1e-4 in the fit region (the library's bar)
+@pytest.mark.parametrize("n_t,n_rec,p", [(1, 1, 2), (15, 63, 31), (16, 64, 33), (17, 65, 64), (65, 127, 65), (64, 129, 2),
+                                         (260, 385, 700), (100, 2050, 640)])
+def test_fp32_batch_tiles(srw, n_t, n_rec, p):
+    wl = line_workload(n_t, n_rec)
+    mask = (np.arange(n_rec) % 7 != 3).astype(np.uint8) if n_rec > 1 else None
+    m, counts = model_and_counts(wl, mask)
+    theta = workloads.fit_region_points(p, seed=n_rec)
+    want, mu = values(m, oracle_matrix(m), theta)
+    with srw.Likelihood(wl, counts, mask=mask) as lk:
+        got = lk.loglik(theta, srw.SRW_FP32)
+        spec = lk.spectrum_batch(theta, srw.SRW_FP32)
+    np.testing.assert_allclose(got, want, rtol=0, atol=1e-4)
+    np.testing.assert_allclose(spec, mu - m.bkg_sum, rtol=1e-6, atol=1e-6 * mu.max())
+
+
+# rank 8: every path adds the same terms in the same order, so a point's value,
+# gradient and profiled value do not depend on the size of the batch that holds
+# it, which decides the path.  (The oracle's values: test_gpu_parity.py.)
+@pytest.mark.parametrize("n_rec,p", [(1, 16), (63, 17), (64, 2432), (65, 2433), (129, 4865), (1025, 33), (2049, 40),
+                                     (70, 9728), (70, 19455), (257, 19456)])
+def test_rank8_and_profiled_rounds(srw, n_rec, p):
+    wl = line_workload(50, n_rec)
+    mask = (np.arange(n_rec) % 5 != 2).astype(np.uint8) if n_rec > 1 else None
+    _, counts = model_and_counts(wl, mask)
+    theta = workloads.fit_region_points(p, seed=p)
+    with srw.Likelihood(wl, counts, mask=mask) as lk:
+        v, g = lk.loglik_linear(theta, grad=True)
+        only = lk.loglik_linear(theta)
+        prof, alpha = lk.loglik_profiled(theta[:5000], 0.05)
+        assert np.all(np.isfinite(v)) and np.all(np.isfinite(g)) and np.all(np.isfinite(prof))
+        np.testing.assert_array_equal(only, v)
+        for k in (0, p // 2, p - 1):
+            v1, g1 = lk.loglik_linear(theta[k:k + 1], grad=True)
+            assert v1[0] == v[k] and np.array_equal(g1[0], g[k])
+            if k < len(prof):
+                p1, a1 = lk.loglik_profiled(theta[k:k + 1], 0.05)
+                assert p1[0] == prof[k] and a1[0] == alpha[k]
