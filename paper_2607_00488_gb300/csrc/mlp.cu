@@ -10,20 +10,26 @@
 // standardized targets, Adam with FP32 master weights and BF16 copies of W and
 // W^T for the tensor cores.
 //
-// Every matrix product is one persistent tcgen05 GEMM, C = A B^T with A
-// [M][K] and B [N][K] BF16, both K-major (128-byte swizzle, TMA-fed), FP32
-// accumulation in TMEM (double-buffered), and an epilogue fused per use:
-//   forward, hidden layer : z = C + b; h = gelu(z) -> H, H^T (BF16), gelu'(z) (FP32)
-//   forward, output (fit) : y = C + b; e = y - t -> dY = 2e/count, dY^T (BF16); sum e^2
-//   backward, data        : dZ = C * gelu'(z) -> dZ, dZ^T (BF16)
-//   backward, weights     : dW = C (FP32)          (C = dZ^T H over the batch)
-//   forward, output (scan): mu = exp(m + s (C + b)) -> Poisson deviance summed per point
-// Activations are stored both row-major (operand A of the next layer's
-// product) and transposed (operand of the weight-gradient product), so every
-// product reads K-major operands.  Roles of a CTA: warp 0 TMA producer, warp 1
-// MMA issuer / TMEM owner, warps 2-9 epilogue: two per TMEM lane quarter
-// (warp w reads lanes 32 (w % 4) ...), each on half the columns.  Every wait
-// is bounded; a timeout raises kStatusTimeout.
+// Every matrix product is one persistent tcgen05 GEMM (BF16, 128-byte swizzle,
+// TMA-fed, FP32 accumulation in double-buffered TMEM) with an epilogue fused
+// per use:
+//   forward, hidden layer : z = A W^T + b; h = gelu(z) -> H (BF16), gelu'(z) (FP32)
+//   forward, output (fit) : y = A W^T + b; e = y - t -> dY = 2e/count (BF16); sum e^2
+//   backward, data        : dZ = (dZ' W) * gelu'(z) -> dZ (BF16)
+//   backward, weights     : dW = dZ^T H over the batch (FP32)
+//   forward, output (scan): mu = exp(m + s (A W^T + b)) -> Poisson deviance summed per point
+// Activations, their gradients and the weights are stored once, row-major.
+// The forward products read both operands K-major; the backward products
+// contract over the rows of a matrix and read it MN-major (the tensor core
+// takes either): no transposed copies are written.  Roles of a CTA: warp 0 TMA
+// producer, warp 1 MMA issuer / TMEM owner, warps 2-9 epilogue: two per TMEM
+// lane quarter (warp w reads lanes 32 (w % 4) ...), each on half the columns.
+// Every wait is bounded; a timeout raises kStatusTimeout.
+//
+// Tile width: a training step's products are small (4096 x 256: 32 tiles of
+// 256 columns on 152 SMs; dW: two), so the tile narrows to 64 columns until
+// the tiles fill the SMs (pick_tile).  Each element accumulates the same
+// products in the same order whatever the width.
 
 #include <algorithm>
 #include <cmath>
@@ -62,13 +68,22 @@ struct EpiArgs {
   int cols_valid;        // output columns >= cols_valid are padding
   const float* bias;     // [N]
   __nv_bfloat16* out_bf; // row-major BF16 [M][N]
-  __nv_bfloat16* out_t;  // transposed BF16 [N][M]
-  float* out_f32;        // FP32 [M][N]: gelu'(z), dW, or y
-  const float* aux;      // fit: targets [M][N]; backward data: gelu'(z) [M][N]
-  float scale;           // fit: 2 / (rows_valid * cols_valid)
+  float* out_f32;        // FP32 [M][ld]: gelu'(z), dW, or y
+  int ld;                // its row stride
+  const float* aux;      // backward data: gelu'(z) [M][N]
+  const struct StepParams* step;  // fit: the step's targets, rows and error scale
   double* loss;          // fit: += sum of squared errors
   const float4* binc;    // scan: per bin {m_j + s_j b_j, s_j, n_j, n_j ln n_j - n_j} (masked: {0, 0, 0, -1})
   double* parts;         // scan: per (column half-tile, row) partial sums of the deviance
+};
+
+// What one training step differs in from the next (device memory, written by
+// the step's first kernel).
+struct StepParams {
+  const float* targets;  // [M][n_out_pad]
+  int rows;              // points of the batch; the rows above are padding
+  float scale;           // 2 / (rows * n_out)
+  float lr, c1, c2;      // Adam: learning rate, 1 - beta1^t, 1 - beta2^t
 };
 
 template <int BN>
@@ -76,7 +91,7 @@ struct GemmShape {
   static constexpr int kAB = kBM * kBK * 2;
   static constexpr int kBB = BN * kBK * 2;
   static constexpr int kStageBytes = kAB + kBB;
-  static constexpr int kStages = (200 * 1024 / kStageBytes) < 6 ? (200 * 1024 / kStageBytes) : 6;
+  static constexpr int kStages = (200 * 1024 / kStageBytes) < 8 ? (200 * 1024 / kStageBytes) : 8;
   static constexpr int kSmem = kStages * kStageBytes + 1024;
   static constexpr int kTmemCols = 2 * BN;
 };
@@ -107,6 +122,8 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 int K, const EpiArgs E, unsigned* status) {
   using S = GemmShape<BN>;
   constexpr int ST = S::kStages;
+  constexpr bool kAMn = MODE == kWgrad, kBMn = MODE == kWgrad || MODE == kBwdData;
+  constexpr uint32_t kMnChunk = 64 * kBK * 2;  // bytes of a 64 x 64 box
   extern __shared__ unsigned char dsmem_raw[];
   // 1024-byte aligned base for the swizzled tiles, formed by pointer arithmetic on
   // the shared array so that plain loads through it stay shared-memory loads
@@ -162,8 +179,18 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             break;
           }
           ptx::mbar_arrive_expect_tx(&full[st], (uint32_t)S::kStageBytes);
-          tma_load_2d(a_s(st), &map_a, kb * kBK, m0, &full[st]);
-          tma_load_2d(b_s(st), &map_b, kb * kBK, n0, &full[st]);
+          if (kAMn) {  // boxes of 64 along M x 64 along K
+            for (int c = 0; c < kBM / 64; ++c)
+              tma_load_2d(a_s(st) + c * kMnChunk, &map_a, m0 + 64 * c, kb * kBK, &full[st]);
+          } else {
+            tma_load_2d(a_s(st), &map_a, kb * kBK, m0, &full[st]);
+          }
+          if (kBMn) {
+            for (int c = 0; c < BN / 64; ++c)
+              tma_load_2d(b_s(st) + c * kMnChunk, &map_b, n0 + 64 * c, kb * kBK, &full[st]);
+          } else {
+            tma_load_2d(b_s(st), &map_b, kb * kBK, n0, &full[st]);
+          }
           issued = g + 1;
         }
       }
@@ -172,7 +199,7 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
   } else if (warp == kMmaWarp) {
     if (lane == 0) {
-      constexpr uint32_t idesc = idesc_f16kind(kBM, BN, false);
+      constexpr uint32_t idesc = idesc_f16kind(kBM, BN, false, kAMn, kBMn);
       int g = 0, tc = -1;
       bool issued_any = false;
       for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
@@ -197,7 +224,10 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           const uint32_t as = ptx::smem_addr(a_s(st)), bs = ptx::smem_addr(b_s(st));
 #pragma unroll
           for (int ks = 0; ks < kBK / 16; ++ks)
-            mma_bf16(d_tmem, smem_desc_sw128(as + ks * 32u), smem_desc_sw128(bs + ks * 32u), idesc, (kb | ks) != 0);
+            // 16 of K: 32 bytes along a K-major row, 16 rows of 128 bytes of an MN-major tile
+            mma_bf16(d_tmem, kAMn ? smem_desc_mn(as + ks * 2048u, kMnChunk) : smem_desc_sw128(as + ks * 32u),
+                     kBMn ? smem_desc_mn(bs + ks * 2048u, kMnChunk) : smem_desc_sw128(bs + ks * 32u), idesc,
+                     (kb | ks) != 0);
           issued_any = true;
           mma_commit(&empty[st]);
         }
@@ -225,7 +255,7 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       }
       tc_fence_after();
       const int m = m0 + q * 32 + lane;
-      const bool row_on = m < E.rows_valid;
+      const bool row_on = m < (MODE == kFwdOutFit ? E.step->rows : E.rows_valid);
       const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
       float sse = 0.f;
       dfloat dev = {0.f, 0.f};
@@ -244,22 +274,25 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             if (MODE == kFwdHidden) gz[k] = gelu_grad_f(z);
           }
           store_bf16x16(E.out_bf + (size_t)m * N + n, v);
-          if (MODE == kFwdHidden) {
-            store_f32x16(E.out_f32 + (size_t)m * N + n, gz);
-#pragma unroll
-            for (int k = 0; k < 16; ++k) E.out_t[(size_t)(n + k) * M + m] = __float2bfloat16_rn(v[k]);
-          }
+          if (MODE == kFwdHidden) store_f32x16(E.out_f32 + (size_t)m * N + n, gz);
         } else if (MODE == kFwdOutFit) {
+          // the targets' rows are padded like the tile: a thread's 64 bytes in four loads
+          const float4* tp = reinterpret_cast<const float4*>(E.step->targets + (size_t)m * N + n);
+          const float scale = E.step->scale;
 #pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const float y = v[k] + __ldg(E.bias + n + k);
-            const float e = (row_on && n + k < E.cols_valid) ? y - E.aux[(size_t)m * N + n + k] : 0.f;
-            sse = fmaf(e, e, sse);
-            v[k] = e * E.scale;
+          for (int k4 = 0; k4 < 4; ++k4) {
+            const float4 t4 = row_on ? __ldg(tp + k4) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float tg[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int k = 4 * k4 + i;
+              const float y = v[k] + __ldg(E.bias + n + k);
+              const float e = (row_on && n + k < E.cols_valid) ? y - tg[i] : 0.f;
+              sse = fmaf(e, e, sse);
+              v[k] = e * scale;
+            }
           }
           store_bf16x16(E.out_bf + (size_t)m * N + n, v);
-#pragma unroll
-          for (int k = 0; k < 16; ++k) E.out_t[(size_t)(n + k) * M + m] = __float2bfloat16_rn(v[k]);
         } else if (MODE == kBwdData) {
           const float4* gp = reinterpret_cast<const float4*>(E.aux + (size_t)m * N + n);
 #pragma unroll
@@ -271,10 +304,8 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             v[4 * k4 + 3] *= gz.w;
           }
           store_bf16x16(E.out_bf + (size_t)m * N + n, v);
-#pragma unroll
-          for (int k = 0; k < 16; ++k) E.out_t[(size_t)(n + k) * M + m] = __float2bfloat16_rn(v[k]);
         } else if (MODE == kWgrad) {
-          store_f32x16(E.out_f32 + (size_t)m * N + n, v);
+          store_f32x16(E.out_f32 + (size_t)m * E.ld + n, v);
         } else if (MODE == kFwdOut) {
 #pragma unroll
           for (int k = 0; k < 16; ++k) v[k] += __ldg(E.bias + n + k);
@@ -312,12 +343,14 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   if (warp == kMmaWarp) tmem_dealloc(tmem_base, S::kTmemCols);
 }
 
-// theta [rows][5] -> X0 [M][128] and X0^T [128][M] (BF16), normalised to the
-// box.  Only columns 0-7 of X0 and rows 0-4 of X0^T are written: the padding
-// is zeroed once when the buffers are made.
+// theta [rows][5] -> X0 [M][128] (BF16), normalised to the box; only columns
+// 0-7 are written: the padding is zeroed once when the buffer is made.  In
+// training the kernel also publishes the step's parameters.
 __global__ void mlp_input_kernel(const float* __restrict__ theta, int rows, int M, float4 c0, float c4, float4 h0,
-                                 float h4, __nv_bfloat16* __restrict__ x, __nv_bfloat16* __restrict__ xt) {
+                                 float h4, __nv_bfloat16* __restrict__ x, const StepParams step,
+                                 StepParams* __restrict__ step_out) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m == 0 && step_out != nullptr) *step_out = step;
   if (m >= M) return;
   float u[kIn] = {0.f, 0.f, 0.f, 0.f, 0.f};
   if (m < rows) {
@@ -330,9 +363,6 @@ __global__ void mlp_input_kernel(const float* __restrict__ theta, int rows, int 
   }
   *reinterpret_cast<uint4*>(x + (size_t)m * kInPad) =
       make_uint4(pack_bf16x2(u[0], u[1]), pack_bf16x2(u[2], u[3]), pack_bf16x2(u[4], 0.f), 0u);
-  if (xt)
-#pragma unroll
-    for (int k = 0; k < kIn; ++k) xt[(size_t)k * M + m] = __float2bfloat16_rn(u[k]);
 }
 
 // Per-bin constants of the scan epilogue (from the standardization, the output
@@ -351,66 +381,99 @@ __global__ void scan_consts_kernel(const float* __restrict__ mean, const float* 
   out[j] = c;
 }
 
-// db[r] = sum_m dZ^T[r][m]: one warp per row.
-__global__ void rowsum_kernel(const __nv_bfloat16* __restrict__ a, int rows, int cols, float* __restrict__ out) {
-  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (r >= rows) return;
-  const int lane = threadIdx.x & 31;
-  float s = 0.f;
-  for (int c = lane; c < cols; c += 32) s += __bfloat162float(a[(size_t)r * cols + c]);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) out[r] = s;
+// db[c] = sum_m dZ[m][c]: a block of 64 threads takes 16 columns; thread l of
+// each half sums rows l, l + 32, ... of its eight, and the 32 partial sums are
+// added as a binary tree (16, 8, 4, 2, 1).
+constexpr int kColsumCols = 16;
+template <int K>
+__device__ __forceinline__ void add_rows(const uint4* src, size_t step, float* acc) {
+  uint4 v[K];
+#pragma unroll
+  for (int i = 0; i < K; ++i)
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[i].x), "=r"(v[i].y), "=r"(v[i].z), "=r"(v[i].w)
+                 : "l"(src + i * step));
+#pragma unroll
+  for (int i = 0; i < K; ++i) {
+    const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      acc[2 * k] += __uint_as_float(w[k] << 16);
+      acc[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u);
+    }
+  }
+}
+__global__ void __launch_bounds__(64, 1)
+colsum_kernel(const __nv_bfloat16* __restrict__ a, int rows, int cols, float* __restrict__ out) {
+  __shared__ float s[32][kColsumCols + 1];
+  const int l = threadIdx.x >> 1, c8 = (threadIdx.x & 1) * 8;
+  const uint4* src = reinterpret_cast<const uint4*>(a + (size_t)l * cols + blockIdx.x * kColsumCols + c8);
+  const size_t step = (size_t)32 * cols / 8;
+  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  // the sums are a chain, their loads are not: sixteen (then four) rows in
+  // flight (the launch bound leaves the registers for them; without it the
+  // compiler kept to 32 and to one row's latency at a time, 27 us for 4096 rows)
+  int i = 0;
+  const int n = rows / 32;  // rows is a multiple of 128
+  for (; i + 16 <= n; i += 16) add_rows<16>(src + i * step, step, acc);
+  for (; i < n; i += 4) add_rows<4>(src + i * step, step, acc);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) s[l][c8 + k] = acc[k];
+  for (int o = 16; o > 0; o >>= 1) {
+    __syncthreads();
+    for (int q = threadIdx.x; q < o * kColsumCols; q += 64) {
+      const int r = q / kColsumCols, c = q % kColsumCols;
+      s[r][c] += s[r + o][c];
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < kColsumCols) out[blockIdx.x * kColsumCols + threadIdx.x] = s[0][threadIdx.x];
 }
 
-// One flat parameter block of a layer for the Adam update.
-struct AdamLayer {
-  float* w;              // master FP32 [out][in] (weights) or [out] (biases)
+// One layer's weights or biases for the Adam update (n a multiple of 4).
+struct AdamBlock {
+  float* w;              // master FP32
   const float* g;
   float* m;
   float* v;
-  __nv_bfloat16* w_bf;   // BF16 copy [out][in] (nullptr for biases)
-  __nv_bfloat16* wt_bf;  // BF16 transposed copy [in][out]
-  int out, in;           // in = 1 for biases
-  long long first;       // offset of this block in the flat index space
-};
-struct AdamArgs {
-  AdamLayer L[8];
-  int n_layers;
-  long long total;
-  float lr, beta1, beta2, eps, c1, c2;  // c1 = 1 - beta1^t, c2 = 1 - beta2^t
+  __nv_bfloat16* w_bf;   // BF16 copy (nullptr for biases)
+  int n;
 };
 
-__global__ void adam_kernel(const AdamArgs A) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= A.total) return;
-  int l = 0;
-  while (l + 1 < A.n_layers && i >= A.L[l + 1].first) ++l;
-  const AdamLayer& L = A.L[l];
-  const long long k = i - L.first;
-  const float g = L.g[k];
-  const float m = A.beta1 * L.m[k] + (1.f - A.beta1) * g;
-  const float v = A.beta2 * L.v[k] + (1.f - A.beta2) * g * g;
-  L.m[k] = m;
-  L.v[k] = v;
-  const float w = L.w[k] - A.lr * (m / A.c1) / (sqrtf(v / A.c2) + A.eps);
-  L.w[k] = w;
-  if (L.w_bf) {
-    const __nv_bfloat16 b = __float2bfloat16_rn(w);
-    L.w_bf[k] = b;
-    const int o = (int)(k / L.in), c = (int)(k % L.in);
-    L.wt_bf[(size_t)c * L.out + o] = b;
-  }
+__device__ __forceinline__ float adam_one(float w, float g, float& m, float& v, float beta1, float beta2, float eps,
+                                          const StepParams& p) {
+  // one fused and one rounded product each, whatever the compiler would contract
+  m = __fmaf_rn(1.f - beta1, g, __fmul_rn(beta1, m));
+  v = __fmaf_rn(beta2, v, __fmul_rn(__fmul_rn(1.f - beta2, g), g));
+  return w - p.lr * (m / p.c1) / (sqrtf(v / p.c2) + eps);
 }
 
-// FP32 master -> BF16 copies (after the weights are set from the host).
-__global__ void cast_weights_kernel(const float* __restrict__ w, int out, int in, __nv_bfloat16* __restrict__ w_bf,
-                                    __nv_bfloat16* __restrict__ wt_bf) {
-  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= (long long)out * in) return;
-  const __nv_bfloat16 b = __float2bfloat16_rn(w[k]);
-  w_bf[k] = b;
-  const int o = (int)(k / in), c = (int)(k % in);
-  wt_bf[(size_t)c * out + o] = b;
+// One layer: four elements a thread, the weights' blocks first.
+__global__ void adam_kernel(const AdamBlock W, const AdamBlock B, float beta1, float beta2, float eps,
+                            const StepParams* __restrict__ step) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, nw = W.n / 4;
+  const bool bias = i >= nw;
+  const AdamBlock& L = bias ? B : W;
+  const int k = bias ? i - nw : i;
+  if (k >= L.n / 4) return;
+  const StepParams p = *step;
+  float4 w = reinterpret_cast<float4*>(L.w)[k], m = reinterpret_cast<float4*>(L.m)[k],
+         v = reinterpret_cast<float4*>(L.v)[k];
+  const float4 g = reinterpret_cast<const float4*>(L.g)[k];
+  w.x = adam_one(w.x, g.x, m.x, v.x, beta1, beta2, eps, p);
+  w.y = adam_one(w.y, g.y, m.y, v.y, beta1, beta2, eps, p);
+  w.z = adam_one(w.z, g.z, m.z, v.z, beta1, beta2, eps, p);
+  w.w = adam_one(w.w, g.w, m.w, v.w, beta1, beta2, eps, p);
+  reinterpret_cast<float4*>(L.w)[k] = w;
+  reinterpret_cast<float4*>(L.m)[k] = m;
+  reinterpret_cast<float4*>(L.v)[k] = v;
+  if (!bias) reinterpret_cast<uint2*>(L.w_bf)[k] = make_uint2(pack_bf16x2(w.x, w.y), pack_bf16x2(w.z, w.w));
+}
+
+// FP32 master -> BF16 copy (after the weights are set from the host).
+__global__ void cast_weights_kernel(const float* __restrict__ w, int n, __nv_bfloat16* __restrict__ w_bf) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n) w_bf[k] = __float2bfloat16_rn(w[k]);
 }
 
 // Training targets: dst [rows][ld] = log(mu_sig + b) from src [rows][n]
@@ -657,33 +720,49 @@ cudaError_t launch_mode(const Gemm& g, int sm_count, unsigned* status, cudaStrea
   return srw::launch_result();
 }
 
-cudaError_t run_gemm(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s) {
-  if (g.bn == 256) {
-    switch (g.mode) {
-      case kFwdHidden: return launch_mode<256, kFwdHidden>(g, sm_count, status, s);
-      case kFwdOutFit: return launch_mode<256, kFwdOutFit>(g, sm_count, status, s);
-      case kBwdData: return launch_mode<256, kBwdData>(g, sm_count, status, s);
-      case kWgrad: return launch_mode<256, kWgrad>(g, sm_count, status, s);
-      case kFwdOut: return launch_mode<256, kFwdOut>(g, sm_count, status, s);
-      case kFwdScan: return launch_mode<256, kFwdScan>(g, sm_count, status, s);
-      case kFwdHiddenScan: return launch_mode<256, kFwdHiddenScan>(g, sm_count, status, s);
-    }
-  } else {
-    if (g.mode == kWgrad) return launch_mode<128, kWgrad>(g, sm_count, status, s);
+template <int BN>
+cudaError_t launch_width(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s) {
+  switch (g.mode) {
+    case kFwdHidden: return launch_mode<BN, kFwdHidden>(g, sm_count, status, s);
+    case kFwdOutFit: return launch_mode<BN, kFwdOutFit>(g, sm_count, status, s);
+    case kBwdData: return launch_mode<BN, kBwdData>(g, sm_count, status, s);
+    case kFwdOut: return launch_mode<BN, kFwdOut>(g, sm_count, status, s);
+    case kFwdScan: return launch_mode<BN, kFwdScan>(g, sm_count, status, s);
+    case kFwdHiddenScan: return launch_mode<BN, kFwdHiddenScan>(g, sm_count, status, s);
   }
   return cudaErrorInvalidValue;
 }
 
-cudaError_t gemm_attrs() {
-  cudaError_t e = gemm_attr<256, kFwdHidden>();
-  if (e == cudaSuccess) e = gemm_attr<256, kFwdOutFit>();
-  if (e == cudaSuccess) e = gemm_attr<256, kBwdData>();
-  if (e == cudaSuccess) e = gemm_attr<256, kWgrad>();
-  if (e == cudaSuccess) e = gemm_attr<256, kFwdOut>();
-  if (e == cudaSuccess) e = gemm_attr<256, kFwdScan>();
-  if (e == cudaSuccess) e = gemm_attr<256, kFwdHiddenScan>();
-  if (e == cudaSuccess) e = gemm_attr<128, kWgrad>();
+cudaError_t run_gemm(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s) {
+  if (g.mode == kWgrad) return launch_mode<64, kWgrad>(g, sm_count, status, s);
+  return g.bn == 256 ? launch_width<256>(g, sm_count, status, s)
+                     : g.bn == 128 ? launch_width<128>(g, sm_count, status, s) : launch_width<64>(g, sm_count, status, s);
+}
+
+template <int BN>
+cudaError_t gemm_attrs_width() {
+  cudaError_t e = gemm_attr<BN, kFwdHidden>();
+  if (e == cudaSuccess) e = gemm_attr<BN, kFwdOutFit>();
+  if (e == cudaSuccess) e = gemm_attr<BN, kBwdData>();
+  if (e == cudaSuccess) e = gemm_attr<BN, kFwdOut>();
+  if (e == cudaSuccess) e = gemm_attr<BN, kFwdScan>();
+  if (e == cudaSuccess) e = gemm_attr<BN, kFwdHiddenScan>();
   return e;
+}
+
+cudaError_t gemm_attrs() {
+  cudaError_t e = gemm_attrs_width<256>();
+  if (e == cudaSuccess) e = gemm_attrs_width<128>();
+  if (e == cudaSuccess) e = gemm_attrs_width<64>();
+  if (e == cudaSuccess) e = gemm_attr<64, kWgrad>();
+  return e;
+}
+
+// Widest tile that gives every SM two tiles, else 64 columns (see the header).
+int pick_tile(int M, int N, int sm_count) {
+  for (int bn = 256; bn > 64; bn /= 2)
+    if ((long long)(M / kBM) * (N / bn) >= 2LL * sm_count) return bn;
+  return 64;
 }
 
 }  // namespace
@@ -699,22 +778,22 @@ struct SurrogateLayer {
   float* mw = nullptr, *vw = nullptr, *mb = nullptr, *vb = nullptr;
   float* gw = nullptr, *gb = nullptr;  // gradients
   __nv_bfloat16* w_bf = nullptr;       // [out][in]
-  __nv_bfloat16* wt_bf = nullptr;      // [in][out]
 };
 
-// Activations of one batch size (training buffers include transposes).
+// Activations of one batch size.
 struct SurrogateBatch {
   int M = 0;
   bool train = false;
-  __nv_bfloat16 *x = nullptr, *xt = nullptr;
-  __nv_bfloat16 *h[3] = {}, *ht[3] = {};
+  __nv_bfloat16* x = nullptr;
+  __nv_bfloat16* h[3] = {};
   float* gz[3] = {};
-  __nv_bfloat16 *dy = nullptr, *dyt = nullptr;
-  __nv_bfloat16 *dz[3] = {}, *dzt[3] = {};
+  __nv_bfloat16* dy = nullptr;
+  __nv_bfloat16* dz[3] = {};
   float* y = nullptr;       // FP32 network output (forward hook)
-  double* parts = nullptr;  // scan partials [n_out_pad / 256][M]
+  double* parts = nullptr;  // scan partials [2 n_out_pad / tile width][M]
   double* loss = nullptr;
   Gemm fwd[4], fwd_out, fwd_scan, wgrad[4], bwd[3];
+  cudaGraphExec_t step = nullptr;  // captured training step (after its input kernel)
 };
 
 struct srw_surrogate_ctx {
@@ -733,6 +812,11 @@ struct srw_surrogate_ctx {
   cudaStream_t stream = nullptr;
   std::vector<SurrogateBatch*> batches;
   uint32_t* d_sobol = nullptr;  // direction numbers [5][32]
+  srw::StepParams* d_step = nullptr;  // the training step in flight
+  // branches of a captured training step: a layer's weight gradient and update
+  // (0-3), the bias gradients (4); events: forks and joins of the branches
+  cudaStream_t side[5] = {};
+  cudaEvent_t fork[10] = {};
   std::string err;
 };
 
@@ -804,10 +888,11 @@ struct CallEvents {
 int round_up(long long x, int m) { return (int)((x + m - 1) / m * m); }
 
 void free_batch(SurrogateBatch* B) {
-  sfree(B->x); sfree(B->xt); sfree(B->dy); sfree(B->dyt); sfree(B->y); sfree(B->parts); sfree(B->loss);
+  sfree(B->x); sfree(B->dy); sfree(B->y); sfree(B->parts); sfree(B->loss);
   for (int k = 0; k < 3; ++k) {
-    sfree(B->h[k]); sfree(B->ht[k]); sfree(B->gz[k]); sfree(B->dz[k]); sfree(B->dzt[k]);
+    sfree(B->h[k]); sfree(B->gz[k]); sfree(B->dz[k]);
   }
+  if (B->step) cudaGraphExecDestroy(B->step);
   delete B;
 }
 
@@ -839,16 +924,20 @@ srw::EpiArgs epi0(int M, int N, int rows_valid, int cols_valid) {
   return E;
 }
 
+// C[M][N] over K: forward modes read A [M][K] and B [N][K]; kBwdData reads A
+// [M][K] and B [K][N]; kWgrad A [K][M] and B [K][ldb].
 cudaError_t prep(Gemm& g, const __nv_bfloat16* A, const __nv_bfloat16* B, int M, int N, int K, int mode, int bn,
-                 const srw::EpiArgs& E) {
+                 const srw::EpiArgs& E, int lda = 0, int ldb = 0) {
   g.M = M;
   g.N = N;
   g.K = K;
   g.mode = mode;
   g.bn = bn;
   g.E = E;
-  cudaError_t e = srw::make_map(&g.ma, A, M, K, srw::kBM);
-  if (e == cudaSuccess) e = srw::make_map(&g.mb, B, N, K, bn);
+  const bool a_mn = mode == srw::kWgrad, b_mn = a_mn || mode == srw::kBwdData;
+  cudaError_t e = a_mn ? srw::make_map(&g.ma, A, K, M, srw::kBK) : srw::make_map(&g.ma, A, M, lda ? lda : K, srw::kBM);
+  if (e == cudaSuccess)
+    e = b_mn ? srw::make_map(&g.mb, B, K, ldb ? ldb : N, srw::kBK) : srw::make_map(&g.mb, B, N, ldb ? ldb : K, bn);
   return e;
 }
 
@@ -866,18 +955,14 @@ srw_status get_batch(srw_surrogate s, int M, bool train, SurrogateBatch** out) {
   const int H = srw::kHidden, NO = s->n_out_pad;
   cudaError_t e = salloc(&B->x, (size_t)M * srw::kInPad);
   for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = salloc(&B->h[k], (size_t)M * H);
-  if (e == cudaSuccess) e = salloc(&B->parts, (size_t)(NO / 256) * 2 * M);
+  const int bn_h = srw::pick_tile(M, H, s->sm_count), bn_o = srw::pick_tile(M, NO, s->sm_count);
+  if (e == cudaSuccess) e = salloc(&B->parts, (size_t)(NO / bn_o) * 2 * M);
   if (e == cudaSuccess) e = cudaMemset(B->x, 0, sizeof(__nv_bfloat16) * (size_t)M * srw::kInPad);
   if (e == cudaSuccess) e = salloc(&B->loss, 1);
   if (train) {
-    if (e == cudaSuccess) e = salloc(&B->xt, (size_t)M * srw::kInPad);
-    if (e == cudaSuccess) e = cudaMemset(B->xt, 0, sizeof(__nv_bfloat16) * (size_t)M * srw::kInPad);
-    for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = salloc(&B->ht[k], (size_t)M * H);
     for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = salloc(&B->gz[k], (size_t)M * H);
     for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = salloc(&B->dz[k], (size_t)M * H);
-    for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = salloc(&B->dzt[k], (size_t)M * H);
     if (e == cudaSuccess) e = salloc(&B->dy, (size_t)M * NO);
-    if (e == cudaSuccess) e = salloc(&B->dyt, (size_t)M * NO);
   }
   if (e != cudaSuccess) {
     free_batch(B);
@@ -889,53 +974,52 @@ srw_status get_batch(srw_surrogate s, int M, bool train, SurrogateBatch** out) {
     srw::EpiArgs E = epi0(M, H, M, H);
     E.bias = s->L[l].b;
     E.out_bf = B->h[l];
-    if (train) {
-      E.out_t = B->ht[l];
-      E.out_f32 = B->gz[l];
-    }
-    e = prep(B->fwd[l], act_in[l], s->L[l].w_bf, M, H, s->L[l].in, train ? srw::kFwdHidden : srw::kFwdHiddenScan, 256, E);
+    if (train) E.out_f32 = B->gz[l];
+    // the first layer contracts over one K block: the padded inputs above it are zero
+    e = prep(B->fwd[l], act_in[l], s->L[l].w_bf, M, H, l == 0 ? srw::kBK : s->L[l].in,
+             train ? srw::kFwdHidden : srw::kFwdHiddenScan, bn_h, E, s->L[l].in, s->L[l].in);
   }
   // forward, output: plain y (hook) and the scan's deviance
   if (e == cudaSuccess) {
     srw::EpiArgs E = epi0(M, NO, M, s->n_out);
     E.bias = s->L[3].b;
     E.out_f32 = B->y;
-    e = prep(B->fwd_out, B->h[2], s->L[3].w_bf, M, NO, H, srw::kFwdOut, 256, E);
+    e = prep(B->fwd_out, B->h[2], s->L[3].w_bf, M, NO, H, srw::kFwdOut, bn_o, E);
   }
   if (e == cudaSuccess) {
     srw::EpiArgs E = epi0(M, NO, M, s->n_out);
     E.bias = s->L[3].b;
     E.binc = s->binc;
     E.parts = B->parts;
-    e = prep(B->fwd_scan, B->h[2], s->L[3].w_bf, M, NO, H, srw::kFwdScan, 256, E);
+    e = prep(B->fwd_scan, B->h[2], s->L[3].w_bf, M, NO, H, srw::kFwdScan, bn_o, E);
   }
   if (train) {
     if (e == cudaSuccess) {  // fit output: targets set per call
       srw::EpiArgs E = epi0(M, NO, M, s->n_out);
       E.bias = s->L[3].b;
       E.out_bf = B->dy;
-      E.out_t = B->dyt;
       E.loss = B->loss;
-      e = prep(B->fwd[3], B->h[2], s->L[3].w_bf, M, NO, H, srw::kFwdOutFit, 256, E);
+      E.step = s->d_step;
+      e = prep(B->fwd[3], B->h[2], s->L[3].w_bf, M, NO, H, srw::kFwdOutFit, bn_o, E);
     }
     // weight gradients dW_l = dZ_l^T A_l over the batch (K = M)
-    const __nv_bfloat16* dzt[4] = {B->dzt[0], B->dzt[1], B->dzt[2], B->dyt};
-    const __nv_bfloat16* actt[4] = {B->xt, B->ht[0], B->ht[1], B->ht[2]};
+    // (the first layer's gradient beyond its first 64 inputs is zero from the start: those are padding)
+    const __nv_bfloat16* dz_of[4] = {B->dz[0], B->dz[1], B->dz[2], B->dy};
     for (int l = 0; l < 4 && e == cudaSuccess; ++l) {
-      const int out = s->L[l].out, in = s->L[l].in;
-      srw::EpiArgs E = epi0(out, in, out, in);
+      const int out = s->L[l].out, in = s->L[l].in, n = l == 0 ? 64 : in;
+      srw::EpiArgs E = epi0(out, n, out, n);
       E.out_f32 = s->L[l].gw;
-      e = prep(B->wgrad[l], dzt[l], actt[l], out, in, M, srw::kWgrad, in >= 256 ? 256 : 128, E);
+      E.ld = in;
+      e = prep(B->wgrad[l], dz_of[l], act_in[l], out, n, M, srw::kWgrad, 64, E, 0, in);
     }
-    // backward data: dZ_{l-1} = (dZ_l W_l) * gelu'(z_{l-1}), l = 3, 2, 1 (W_l^T is the K-major operand)
+    // backward data: dZ_{l-1} = (dZ_l W_l) * gelu'(z_{l-1}), l = 3, 2, 1
     const __nv_bfloat16* dz_in[3] = {B->dz[1], B->dz[2], B->dy};
     for (int l = 0; l < 3 && e == cudaSuccess; ++l) {  // produces dz[l] from layer l+1
       const int K = s->L[l + 1].out;
       srw::EpiArgs E = epi0(M, H, M, H);
       E.aux = B->gz[l];
       E.out_bf = B->dz[l];
-      E.out_t = B->dzt[l];
-      e = prep(B->bwd[l], dz_in[l], s->L[l + 1].wt_bf, M, H, K, srw::kBwdData, 256, E);
+      e = prep(B->bwd[l], dz_in[l], s->L[l + 1].w_bf, M, H, K, srw::kBwdData, bn_h, E);
     }
   }
   if (e != cudaSuccess) {
@@ -947,78 +1031,137 @@ srw_status get_batch(srw_surrogate s, int M, bool train, SurrogateBatch** out) {
   return SRW_OK;
 }
 
-cudaError_t launch_input(srw_surrogate s, const float* theta, int rows, SurrogateBatch* B, cudaStream_t st) {
+cudaError_t launch_input(srw_surrogate s, const float* theta, int rows, SurrogateBatch* B, cudaStream_t st,
+                         const srw::StepParams* step = nullptr) {
   const float4 c0 = make_float4(s->centre[0], s->centre[1], s->centre[2], s->centre[3]);
   const float4 h0 = make_float4(s->half[0], s->half[1], s->half[2], s->half[3]);
   srw::mlp_input_kernel<<<(B->M + 255) / 256, 256, 0, st>>>(theta, rows, B->M, c0, s->centre[4], h0, s->half[4], B->x,
-                                                            B->train ? B->xt : nullptr);
+                                                            step ? *step : srw::StepParams{}, step ? s->d_step : nullptr);
   return srw::launch_result();
 }
 
-// Forward through the hidden layers (rows of theta; B->M >= rows).
-cudaError_t forward_hidden(srw_surrogate s, const float* theta, int rows, SurrogateBatch* B, bool train, cudaStream_t st) {
+// Inference through the hidden layers (rows of theta; B->M >= rows).
+cudaError_t forward_hidden(srw_surrogate s, const float* theta, int rows, SurrogateBatch* B, cudaStream_t st) {
   cudaError_t e = launch_input(s, theta, rows, B, st);
   for (int l = 0; l < 3 && e == cudaSuccess; ++l) {
     Gemm g = B->fwd[l];
-    if (!train) {  // inference: activations only
-      g.mode = srw::kFwdHiddenScan;
-      g.E.out_t = nullptr;
-      g.E.out_f32 = nullptr;
-    }
-    g.E.rows_valid = rows;
+    g.mode = srw::kFwdHiddenScan;  // activations only
+    g.E.out_f32 = nullptr;
     e = srw::run_gemm(g, s->sm_count, s->d_status, st);
   }
   return e;
 }
 
-// One forward + backward pass over rows points with standardized targets
-// t [M][n_out_pad] (FP32, device); gradients land in L[l].gw / gb, the summed
-// squared error in B->loss.
-cudaError_t fit_pass(srw_surrogate s, const float* theta, const float* targets, int rows, SurrogateBatch* B,
-                     cudaStream_t st, bool reset_loss = true) {
-  cudaError_t e = reset_loss ? cudaMemsetAsync(B->loss, 0, sizeof(double), st) : cudaSuccess;
-  if (e == cudaSuccess) e = forward_hidden(s, theta, rows, B, true, st);
-  if (e != cudaSuccess) return e;
-  Gemm g = B->fwd[3];
-  g.E.aux = targets;
-  g.E.rows_valid = rows;
-  g.E.scale = 2.0f / ((float)rows * (float)s->n_out);
-  if ((e = srw::run_gemm(g, s->sm_count, s->d_status, st)) != cudaSuccess) return e;
-  // output layer gradients, then down the hidden layers
+// Parameters of a step on `rows` points; adam_t is the step's number (0: no update follows).
+srw::StepParams step_params(srw_surrogate s, const float* targets, int rows, float lr, long long adam_t) {
+  srw::StepParams p{};
+  p.targets = targets;
+  p.rows = rows;
+  p.scale = 2.0f / ((float)rows * (float)s->n_out);
+  p.lr = lr;
+  p.c1 = (float)(1.0 - std::pow((double)0.9f, (double)adam_t));
+  p.c2 = (float)(1.0 - std::pow((double)0.999f, (double)adam_t));
+  return p;
+}
+
+cudaError_t layer_wgrad(srw_surrogate s, SurrogateBatch* B, int l, cudaStream_t st) {
+  return srw::run_gemm(B->wgrad[l], s->sm_count, s->d_status, st);
+}
+cudaError_t layer_bias(srw_surrogate s, SurrogateBatch* B, int l, cudaStream_t st) {
+  SurrogateLayer& L = s->L[l];
+  srw::colsum_kernel<<<L.out / srw::kColsumCols, 64, 0, st>>>(l == 3 ? B->dy : B->dz[l], B->M, L.out, L.gb);
+  return srw::launch_result();
+}
+cudaError_t layer_adam(srw_surrogate s, int l, cudaStream_t st) {
+  SurrogateLayer& L = s->L[l];
+  const srw::AdamBlock w{L.w, L.gw, L.mw, L.vw, L.w_bf, L.out * L.in}, b{L.b, L.gb, L.mb, L.vb, nullptr, L.out};
+  srw::adam_kernel<<<((L.out * L.in + L.out) / 4 + 255) / 256, 256, 0, st>>>(w, b, 0.9f, 0.999f, 1e-8f, s->d_step);
+  return srw::launch_result();
+}
+
+// The step whose inputs and parameters launch_input has put in place: forward,
+// backward (gradients in L[l].gw / gb, the summed squared error in B->loss)
+// and, with `update`, Adam.
+cudaError_t step_body(srw_surrogate s, SurrogateBatch* B, cudaStream_t st, bool update) {
+  cudaError_t e = cudaSuccess;
+  for (int l = 0; l < 4 && e == cudaSuccess; ++l) e = srw::run_gemm(B->fwd[l], s->sm_count, s->d_status, st);
   for (int l = 3; l >= 0 && e == cudaSuccess; --l) {
-    e = srw::run_gemm(B->wgrad[l], s->sm_count, s->d_status, st);
-    const __nv_bfloat16* dzt = l == 3 ? B->dyt : B->dzt[l];
-    if (e == cudaSuccess) {
-      srw::rowsum_kernel<<<(s->L[l].out + 7) / 8, 256, 0, st>>>(dzt, s->L[l].out, B->M, s->L[l].gb);
-      e = srw::launch_result();
-    }
-    if (l > 0 && e == cudaSuccess) e = srw::run_gemm(B->bwd[l - 1], s->sm_count, s->d_status, st);
+    // before this layer's update: the gradient of the layer below uses its weights
+    if (l > 0) e = srw::run_gemm(B->bwd[l - 1], s->sm_count, s->d_status, st);
+    if (e == cudaSuccess) e = layer_wgrad(s, B, l, st);
+    if (e == cudaSuccess) e = layer_bias(s, B, l, st);
+    if (e == cudaSuccess && update) e = layer_adam(s, l, st);
   }
   return e;
 }
 
-cudaError_t adam_update(srw_surrogate s, float lr, float beta1, float beta2, float eps, cudaStream_t st) {
-  ++s->adam_t;
-  srw::AdamArgs A{};
-  long long off = 0;
-  int n = 0;
-  for (int l = 0; l < 4; ++l) {
-    SurrogateLayer& L = s->L[l];
-    A.L[n++] = srw::AdamLayer{L.w, L.gw, L.mw, L.vw, L.w_bf, L.wt_bf, L.out, L.in, off};
-    off += (long long)L.out * L.in;
-    A.L[n++] = srw::AdamLayer{L.b, L.gb, L.mb, L.vb, nullptr, nullptr, L.out, 1, off};
-    off += L.out;
+// The same step (with its update) in branches: each layer's weight gradient
+// and update beside the chain of the data gradients.  A weight gradient is a
+// long contraction in few CTAs (4096 points into 256 x 256: eight CTAs, 23 us),
+// which the other layers' kernels run beside.
+cudaError_t step_branches(srw_surrogate s, SurrogateBatch* B, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  auto ok = [&](cudaError_t r) {
+    if (e == cudaSuccess) e = r;
+  };
+  auto after = [&](cudaStream_t waiter, cudaStream_t of, int ev) {
+    ok(cudaEventRecord(s->fork[ev], of));
+    ok(cudaStreamWaitEvent(waiter, s->fork[ev], 0));
+  };
+  for (int l = 0; l < 4; ++l) ok(srw::run_gemm(B->fwd[l], s->sm_count, s->d_status, st));
+  for (int l = 3; l >= 0; --l) {
+    // dz of layer l is ready on st
+    ok(cudaEventRecord(s->fork[l], st));
+    ok(cudaStreamWaitEvent(s->side[l], s->fork[l], 0));
+    ok(cudaStreamWaitEvent(s->side[4], s->fork[l], 0));
+    ok(layer_wgrad(s, B, l, s->side[l]));
+    ok(layer_bias(s, B, l, s->side[4]));
+    after(s->side[l], s->side[4], 4);
+    if (l > 0) {
+      ok(srw::run_gemm(B->bwd[l - 1], s->sm_count, s->d_status, st));
+      after(s->side[l], st, 5);  // which has read this layer's weights
+    }
+    ok(layer_adam(s, l, s->side[l]));
+    after(st, s->side[l], 6 + l);
   }
-  A.n_layers = n;
-  A.total = off;
-  A.lr = lr;
-  A.beta1 = beta1;
-  A.beta2 = beta2;
-  A.eps = eps;
-  A.c1 = (float)(1.0 - std::pow((double)beta1, (double)s->adam_t));
-  A.c2 = (float)(1.0 - std::pow((double)beta2, (double)s->adam_t));
-  srw::adam_kernel<<<(unsigned)((off + 255) / 256), 256, 0, st>>>(A);
-  return srw::launch_result();
+  return e;
+}
+
+// Captures the branched step of batch B (its buffers, and so the graph, are fixed).
+cudaError_t capture_step(srw_surrogate s, SurrogateBatch* B, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  for (auto& x : s->side)
+    if (!x && e == cudaSuccess) e = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
+  for (auto& x : s->fork)
+    if (!x && e == cudaSuccess) e = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
+  if (e != cudaSuccess) return e;
+  if ((e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return e;
+  const cudaError_t eb = step_branches(s, B, st);
+  cudaGraph_t graph = nullptr;
+  const cudaError_t ee = cudaStreamEndCapture(st, &graph);
+  e = eb != cudaSuccess ? eb : ee;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&B->step, graph, 0);
+  if (graph) cudaGraphDestroy(graph);
+  return e;
+}
+
+// One pass over rows points with standardized targets t [M][n_out_pad] (FP32,
+// device); lr > 0: with Adam's update.
+cudaError_t fit_pass(srw_surrogate s, const float* theta, const float* targets, int rows, SurrogateBatch* B,
+                     cudaStream_t st, float lr = 0.f) {
+  const bool update = lr > 0.f;
+  const srw::StepParams p = step_params(s, targets, rows, lr, update ? ++s->adam_t : 0);
+  const cudaError_t e = launch_input(s, theta, rows, B, st, &p);
+  return e == cudaSuccess ? step_body(s, B, st, update) : e;
+}
+
+// A training step of a fit: the captured step behind its input kernel.
+cudaError_t fit_step(srw_surrogate s, const float* theta, const float* targets, int rows, SurrogateBatch* B,
+                     cudaStream_t st, float lr) {
+  cudaError_t e = B->step ? cudaSuccess : capture_step(s, B, st);
+  const srw::StepParams p = step_params(s, targets, rows, lr, ++s->adam_t);
+  if (e == cudaSuccess) e = launch_input(s, theta, rows, B, st, &p);
+  return e == cudaSuccess ? cudaGraphLaunch(B->step, st) : e;
 }
 
 constexpr int kScanChunk = 1 << 20;  // points per surrogate launch chain in scans
@@ -1033,14 +1176,15 @@ srw_status loglik_device(srw_surrogate s, const float* theta, long long P, T* ou
     SurrogateBatch* B = nullptr;
     srw_status r = get_batch(s, round_up(rows, srw::kBM) < 65536 ? round_up(rows, srw::kBM) : round_up(rows, 65536), false, &B);
     if (r != SRW_OK) return r;
-    cudaError_t e = forward_hidden(s, theta + off * 5, rows, B, false, st);
+    cudaError_t e = forward_hidden(s, theta + off * 5, rows, B, st);
     if (e == cudaSuccess) {
       Gemm g = B->fwd_scan;
       g.E.rows_valid = rows;
       e = srw::run_gemm(g, s->sm_count, s->d_status, st);
     }
+    const int g_bn = B->fwd_scan.bn;
     if (e == cudaSuccess) {
-      srw::scan_reduce_kernel<T><<<(rows + 255) / 256, 256, 0, st>>>(B->parts, s->n_out_pad / 256 * 2, rows, s->h->d_cdata,
+      srw::scan_reduce_kernel<T><<<(rows + 255) / 256, 256, 0, st>>>(B->parts, s->n_out_pad / g_bn * 2, rows, s->h->d_cdata,
                                                                    out + off);
       e = srw::launch_result();
     }
@@ -1084,7 +1228,8 @@ srw_status upload_weights(srw_surrogate s, const float* const* w) {
     S_CUDA(s, cudaMemset(L.vw, 0, sizeof(float) * W.size()), "adam state");
     S_CUDA(s, cudaMemset(L.mb, 0, sizeof(float) * L.out), "adam state");
     S_CUDA(s, cudaMemset(L.vb, 0, sizeof(float) * L.out), "adam state");
-    srw::cast_weights_kernel<<<(unsigned)((W.size() + 255) / 256), 256, 0, s->stream>>>(L.w, L.out, L.in, L.w_bf, L.wt_bf);
+    S_CUDA(s, cudaMemsetAsync(L.gw, 0, sizeof(float) * W.size(), s->stream), "gradients");
+    srw::cast_weights_kernel<<<(unsigned)((W.size() + 255) / 256), 256, 0, s->stream>>>(L.w, (int)W.size(), L.w_bf);
     S_CUDA(s, srw::launch_result(), "cast weights");
   }
   s->adam_t = 0;
@@ -1138,8 +1283,8 @@ srw_status srw_surrogate_create(srw_handle h, const float* centre, const float* 
     if (e == cudaSuccess) e = salloc(&L.gw, nw);
     if (e == cudaSuccess) e = salloc(&L.gb, L.out);
     if (e == cudaSuccess) e = salloc(&L.w_bf, nw);
-    if (e == cudaSuccess) e = salloc(&L.wt_bf, nw);
   }
+  if (e == cudaSuccess) e = salloc(&s->d_step, 1);
   if (e == cudaSuccess) e = salloc(&s->mean, s->n_out_pad);
   if (e == cudaSuccess) e = salloc(&s->stdv, s->n_out_pad);
   if (e == cudaSuccess) e = salloc(&s->binc, s->n_out_pad);
@@ -1208,7 +1353,7 @@ srw_status srw_surrogate_forward(srw_surrogate s, const float* theta, int P, flo
     e = salloc(&B->y, (size_t)M * s->n_out_pad);
     B->fwd_out.E.out_f32 = B->y;
   }
-  if (e == cudaSuccess) e = forward_hidden(s, d_th, P, B, false, s->stream);
+  if (e == cudaSuccess) e = forward_hidden(s, d_th, P, B, s->stream);
   if (e == cudaSuccess) {
     Gemm g = B->fwd_out;
     g.E.rows_valid = P;
@@ -1237,7 +1382,8 @@ srw_status srw_surrogate_gradients(srw_surrogate s, const float* theta, const fl
   S_CUDA(s, cudaMemcpy2DAsync(d_t, sizeof(float) * s->n_out_pad, targets, sizeof(float) * s->n_out,
                               sizeof(float) * s->n_out, P, cudaMemcpyHostToDevice, s->stream),
          "upload targets");
-  cudaError_t e = fit_pass(s, d_th, d_t, P, B, s->stream);
+  cudaError_t e = cudaMemsetAsync(B->loss, 0, sizeof(double), s->stream);
+  if (e == cudaSuccess) e = fit_pass(s, d_th, d_t, P, B, s->stream);
   double sse = 0.0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&sse, B->loss, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
@@ -1277,8 +1423,8 @@ srw_status srw_surrogate_train_step(srw_surrogate s, const float* theta, const f
   S_CUDA(s, cudaMemcpy2DAsync(d_t, sizeof(float) * s->n_out_pad, targets, sizeof(float) * s->n_out,
                               sizeof(float) * s->n_out, P, cudaMemcpyHostToDevice, s->stream),
          "upload targets");
-  cudaError_t e = fit_pass(s, d_th, d_t, P, B, s->stream);
-  if (e == cudaSuccess) e = adam_update(s, lr, 0.9f, 0.999f, 1e-8f, s->stream);
+  cudaError_t e = cudaMemsetAsync(B->loss, 0, sizeof(double), s->stream);
+  if (e == cudaSuccess) e = fit_pass(s, d_th, d_t, P, B, s->stream, lr);
   double sse = 0.0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&sse, B->loss, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
@@ -1358,8 +1504,7 @@ static srw_status fit_impl(srw_surrogate s, const float* theta, long long n, con
       const int rows = (int)std::min<long long>(M, n - b * M);
       const double frac = total > 1 ? (double)t / (double)(total - 1) : 0.0;
       const float lr = (float)(o->lr_final + 0.5 * (o->lr - o->lr_final) * (1.0 + std::cos(3.141592653589793 * frac)));
-      e = fit_pass(s, d_th + b * M * 5, d_t + b * M * NO, rows, B, st, false);
-      if (e == cudaSuccess) e = adam_update(s, lr, 0.9f, 0.999f, 1e-8f, st);
+      e = fit_step(s, d_th + b * M * 5, d_t + b * M * NO, rows, B, st, lr);
     }
     double sse = 0.0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&sse, B->loss, sizeof(double), cudaMemcpyDeviceToHost, st);
@@ -1849,8 +1994,8 @@ srw_status srw_surrogate_load(srw_surrogate s, const char* path, long long* epoc
     off += a.second * sizeof(float);
   }
   for (SurrogateLayer& L : s->L)
-    srw::cast_weights_kernel<<<(unsigned)(((size_t)L.out * L.in + 255) / 256), 256, 0, s->stream>>>(L.w, L.out, L.in,
-                                                                                                  L.w_bf, L.wt_bf);
+    srw::cast_weights_kernel<<<(unsigned)(((size_t)L.out * L.in + 255) / 256), 256, 0, s->stream>>>(
+        L.w, L.out * L.in, L.w_bf);
   S_CUDA(s, srw::launch_result(), "cast weights");
   S_CUDA(s, cudaStreamSynchronize(s->stream), "sync");
   s->adam_t = hd.adam_t;
@@ -2017,13 +2162,18 @@ srw_status srw_surrogate_destroy(srw_surrogate s) {
   for (SurrogateBatch* B : s->batches) free_batch(B);
   for (SurrogateLayer& L : s->L) {
     sfree(L.w); sfree(L.b); sfree(L.mw); sfree(L.vw); sfree(L.mb); sfree(L.vb); sfree(L.gw); sfree(L.gb);
-    sfree(L.w_bf); sfree(L.wt_bf);
+    sfree(L.w_bf);
   }
   sfree(s->mean);
   sfree(s->stdv);
   sfree(s->binc);
   sfree(s->d_status);
   sfree(s->d_sobol);
+  sfree(s->d_step);
+  for (auto& x : s->side)
+    if (x) cudaStreamDestroy(x);
+  for (auto& x : s->fork)
+    if (x) cudaEventDestroy(x);
   if (s->stream) cudaStreamDestroy(s->stream);
   delete s;
   return SRW_OK;

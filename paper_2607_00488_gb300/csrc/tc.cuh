@@ -94,6 +94,18 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t saddr) {
   return d;
 }
 
+// MN-major operand (the tile's rows run along K, 64 BF16 of the M or N
+// dimension each, 128-byte swizzle): 8-row groups along K 1024 bytes apart
+// (SBO), chunks of 64 along M or N `chunk_bytes` apart (LBO).
+__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t saddr, uint32_t chunk_bytes) {
+  uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
+  d |= (uint64_t)(chunk_bytes >> 4) << 16;
+  d |= (uint64_t)(1024u >> 4) << 32;
+  d |= (uint64_t)1u << 46;
+  d |= (uint64_t)2u << 61;
+  return d;
+}
+
 // Descriptor of a K-major tile whose rows hold BK 16-bit elements (BK = 64 or 32).
 template <int BK>
 __device__ __forceinline__ uint64_t smem_desc_k(uint32_t saddr) {
@@ -111,10 +123,11 @@ __device__ __forceinline__ uint32_t swz_offset(int row, int ch) {
                   : (uint32_t)(row * 64 + ((ch ^ ((row >> 1) & 3)) << 4));
 }
 
-// Instruction descriptor, kind::f16, FP32 accumulator, both operands K-major
-// and of one type: BF16 x BF16 (operand format 1) or F16 x F16 (format 0).
-__host__ __device__ constexpr uint32_t idesc_f16kind(int m, int n, bool f16) {
-  return (1u << 4) | ((f16 ? 0u : 1u) << 7) | ((f16 ? 0u : 1u) << 10) | ((uint32_t)(n >> 3) << 17) |
+// Instruction descriptor, kind::f16, FP32 accumulator, operands of one type:
+// BF16 x BF16 (operand format 1) or F16 x F16 (format 0); each K-major, or
+// MN-major where a_mn / b_mn is set.
+__host__ __device__ constexpr uint32_t idesc_f16kind(int m, int n, bool f16, bool a_mn = false, bool b_mn = false) {
+  return (1u << 4) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) | ((f16 ? 0u : 1u) << 7) | ((f16 ? 0u : 1u) << 10) | ((uint32_t)(n >> 3) << 17) |
          ((uint32_t)(m >> 4) << 24);
 }
 
