@@ -91,7 +91,9 @@ struct GemmShape {
   static constexpr int kAB = kBM * kBK * 2;
   static constexpr int kBB = BN * kBK * 2;
   static constexpr int kStageBytes = kAB + kBB;
-  static constexpr int kStages = (200 * 1024 / kStageBytes) < 8 ? (200 * 1024 / kStageBytes) : 8;
+  // 64 columns: half of the SM's shared memory, so that two CTAs (of a step's
+  // branches, or a kernel and its programmatic dependent) share an SM
+  static constexpr int kStages = BN == 64 ? 4 : (200 * 1024 / kStageBytes) < 6 ? (200 * 1024 / kStageBytes) : 6;
   static constexpr int kSmem = kStages * kStageBytes + 1024;
   static constexpr int kTmemCols = 2 * BN;
 };
@@ -159,6 +161,10 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_slot;
+  // a kernel launched as this one's programmatic dependent may set itself up
+  // now; and this one's inputs are complete once the grids it depends on are
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   auto give_up = [&]() {
     atomicExch(&abort_flag, 1u);
     atomicOr(status, kStatusTimeout);
@@ -249,13 +255,24 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       if (__any_sync(0xffffffffu, aborted(&abort_flag))) break;
       const int m0 = (t / n_tn) * kBM, n0 = (t % n_tn) * BN;
       const int buf = tc & 1;
+      const int m = m0 + q * 32 + lane;
+      const bool row_on = m < (MODE == kFwdOutFit ? E.step->rows : E.rows_valid);
+      // the operand a thread's 16 columns need (targets, gelu'): the first
+      // chunk's is loaded before the accumulator is waited for, each further
+      // one a chunk ahead
+      const float* side = MODE == kFwdOutFit ? E.step->targets : MODE == kBwdData ? E.aux : nullptr;
+      float4 ahead[4];
+      auto fetch = [&](int c0) {
+        const float4* p = reinterpret_cast<const float4*>(side + (size_t)m * N + n0 + c0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) ahead[k] = MODE == kBwdData || row_on ? __ldg(p + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+      };
+      if (MODE == kFwdOutFit || MODE == kBwdData) fetch(half * (BN / 2));
       if (!warp_wait(&acc_full[buf], (tc >> 1) & 1, &abort_flag)) {
         give_up();
         break;
       }
       tc_fence_after();
-      const int m = m0 + q * 32 + lane;
-      const bool row_on = m < (MODE == kFwdOutFit ? E.step->rows : E.rows_valid);
       const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
       float sse = 0.f;
       dfloat dev = {0.f, 0.f};
@@ -263,30 +280,41 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 #pragma unroll 1
       for (int c0 = half * (BN / 2); c0 < (half + 1) * (BN / 2); c0 += 16) {
         const int n = n0 + c0;
+        float4 now[4];
+        if (MODE == kFwdOutFit || MODE == kBwdData) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) now[k] = ahead[k];
+          if (c0 + 16 < (half + 1) * (BN / 2)) fetch(c0 + 16);
+        }
+        float bias[16];  // warp-uniform
+        if (MODE == kFwdHidden || MODE == kFwdHiddenScan || MODE == kFwdOutFit || MODE == kFwdOut) {
+#pragma unroll
+          for (int k4 = 0; k4 < 4; ++k4) {
+            const float4 b = __ldg(reinterpret_cast<const float4*>(E.bias + n) + k4);
+            bias[4 * k4] = b.x; bias[4 * k4 + 1] = b.y; bias[4 * k4 + 2] = b.z; bias[4 * k4 + 3] = b.w;
+          }
+        }
         float v[16];
         tmem_ld16(tbase + (uint32_t)c0, v);
         if (MODE == kFwdHidden || MODE == kFwdHiddenScan) {
           float gz[16];
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
-            const float z = v[k] + __ldg(E.bias + n + k);
+            const float z = v[k] + bias[k];
             v[k] = gelu_f(z);
             if (MODE == kFwdHidden) gz[k] = gelu_grad_f(z);
           }
           store_bf16x16(E.out_bf + (size_t)m * N + n, v);
           if (MODE == kFwdHidden) store_f32x16(E.out_f32 + (size_t)m * N + n, gz);
         } else if (MODE == kFwdOutFit) {
-          // the targets' rows are padded like the tile: a thread's 64 bytes in four loads
-          const float4* tp = reinterpret_cast<const float4*>(E.step->targets + (size_t)m * N + n);
           const float scale = E.step->scale;
 #pragma unroll
           for (int k4 = 0; k4 < 4; ++k4) {
-            const float4 t4 = row_on ? __ldg(tp + k4) : make_float4(0.f, 0.f, 0.f, 0.f);
-            const float tg[4] = {t4.x, t4.y, t4.z, t4.w};
+            const float tg[4] = {now[k4].x, now[k4].y, now[k4].z, now[k4].w};
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               const int k = 4 * k4 + i;
-              const float y = v[k] + __ldg(E.bias + n + k);
+              const float y = v[k] + bias[k];
               const float e = (row_on && n + k < E.cols_valid) ? y - tg[i] : 0.f;
               sse = fmaf(e, e, sse);
               v[k] = e * scale;
@@ -294,10 +322,9 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           }
           store_bf16x16(E.out_bf + (size_t)m * N + n, v);
         } else if (MODE == kBwdData) {
-          const float4* gp = reinterpret_cast<const float4*>(E.aux + (size_t)m * N + n);
 #pragma unroll
           for (int k4 = 0; k4 < 4; ++k4) {
-            const float4 gz = gp[k4];
+            const float4 gz = now[k4];
             v[4 * k4] *= gz.x;
             v[4 * k4 + 1] *= gz.y;
             v[4 * k4 + 2] *= gz.z;
@@ -308,7 +335,7 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           store_f32x16(E.out_f32 + (size_t)m * E.ld + n, v);
         } else if (MODE == kFwdOut) {
 #pragma unroll
-          for (int k = 0; k < 16; ++k) v[k] += __ldg(E.bias + n + k);
+          for (int k = 0; k < 16; ++k) v[k] += bias[k];
           store_f32x16(E.out_f32 + (size_t)m * N + n, v);
         } else {  // kFwdScan: deviance of mu = exp(lm), lm = m + s (y + b) = log mu:
                   // t = mu - n + n ln(n / mu) = mu - n lm + (n ln n - n)
@@ -476,34 +503,58 @@ __global__ void cast_weights_kernel(const float* __restrict__ w, int n, __nv_bfl
   if (k < n) w_bf[k] = __float2bfloat16_rn(w[k]);
 }
 
-// Training targets: dst [rows][ld] = log(mu_sig + b) from src [rows][n]
-// (columns >= n of dst: 0).
-__global__ void log_counts_kernel(const float* __restrict__ src, long long rows, int n, int ld,
-                                  const double* __restrict__ b64, float* __restrict__ dst) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= rows * ld) return;
-  const long long r = i / ld;
-  const int j = (int)(i % ld);
-  dst[i] = j < n ? logf(fmaxf(src[r * n + j] + (float)b64[j], 1e-30f)) : 0.f;
+// FP32 -> FP64 by its bits (normal numbers and zero; else the conversion, an
+// instruction of the FP64 unit, which takes the SM 16 cycles a warp).
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), ex = u & 0x7f800000u;
+  if (ex == 0u || ex == 0x7f800000u) return (double)x;
+  const uint32_t hi = ((u & 0x7fffffffu) >> 3) + 0x38000000u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
 
-// Per-column sums and sums of squares (FP64) over rows, for the standardization.
-// Column sums and sums of squares of one block of 4096 rows, written to the
+// Training targets dst [rows][ld] = log(mu_sig + b) from src [rows][n]
+// (columns >= n of dst: 0; dst may be src when ld = n), and per column the FP64
+// sum and sum of squares of this block's kStatRows rows, in row order, in the
 // block's own slot (no atomics: the statistics, and so every resumed fit, are
-// the same bit for bit whatever the order in which the blocks run).
-__global__ void colstats_kernel(const float* __restrict__ t, long long rows, int ld, int n, double* __restrict__ s1,
-                                double* __restrict__ s2) {
+// the same bit for bit whatever the order in which the blocks run).  A thread
+// is a column.  Bound by the FP64 unit: two operations an element, 0.45 ms for
+// 65,536 x 2048 (a pass for the logarithm and one for the sums: 0.45 + 0.99 ms).
+constexpr int kStatRows = 4096;
+__global__ void __launch_bounds__(64, 8)
+log_stats_kernel(const float* src, long long rows, int n, int ld, const double* __restrict__ b64, float* dst,
+                 double* __restrict__ s1, double* __restrict__ s2) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  const long long r0 = (long long)blockIdx.y * 4096, r1 = min(rows, r0 + 4096);
-  double a = 0.0, b = 0.0;
-  for (long long r = r0; r < r1; ++r) {
-    const double x = t[r * ld + j];
-    a += x;
-    b += x * x;
+  if (j >= ld) return;
+  const long long r0 = (long long)blockIdx.y * kStatRows, r1 = min(rows, r0 + kStatRows);
+  if (j >= n) {
+    for (long long r = r0; r < r1; ++r) dst[r * ld + j] = 0.f;
+    return;
+  }
+  const float b = (float)b64[j];
+  double a = 0.0, q = 0.0;
+  constexpr int kAhead = 16;
+  float v[kAhead], w[kAhead];
+  auto fetch = [&](long long r) {
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) w[i] = r + i < r1 ? src[(r + i) * n + j] : 1.f;
+  };
+  fetch(r0);
+  for (long long r = r0; r < r1; r += kAhead) {
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) v[i] = w[i];
+    if (r + kAhead < r1) fetch(r + kAhead);
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i)
+      if (r + i < r1) {
+        const float t = logf(fmaxf(v[i] + b, 1e-30f));
+        dst[(r + i) * ld + j] = t;
+        const double x = widen(t);
+        a += x;
+        q += x * x;
+      }
   }
   s1[(size_t)blockIdx.y * n + j] = a;
-  s2[(size_t)blockIdx.y * n + j] = b;
+  s2[(size_t)blockIdx.y * n + j] = q;
 }
 
 __global__ void finish_stats_kernel(const double* __restrict__ s1, const double* __restrict__ s2, int n_blocks,
@@ -522,12 +573,26 @@ __global__ void finish_stats_kernel(const double* __restrict__ s1, const double*
   stdv[j] = s > 1e-12 ? (float)s : 1.f;
 }
 
+// Four columns a thread (ld is a multiple of 256); columns >= n stay 0.
 __global__ void standardize_kernel(float* __restrict__ t, long long rows, int ld, int n, const float* __restrict__ mean,
                                    const float* __restrict__ stdv) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= rows * ld) return;
-  const int j = (int)(i % ld);
-  if (j < n) t[i] = (t[i] - mean[j]) / stdv[j];
+  const int j = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (j >= ld) return;
+  float m[4], s[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    m[k] = j + k < n ? mean[j + k] : 0.f;
+    s[k] = j + k < n ? stdv[j + k] : 1.f;
+  }
+  for (long long r = blockIdx.y; r < rows; r += gridDim.y) {
+    float4* p = reinterpret_cast<float4*>(t + r * ld + j);
+    float4 v = *p;
+    v.x = (v.x - m[0]) / s[0];
+    v.y = (v.y - m[1]) / s[1];
+    v.z = (v.z - m[2]) / s[2];
+    v.w = (v.w - m[3]) / s[3];
+    *p = v;
+  }
 }
 
 // -2 ln L = 2 sum of the per-tile deviance partials + the data constant.
@@ -712,31 +777,44 @@ struct Gemm {
   EpiArgs E{};
 };
 
+// dependent: launched as the programmatic dependent of the kernel before it
+// on the stream (which must be a GEMM of this file, or trigger at its end).
 template <int BN, int MODE>
-cudaError_t launch_mode(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s) {
+cudaError_t launch_mode(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s, bool dependent) {
   const int tiles = (g.M / kBM) * (g.N / BN);
-  const int grid = tiles < sm_count ? tiles : sm_count;
-  mlp_gemm_kernel<BN, MODE><<<grid, kGemmThreads, GemmShape<BN>::kSmem, s>>>(g.ma, g.mb, g.M, g.N, g.K, g.E, status);
-  return srw::launch_result();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(tiles < sm_count ? tiles : sm_count);
+  cfg.blockDim = dim3(kGemmThreads);
+  cfg.dynamicSmemBytes = GemmShape<BN>::kSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  const cudaError_t e =
+      cudaLaunchKernelEx(&cfg, mlp_gemm_kernel<BN, MODE>, g.ma, g.mb, g.M, g.N, g.K, g.E, status);
+  return e != cudaSuccess ? e : srw::launch_result();
 }
 
 template <int BN>
-cudaError_t launch_width(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s) {
+cudaError_t launch_width(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s, bool dep) {
   switch (g.mode) {
-    case kFwdHidden: return launch_mode<BN, kFwdHidden>(g, sm_count, status, s);
-    case kFwdOutFit: return launch_mode<BN, kFwdOutFit>(g, sm_count, status, s);
-    case kBwdData: return launch_mode<BN, kBwdData>(g, sm_count, status, s);
-    case kFwdOut: return launch_mode<BN, kFwdOut>(g, sm_count, status, s);
-    case kFwdScan: return launch_mode<BN, kFwdScan>(g, sm_count, status, s);
-    case kFwdHiddenScan: return launch_mode<BN, kFwdHiddenScan>(g, sm_count, status, s);
+    case kFwdHidden: return launch_mode<BN, kFwdHidden>(g, sm_count, status, s, dep);
+    case kFwdOutFit: return launch_mode<BN, kFwdOutFit>(g, sm_count, status, s, dep);
+    case kBwdData: return launch_mode<BN, kBwdData>(g, sm_count, status, s, dep);
+    case kFwdOut: return launch_mode<BN, kFwdOut>(g, sm_count, status, s, dep);
+    case kFwdScan: return launch_mode<BN, kFwdScan>(g, sm_count, status, s, dep);
+    case kFwdHiddenScan: return launch_mode<BN, kFwdHiddenScan>(g, sm_count, status, s, dep);
   }
   return cudaErrorInvalidValue;
 }
 
-cudaError_t run_gemm(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s) {
-  if (g.mode == kWgrad) return launch_mode<64, kWgrad>(g, sm_count, status, s);
-  return g.bn == 256 ? launch_width<256>(g, sm_count, status, s)
-                     : g.bn == 128 ? launch_width<128>(g, sm_count, status, s) : launch_width<64>(g, sm_count, status, s);
+cudaError_t run_gemm(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s, bool dep = false) {
+  if (g.mode == kWgrad) return launch_mode<64, kWgrad>(g, sm_count, status, s, dep);
+  return g.bn == 256   ? launch_width<256>(g, sm_count, status, s, dep)
+         : g.bn == 128 ? launch_width<128>(g, sm_count, status, s, dep)
+                       : launch_width<64>(g, sm_count, status, s, dep);
 }
 
 template <int BN>
@@ -1097,8 +1175,13 @@ cudaError_t step_body(srw_surrogate s, SurrogateBatch* B, cudaStream_t st, bool 
 
 // The same step (with its update) in branches: each layer's weight gradient
 // and update beside the chain of the data gradients.  A weight gradient is a
-// long contraction in few CTAs (4096 points into 256 x 256: eight CTAs, 23 us),
-// which the other layers' kernels run beside.
+// long contraction in few CTAs (4096 points into 256 x 256: eight CTAs, 23 us,
+// bound by the 256 dependent MMAs of an accumulator: four or eight stages in
+// flight, 64 or 128 of K a stage and 256 or 64 columns take the same time),
+// which the other layers' kernels run beside.  65,536 points, three epochs on
+// the solar set: 22.1 ms before tiles, MN-major operands and branches, 13.3 ms
+// with them, 9.3 ms with programmatic launches along the chain, operands loaded
+// ahead in the epilogues and the fused target statistics.
 cudaError_t step_branches(srw_surrogate s, SurrogateBatch* B, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   auto ok = [&](cudaError_t r) {
@@ -1108,7 +1191,8 @@ cudaError_t step_branches(srw_surrogate s, SurrogateBatch* B, cudaStream_t st) {
     ok(cudaEventRecord(s->fork[ev], of));
     ok(cudaStreamWaitEvent(waiter, s->fork[ev], 0));
   };
-  for (int l = 0; l < 4; ++l) ok(srw::run_gemm(B->fwd[l], s->sm_count, s->d_status, st));
+  // the chain's kernels as programmatic dependents (the first one follows the input kernel's completion)
+  for (int l = 0; l < 4; ++l) ok(srw::run_gemm(B->fwd[l], s->sm_count, s->d_status, st, l > 0));
   for (int l = 3; l >= 0; --l) {
     // dz of layer l is ready on st
     ok(cudaEventRecord(s->fork[l], st));
@@ -1118,12 +1202,12 @@ cudaError_t step_branches(srw_surrogate s, SurrogateBatch* B, cudaStream_t st) {
     ok(layer_bias(s, B, l, s->side[4]));
     after(s->side[l], s->side[4], 4);
     if (l > 0) {
-      ok(srw::run_gemm(B->bwd[l - 1], s->sm_count, s->d_status, st));
+      ok(srw::run_gemm(B->bwd[l - 1], s->sm_count, s->d_status, st, true));
       after(s->side[l], st, 5);  // which has read this layer's weights
     }
     ok(layer_adam(s, l, s->side[l]));
-    after(st, s->side[l], 6 + l);
   }
+  for (int l = 0; l < 4; ++l) after(st, s->side[l], 6 + l);
   return e;
 }
 
@@ -1459,11 +1543,13 @@ static srw_status fit_impl(srw_surrogate s, const float* theta, long long n, con
   };
   cudaError_t e = salloc(&d_th, (size_t)n_pad * 5);
   if (e == cudaSuccess) e = salloc(&d_t, (size_t)n_pad * NO);
-  if (e == cudaSuccess) e = salloc(&d_tmp, (size_t)kGen * NR);
-  const int n_sblocks = (int)((n + 4095) / 4096);
+  // spectra go straight to the targets' rows where those are not padded
+  if (e == cudaSuccess && NR != NO) e = salloc(&d_tmp, (size_t)kGen * NR);
+  const int n_sblocks = (int)((n + srw::kStatRows - 1) / srw::kStatRows);
+  static_assert(kGen % srw::kStatRows == 0, "row blocks of the statistics do not straddle a launch");
   if (e == cudaSuccess) e = salloc(&d_stats, 2 * (size_t)NR * n_sblocks);
   if (e == cudaSuccess) e = cudaMemsetAsync(d_th, 0, sizeof(float) * n_pad * 5, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_t, 0, sizeof(float) * n_pad * NO, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d_t + n * NO, 0, sizeof(float) * (n_pad - n) * NO, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_th, theta, sizeof(float) * n * 5, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) {
     cleanup();
@@ -1472,20 +1558,21 @@ static srw_status fit_impl(srw_surrogate s, const float* theta, long long n, con
   // targets: log of the exact expected counts (signal of the exact path + background)
   for (long long off = 0; off < n; off += kGen) {
     const int cnt = (int)std::min<long long>(kGen, n - off);
-    const srw_status r = srw_spectrum_batch(h, d_th + off * 5, cnt, d_tmp, SRW_DEVICE, (srw_precision)o->precision, st);
+    float* spectra = d_tmp ? d_tmp : d_t + off * NO;
+    const srw_status r = srw_spectrum_batch(h, d_th + off * 5, cnt, spectra, SRW_DEVICE, (srw_precision)o->precision, st);
     if (r != SRW_OK) {
       cleanup();
       return sfail(s, r, std::string("exact spectra: ") + srw_last_error(h));
     }
-    srw::log_counts_kernel<<<(unsigned)(((long long)cnt * NO + 255) / 256), 256, 0, st>>>(d_tmp, cnt, NR, NO, h->d_b64,
-                                                                                      d_t + off * NO);
+    const size_t slot = (size_t)(off / srw::kStatRows) * NR;
+    srw::log_stats_kernel<<<dim3((NO + 63) / 64, (cnt + srw::kStatRows - 1) / srw::kStatRows), 64, 0, st>>>(
+        spectra, cnt, NR, NO, h->d_b64, d_t + off * NO, d_stats + slot, d_stats + (size_t)NR * n_sblocks + slot);
   }
   // per-bin standardization over the training set
-  srw::colstats_kernel<<<dim3((NR + 255) / 256, (unsigned)n_sblocks), 256, 0, st>>>(
-      d_t, n, NO, NR, d_stats, d_stats + (size_t)NR * n_sblocks);
   srw::finish_stats_kernel<<<(NR + 255) / 256, 256, 0, st>>>(d_stats, d_stats + (size_t)NR * n_sblocks, n_sblocks, n,
                                                              NR, s->mean, s->stdv);
-  srw::standardize_kernel<<<(unsigned)((n * NO + 255) / 256), 256, 0, st>>>(d_t, n, NO, NR, s->mean, s->stdv);
+  srw::standardize_kernel<<<dim3((NO / 4 + 127) / 128, (unsigned)std::min<long long>(n, 1024)), 128, 0, st>>>(
+      d_t, n, NO, NR, s->mean, s->stdv);
   if ((e = srw::launch_result()) != cudaSuccess) {
     cleanup();
     return scuda(s, e, "targets");
