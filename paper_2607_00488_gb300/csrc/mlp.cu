@@ -40,6 +40,7 @@
 #include <vector>
 
 #include "dfloat.cuh"
+#include "f32x2.cuh"
 #include "poisson.cuh"
 #include "ptx.cuh"
 #include "srw_internal.h"
@@ -54,13 +55,16 @@ constexpr int kBM = 128;
 constexpr int kBK = 64;
 constexpr int kTmaWarp = 0;
 constexpr int kMmaWarp = 1;
-constexpr int kEpiWarps = 8;                     // two per TMEM lane quarter, each on half the columns
-constexpr int kGemmThreads = (2 + kEpiWarps) * 32;
 constexpr int kIn = 5;          // theta components
 constexpr int kInPad = 128;     // padded input width (one 128-row operand tile)
 constexpr int kHidden = 256;
 
 enum EpiMode { kFwdHidden = 0, kFwdOutFit = 1, kBwdData = 2, kWgrad = 3, kFwdOut = 4, kFwdScan = 5, kFwdHiddenScan = 6 };
+
+// Epilogue warps: two per TMEM lane quarter, each on half the columns; four in
+// the scan's hidden layers, whose epilogue (erf) bounds them by issue.
+constexpr int epi_warps(int mode) { return mode == kFwdHiddenScan ? 16 : 8; }
+constexpr int gemm_threads(int mode) { return (2 + epi_warps(mode)) * 32; }
 
 struct EpiArgs {
   int M, N;              // output rows, columns (multiples of 128 and of the tile width)
@@ -73,8 +77,9 @@ struct EpiArgs {
   const float* aux;      // backward data: gelu'(z) [M][N]
   const struct StepParams* step;  // fit: the step's targets, rows and error scale
   double* loss;          // fit: += sum of squared errors
-  const float4* binc;    // scan: per bin {m_j + s_j b_j, s_j, n_j, n_j ln n_j - n_j} (masked: {0, 0, 0, -1})
-  double* parts;         // scan: per (column half-tile, row) partial sums of the deviance
+  // scan: per tile of 128 bins the rows m_j + s_j b_j, s_j, -n_j and n_j ln n_j - n_j (masked bins: 0, 0, 0, -1)
+  const float* binc;
+  double* parts;         // scan: partial sums of the deviance (mlp_scan_kernel)
 };
 
 // What one training step differs in from the next (device memory, written by
@@ -119,11 +124,12 @@ __device__ __forceinline__ void store_f32x16(float* dst, const float* v) {
 }
 
 template <int BN, int MODE>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(gemm_threads(MODE), 1)
 mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M, int N,
                 int K, const EpiArgs E, unsigned* status) {
   using S = GemmShape<BN>;
   constexpr int ST = S::kStages;
+  constexpr int kEpiWarps = epi_warps(MODE), kSpan = BN / (kEpiWarps / 4);  // columns of an epilogue warp
   constexpr bool kAMn = MODE == kWgrad, kBMn = MODE == kWgrad || MODE == kBwdData;
   constexpr uint32_t kMnChunk = 64 * kBK * 2;  // bytes of a 64 x 64 box
   extern __shared__ unsigned char dsmem_raw[];
@@ -204,51 +210,51 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         ptx::mbar_wait(&full[u % ST], (u / ST) & 1, nullptr, 100000000ull);
     }
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_f16kind(kBM, BN, false, kAMn, kBMn);
-      int g = 0, tc = -1;
-      bool issued_any = false;
-      for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-        ++tc;
-        if (aborted(&abort_flag)) break;
-        const int buf = tc & 1;
-        if (!ptx::mbar_wait(&acc_empty[buf], ((tc >> 1) & 1) ^ 1, &abort_flag)) {
+    // the whole warp walks the tiles; its elected lane issues
+    constexpr uint32_t idesc = idesc_f16kind(kBM, BN, false, kAMn, kBMn);
+    const uint32_t leader = elect_one();
+    int g = 0, tc = -1;
+    bool issued_any = false;
+    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+      ++tc;
+      const int buf = tc & 1;
+      if (!warp_wait(&acc_empty[buf], ((tc >> 1) & 1) ^ 1, &abort_flag)) {
+        give_up();
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
+      bool ok = true;
+      for (int kb = 0; kb < n_kb; ++kb, ++g) {
+        const int st = g % ST;
+        if (!warp_wait(&full[st], (g / ST) & 1, &abort_flag)) {
           give_up();
+          ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
-        bool ok = true;
-        for (int kb = 0; kb < n_kb; ++kb, ++g) {
-          const int st = g % ST;
-          if (!ptx::mbar_wait(&full[st], (g / ST) & 1, &abort_flag)) {
-            give_up();
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t as = ptx::smem_addr(a_s(st)), bs = ptx::smem_addr(b_s(st));
+        const uint32_t as = ptx::smem_addr(a_s(st)), bs = ptx::smem_addr(b_s(st));
+        const uint64_t ad = kAMn ? smem_desc_mn(as, kMnChunk) : smem_desc_sw128(as);
+        const uint64_t bd = kBMn ? smem_desc_mn(bs, kMnChunk) : smem_desc_sw128(bs);
 #pragma unroll
-          for (int ks = 0; ks < kBK / 16; ++ks)
-            // 16 of K: 32 bytes along a K-major row, 16 rows of 128 bytes of an MN-major tile
-            mma_bf16(d_tmem, kAMn ? smem_desc_mn(as + ks * 2048u, kMnChunk) : smem_desc_sw128(as + ks * 32u),
-                     kBMn ? smem_desc_mn(bs + ks * 2048u, kMnChunk) : smem_desc_sw128(bs + ks * 32u), idesc,
-                     (kb | ks) != 0);
-          issued_any = true;
-          mma_commit(&empty[st]);
-        }
-        if (!ok) break;
-        mma_commit(&acc_full[buf]);
+        for (int ks = 0; ks < kBK / 16; ++ks)
+          // 16 of K, in the descriptors' 16-byte units: 32 bytes along a K-major row, 16 rows of 128 bytes of
+          // an MN-major tile
+          mma_bf16_warp(d_tmem, ad + (kAMn ? 128 : 2) * ks, bd + (kBMn ? 128 : 2) * ks, idesc, (kb | ks) != 0, leader);
+        issued_any = true;
+        mma_commit_warp(&empty[st], leader);
       }
-      if (issued_any) {
-        mma_commit(&drain);
-        ptx::mbar_wait(&drain, 0, nullptr, 100000000ull);
-      }
+      if (!ok) break;
+      mma_commit_warp(&acc_full[buf], leader);
+    }
+    if (issued_any) {
+      mma_commit_warp(&drain, leader);
+      ptx::mbar_wait(&drain, 0, nullptr, 100000000ull);
     }
   } else {
     // ------------------------------------------------------------ epilogue
     const int q = warp & 3;                  // TMEM lanes 32 q .. 32 q + 31
-    const int half = (warp - 2) >> 2;        // columns [half BN/2, (half + 1) BN/2)
+    const int part = (warp - 2) >> 2;        // columns [part kSpan, (part + 1) kSpan)
     int tc = -1;
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
       ++tc;
@@ -267,7 +273,7 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 #pragma unroll
         for (int k = 0; k < 4; ++k) ahead[k] = MODE == kBwdData || row_on ? __ldg(p + k) : make_float4(0.f, 0.f, 0.f, 0.f);
       };
-      if (MODE == kFwdOutFit || MODE == kBwdData) fetch(half * (BN / 2));
+      if (MODE == kFwdOutFit || MODE == kBwdData) fetch(part * kSpan);
       if (!warp_wait(&acc_full[buf], (tc >> 1) & 1, &abort_flag)) {
         give_up();
         break;
@@ -275,16 +281,14 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       tc_fence_after();
       const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
       float sse = 0.f;
-      dfloat dev = {0.f, 0.f};
-      bool infinite = false;
 #pragma unroll 1
-      for (int c0 = half * (BN / 2); c0 < (half + 1) * (BN / 2); c0 += 16) {
+      for (int c0 = part * kSpan; c0 < (part + 1) * kSpan; c0 += 16) {
         const int n = n0 + c0;
         float4 now[4];
         if (MODE == kFwdOutFit || MODE == kBwdData) {
 #pragma unroll
           for (int k = 0; k < 4; ++k) now[k] = ahead[k];
-          if (c0 + 16 < (half + 1) * (BN / 2)) fetch(c0 + 16);
+          if (c0 + 16 < (part + 1) * kSpan) fetch(c0 + 16);
         }
         float bias[16];  // warp-uniform
         if (MODE == kFwdHidden || MODE == kFwdHiddenScan || MODE == kFwdOutFit || MODE == kFwdOut) {
@@ -333,21 +337,10 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           store_bf16x16(E.out_bf + (size_t)m * N + n, v);
         } else if (MODE == kWgrad) {
           store_f32x16(E.out_f32 + (size_t)m * E.ld + n, v);
-        } else if (MODE == kFwdOut) {
+        } else {  // kFwdOut
 #pragma unroll
           for (int k = 0; k < 16; ++k) v[k] += bias[k];
           store_f32x16(E.out_f32 + (size_t)m * N + n, v);
-        } else {  // kFwdScan: deviance of mu = exp(lm), lm = m + s (y + b) = log mu:
-                  // t = mu - n + n ln(n / mu) = mu - n lm + (n ln n - n)
-          float ts = 0.f;
-#pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const float4 c = __ldg(E.binc + n + k);
-            const float lm = fmaf(c.y, v[k], c.x);
-            ts += fmaf(-c.z, lm, __expf(lm) + c.w);
-          }
-          if (isinf(ts)) infinite = true;
-          else dev = df_add(dev, ts);
         }
       }
       tc_fence_before();
@@ -358,9 +351,6 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         for (int o = 16; o > 0; o >>= 1) sse += __shfl_xor_sync(0xffffffffu, sse, o);
         if (lane == 0) atomicAdd(E.loss, (double)sse);
       }
-      if (MODE == kFwdScan && row_on)
-        E.parts[((size_t)(n0 / BN) * 2 + half) * E.rows_valid + m] =
-            infinite ? __longlong_as_double(0x7ff0000000000000LL) : (double)dev.hi + (double)dev.lo;
     }
   }
 
@@ -368,6 +358,234 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   __syncthreads();
   tc_fence_after();
   if (warp == kMmaWarp) tmem_dealloc(tmem_base, S::kTmemCols);
+}
+
+// Output layer of a scan fused with its Poisson deviance: per point the sum over
+// the bins of t = mu - n + n ln(n / mu) = mu - n lm + (n ln n - n), mu = exp(lm),
+// lm = m + s (y + b) = log mu, with the constants of E.binc.
+//
+// Three units are near balance per 128 x 256 outputs (about 2000 cycles each):
+// the tensor core, the exponentials (16 a cycle) and the instruction issue; as
+// an epilogue of the general GEMM the layer took 6400, with eight warps each
+// loading 16 bytes of constants per output and 192 KB of operands per tile.
+// Here a CTA keeps the activations of 256 points (128 KB) and streams the
+// weights and the bins' constants past them, 128 bins at a time; a lane owns
+// two points, so the constants serve both, and takes two bins at a time in
+// packed FP32; sixteen warps take a quarter of the lanes and of the bins each,
+// and the sums stay in registers over all of the CTA's bins.
+//
+// Unit: 256 points x the bins of one of `groups` equal parts (more parts for
+// small batches).  Partial sums: parts[group * 4 + quarter of the bins][row].
+constexpr int kScanWarps = 16;
+constexpr int kScanThreads = (2 + kScanWarps) * 32;
+constexpr int kScanRows = 2 * kBM, kScanBins = 128, kScanKb = kHidden / kBK, kScanRing = 5;
+constexpr int kScanTile = kBM * kBK * 2;  // bytes of a 128 x 64 operand tile
+constexpr int kScanConsts = 4 * kScanBins * 4;  // bytes of a tile's constants, see EpiArgs::binc
+constexpr int kScanSmem = (2 * kScanKb + kScanRing) * kScanTile + 2 * kScanConsts + 1024;
+
+// Two bins' terms exp(lm) + w - n lm with lm = x + y v (nz = -n); exp as
+// 2^(lm log2 e) with the hardware's exponential.
+__device__ __forceinline__ float2 scan_terms(uint64_t v, uint64_t x, uint64_t y, uint64_t nz, uint64_t w) {
+  const uint64_t lm = fma2(y, v, x);
+  const float2 e = unpk(mul2(lm, pk(1.44269504f, 1.44269504f)));
+  float a, b;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(e.x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(b) : "f"(e.y));
+  return unpk(fma2(nz, lm, add2(pk(a, b), w)));
+}
+
+__global__ void __launch_bounds__(kScanThreads, 1)
+mlp_scan_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M, int N,
+                int groups, const EpiArgs E, unsigned* status) {
+  extern __shared__ unsigned char dsmem_raw[];
+  unsigned char* smem = dsmem_raw + ((1024u - (ptx::smem_addr(dsmem_raw) & 1023u)) & 1023u);
+  __shared__ __align__(8) uint64_t a_full[kScanKb], a_empty[kScanKb], b_full[kScanRing], b_empty[kScanRing];
+  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], c_full[2], c_empty[2], drain;
+  __shared__ uint32_t tmem_slot;
+  __shared__ unsigned abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int units = (M / kScanRows) * groups, tiles = N / kScanBins / groups;  // bins: `tiles` tiles of a unit
+  auto a_s = [&](int kb, int h) { return smem + (size_t)(2 * kb + h) * kScanTile; };
+  auto b_s = [&](int st) { return smem + (size_t)(2 * kScanKb + st) * kScanTile; };
+  auto c_s = [&](int sl) { return smem + (size_t)(2 * kScanKb + kScanRing) * kScanTile + (size_t)sl * kScanConsts; };
+
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < kScanKb; ++k) {
+      ptx::mbar_init(&a_full[k], 1);
+      ptx::mbar_init(&a_empty[k], 1);
+    }
+    for (int k = 0; k < kScanRing; ++k) {
+      ptx::mbar_init(&b_full[k], 1);
+      ptx::mbar_init(&b_empty[k], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      ptx::mbar_init(&acc_full[b], 1);
+      ptx::mbar_init(&acc_empty[b], kScanWarps);
+      ptx::mbar_init(&c_full[b], 1);
+      ptx::mbar_init(&c_empty[b], kScanWarps);
+    }
+    ptx::mbar_init(&drain, 1);
+    abort_flag = 0u;
+    ptx::fence_barrier_init();
+  }
+  if (warp == kMmaWarp) tmem_alloc(&tmem_slot, 512);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_slot;
+  auto give_up = [&]() {
+    atomicExch(&abort_flag, 1u);
+    atomicOr(status, kStatusTimeout);
+  };
+
+  if (warp == kTmaWarp) {
+    if (lane == 0) {
+      int g = 0, tc = 0, ua = 0;  // weight tiles, tiles of constants and units whose copies were posted
+      int a_posted[kScanKb] = {};
+      bool ok = true;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++ua) {
+        const int m0 = (u / groups) * kScanRows, n0 = (u % groups) * tiles * kScanBins;
+        for (int t = 0; t < tiles && ok; ++t) {
+          const int sl = tc & 1;
+          if (!ptx::mbar_wait(&c_empty[sl], ((tc >> 1) & 1) ^ 1, &abort_flag)) {
+            ok = false;
+            break;
+          }
+          ptx::mbar_arrive_expect_tx(&c_full[sl], kScanConsts);
+          ptx::bulk_g2s(c_s(sl), E.binc + (size_t)(n0 + t * kScanBins) * 4, kScanConsts, &c_full[sl]);
+          ++tc;
+          for (int kb = 0; kb < kScanKb; ++kb, ++g) {
+            if (t == 0) {  // the unit's activations, a K block as soon as the last unit's products left it
+              if (!ptx::mbar_wait(&a_empty[kb], (ua & 1) ^ 1, &abort_flag)) {
+                ok = false;
+                break;
+              }
+              ptx::mbar_arrive_expect_tx(&a_full[kb], 2 * kScanTile);
+              tma_load_2d(a_s(kb, 0), &map_a, kb * kBK, m0, &a_full[kb]);
+              tma_load_2d(a_s(kb, 1), &map_a, kb * kBK, m0 + kBM, &a_full[kb]);
+              ++a_posted[kb];
+            }
+            const int st = g % kScanRing;
+            if (!ptx::mbar_wait(&b_empty[st], ((g / kScanRing) & 1) ^ 1, &abort_flag)) {
+              ok = false;
+              break;
+            }
+            ptx::mbar_arrive_expect_tx(&b_full[st], kScanTile);
+            tma_load_2d(b_s(st), &map_b, kb * kBK, n0 + t * kScanBins, &b_full[st]);
+          }
+        }
+      }
+      if (!ok) give_up();
+      // never end with copies in flight
+      for (int q = max(0, g - kScanRing); q < g; ++q)
+        ptx::mbar_wait(&b_full[q % kScanRing], (q / kScanRing) & 1, nullptr, 100000000ull);
+      for (int q = max(0, tc - 2); q < tc; ++q) ptx::mbar_wait(&c_full[q & 1], (q >> 1) & 1, nullptr, 100000000ull);
+      for (int kb = 0; kb < kScanKb; ++kb)
+        if (a_posted[kb] > 0) ptx::mbar_wait(&a_full[kb], (a_posted[kb] - 1) & 1, nullptr, 100000000ull);
+    }
+  } else if (warp == kMmaWarp) {
+    constexpr uint32_t idesc = idesc_f16kind(kBM, kScanBins, false);
+    const uint32_t leader = elect_one();
+    int g = 0, tc = 0, ua = 0;
+    bool ok = true, issued_any = false;
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++ua)
+      for (int t = 0; t < tiles && ok; ++t, ++tc) {
+        const int buf = tc & 1;
+        if (!warp_wait(&acc_empty[buf], ((tc >> 1) & 1) ^ 1, &abort_flag)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        for (int kb = 0; kb < kScanKb; ++kb, ++g) {
+          const int st = g % kScanRing;
+          if ((t == 0 && !warp_wait(&a_full[kb], ua & 1, &abort_flag)) ||
+              !warp_wait(&b_full[st], (g / kScanRing) & 1, &abort_flag)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint64_t bd = smem_desc_sw128(ptx::smem_addr(b_s(st)));
+          const uint64_t a0 = smem_desc_sw128(ptx::smem_addr(a_s(kb, 0)));
+          const uint64_t a1 = smem_desc_sw128(ptx::smem_addr(a_s(kb, 1)));
+          const uint32_t d = tmem_base + (uint32_t)(buf * 256);
+#pragma unroll
+          for (int ks = 0; ks < kBK / 16; ++ks) {  // 16 of K: 32 bytes, 2 in the descriptor's address field
+            mma_bf16_warp(d, a0 + 2 * ks, bd + 2 * ks, idesc, (kb | ks) != 0, leader);
+            mma_bf16_warp(d + kScanBins, a1 + 2 * ks, bd + 2 * ks, idesc, (kb | ks) != 0, leader);
+          }
+          issued_any = true;
+          mma_commit_warp(&b_empty[st], leader);
+          if (t == tiles - 1) mma_commit_warp(&a_empty[kb], leader);
+        }
+        if (ok) mma_commit_warp(&acc_full[buf], leader);
+      }
+    if (!ok) give_up();
+    if (issued_any) {
+      mma_commit_warp(&drain, leader);
+      ptx::mbar_wait(&drain, 0, nullptr, 100000000ull);
+    }
+  } else {
+    const int q = warp & 3, part = (warp - 2) >> 2;  // lanes 32 q ..; bins 32 part .. of a tile
+    int tc = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+      const int m = (u / groups) * kScanRows + q * 32 + lane, n0 = (u % groups) * tiles * kScanBins;
+      dfloat dev[2] = {{0.f, 0.f}, {0.f, 0.f}};
+      bool infinite[2] = {false, false};
+      for (int t = 0; t < tiles; ++t, ++tc) {
+        const int buf = tc & 1;
+        if (!warp_wait(&c_full[buf], (tc >> 1) & 1, &abort_flag) ||
+            !warp_wait(&acc_full[buf], (tc >> 1) & 1, &abort_flag)) {
+          give_up();
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + part * 32);
+        const ulonglong2* cs = reinterpret_cast<const ulonglong2*>(c_s(buf)) + part * 8;  // 4 bins each, rows of 32
+#pragma unroll 1
+        for (int c0 = 0; c0 < 32; c0 += 16) {
+          float v[2][16];
+          tmem_ld16(tbase + (uint32_t)c0, v[0]);
+          tmem_ld16(tbase + (uint32_t)(kScanBins + c0), v[1]);
+          float ts[2] = {0.f, 0.f};
+#pragma unroll
+          for (int k = 0; k < 16; k += 4) {
+            const ulonglong2* c = cs + (c0 + k) / 4;
+            const ulonglong2 cx = c[0], cy = c[32], cz = c[64], cw = c[96];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float2 t0 = scan_terms(pk(v[h][k], v[h][k + 1]), cx.x, cy.x, cz.x, cw.x);
+              const float2 t1 = scan_terms(pk(v[h][k + 2], v[h][k + 3]), cx.y, cy.y, cz.y, cw.y);
+              ts[h] = (((ts[h] + t0.x) + t0.y) + t1.x) + t1.y;
+            }
+          }
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (isinf(ts[h])) infinite[h] = true;
+            else dev[h] = df_add(dev[h], ts[h]);
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          ptx::mbar_arrive(&acc_empty[buf]);
+          ptx::mbar_arrive(&c_empty[buf]);
+        }
+      }
+      if (!ok) break;
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (m + h * kBM < E.rows_valid)
+          E.parts[(size_t)((u % groups) * 4 + part) * E.rows_valid + m + h * kBM] =
+              infinite[h] ? __longlong_as_double(0x7ff0000000000000LL) : (double)dev[h].hi + (double)dev[h].lo;
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == kMmaWarp) tmem_dealloc(tmem_base, 512);
 }
 
 // theta [rows][5] -> X0 [M][128] (BF16), normalised to the box; only columns
@@ -392,20 +610,24 @@ __global__ void mlp_input_kernel(const float* __restrict__ theta, int rows, int 
       make_uint4(pack_bf16x2(u[0], u[1]), pack_bf16x2(u[2], u[3]), pack_bf16x2(u[4], 0.f), 0u);
 }
 
-// Per-bin constants of the scan epilogue (from the standardization, the output
-// bias and the data): {m_j + s_j b_j, s_j, n_j, n_j ln n_j - n_j}; masked bins
-// and padding columns {0, 0, 0, -1} (exp(0) - 1 = 0).
+// Per-bin constants of the scan (from the standardization, the output bias and
+// the data), laid out as EpiArgs::binc says; masked bins and padding columns
+// {0, 0, 0, -1} (exp(0) - 1 = 0).
 __global__ void scan_consts_kernel(const float* __restrict__ mean, const float* __restrict__ stdv,
                                    const float* __restrict__ bias, const float2* __restrict__ nb, int n, int n_pad,
-                                   float4* __restrict__ out) {
+                                   float* __restrict__ out) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n_pad) return;
   float4 c = make_float4(0.f, 0.f, 0.f, -1.f);
   if (j < n && nb[j].x >= 0.f) {
     const float nj = nb[j].x;
-    c = make_float4(fmaf(stdv[j], bias[j], mean[j]), stdv[j], nj, nj > 0.f ? nj * logf(nj) - nj : 0.f);
+    c = make_float4(fmaf(stdv[j], bias[j], mean[j]), stdv[j], -nj, nj > 0.f ? nj * logf(nj) - nj : 0.f);
   }
-  out[j] = c;
+  float* o = out + (size_t)(j / kScanBins) * 4 * kScanBins + j % kScanBins;
+  o[0] = c.x;
+  o[kScanBins] = c.y;
+  o[2 * kScanBins] = c.z;
+  o[3 * kScanBins] = c.w;
 }
 
 // db[c] = sum_m dZ[m][c]: a block of 64 threads takes 16 columns; thread l of
@@ -784,7 +1006,7 @@ cudaError_t launch_mode(const Gemm& g, int sm_count, unsigned* status, cudaStrea
   const int tiles = (g.M / kBM) * (g.N / BN);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(tiles < sm_count ? tiles : sm_count);
-  cfg.blockDim = dim3(kGemmThreads);
+  cfg.blockDim = dim3(gemm_threads(MODE));
   cfg.dynamicSmemBytes = GemmShape<BN>::kSmem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -804,14 +1026,28 @@ cudaError_t launch_width(const Gemm& g, int sm_count, unsigned* status, cudaStre
     case kFwdOutFit: return launch_mode<BN, kFwdOutFit>(g, sm_count, status, s, dep);
     case kBwdData: return launch_mode<BN, kBwdData>(g, sm_count, status, s, dep);
     case kFwdOut: return launch_mode<BN, kFwdOut>(g, sm_count, status, s, dep);
-    case kFwdScan: return launch_mode<BN, kFwdScan>(g, sm_count, status, s, dep);
     case kFwdHiddenScan: return launch_mode<BN, kFwdHiddenScan>(g, sm_count, status, s, dep);
   }
   return cudaErrorInvalidValue;
 }
 
+// Parts that a scan's bins are cut into: the fewest that give every SM two
+// units (of 256 points), as far as the tiles of 128 bins go round.
+int scan_groups(int M, int N, int sm_count) {
+  const int tiles = N / kScanBins;
+  int groups = 1;
+  while ((long long)(M / kScanRows) * groups < 2LL * sm_count && tiles % (2 * groups) == 0) groups *= 2;
+  return groups;
+}
+
 cudaError_t run_gemm(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s, bool dep = false) {
   if (g.mode == kWgrad) return launch_mode<64, kWgrad>(g, sm_count, status, s, dep);
+  if (g.mode == kFwdScan) {
+    const int groups = scan_groups(g.M, g.N, sm_count), units = g.M / kScanRows * groups;
+    mlp_scan_kernel<<<units < sm_count ? units : sm_count, kScanThreads, kScanSmem, s>>>(g.ma, g.mb, g.M, g.N, groups,
+                                                                                        g.E, status);
+    return srw::launch_result();
+  }
   return g.bn == 256   ? launch_width<256>(g, sm_count, status, s, dep)
          : g.bn == 128 ? launch_width<128>(g, sm_count, status, s, dep)
                        : launch_width<64>(g, sm_count, status, s, dep);
@@ -823,7 +1059,6 @@ cudaError_t gemm_attrs_width() {
   if (e == cudaSuccess) e = gemm_attr<BN, kFwdOutFit>();
   if (e == cudaSuccess) e = gemm_attr<BN, kBwdData>();
   if (e == cudaSuccess) e = gemm_attr<BN, kFwdOut>();
-  if (e == cudaSuccess) e = gemm_attr<BN, kFwdScan>();
   if (e == cudaSuccess) e = gemm_attr<BN, kFwdHiddenScan>();
   return e;
 }
@@ -833,6 +1068,8 @@ cudaError_t gemm_attrs() {
   if (e == cudaSuccess) e = gemm_attrs_width<128>();
   if (e == cudaSuccess) e = gemm_attrs_width<64>();
   if (e == cudaSuccess) e = gemm_attr<64, kWgrad>();
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(mlp_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kScanSmem);
   return e;
 }
 
@@ -868,7 +1105,7 @@ struct SurrogateBatch {
   __nv_bfloat16* dy = nullptr;
   __nv_bfloat16* dz[3] = {};
   float* y = nullptr;       // FP32 network output (forward hook)
-  double* parts = nullptr;  // scan partials [2 n_out_pad / tile width][M]
+  double* parts = nullptr;  // scan partials [4 scan_groups][M]
   double* loss = nullptr;
   Gemm fwd[4], fwd_out, fwd_scan, wgrad[4], bwd[3];
   cudaGraphExec_t step = nullptr;  // captured training step (after its input kernel)
@@ -882,7 +1119,7 @@ struct srw_surrogate_ctx {
   SurrogateLayer L[4];
   float* mean = nullptr;  // per-bin standardization of log mu
   float* stdv = nullptr;
-  float4* binc = nullptr;  // per-bin constants of the scan epilogue
+  float* binc = nullptr;   // per-bin constants of the scan (four a bin)
   int stats_ready = 0;
   long long adam_t = 0;
   long long epochs_done = 0;  // completed epochs of the last (resumable) fit
@@ -1034,7 +1271,7 @@ srw_status get_batch(srw_surrogate s, int M, bool train, SurrogateBatch** out) {
   cudaError_t e = salloc(&B->x, (size_t)M * srw::kInPad);
   for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = salloc(&B->h[k], (size_t)M * H);
   const int bn_h = srw::pick_tile(M, H, s->sm_count), bn_o = srw::pick_tile(M, NO, s->sm_count);
-  if (e == cudaSuccess) e = salloc(&B->parts, (size_t)(NO / bn_o) * 2 * M);
+  if (e == cudaSuccess) e = salloc(&B->parts, (size_t)srw::scan_groups(M, NO, s->sm_count) * 4 * M);
   if (e == cudaSuccess) e = cudaMemset(B->x, 0, sizeof(__nv_bfloat16) * (size_t)M * srw::kInPad);
   if (e == cudaSuccess) e = salloc(&B->loss, 1);
   if (train) {
@@ -1069,7 +1306,7 @@ srw_status get_batch(srw_surrogate s, int M, bool train, SurrogateBatch** out) {
     E.bias = s->L[3].b;
     E.binc = s->binc;
     E.parts = B->parts;
-    e = prep(B->fwd_scan, B->h[2], s->L[3].w_bf, M, NO, H, srw::kFwdScan, bn_o, E);
+    e = prep(B->fwd_scan, B->h[2], s->L[3].w_bf, M, NO, H, srw::kFwdScan, srw::kScanBins, E);
   }
   if (train) {
     if (e == cudaSuccess) {  // fit output: targets set per call
@@ -1258,7 +1495,8 @@ srw_status loglik_device(srw_surrogate s, const float* theta, long long P, T* ou
   for (long long off = 0; off < P; off += kScanChunk) {
     const int rows = (int)std::min<long long>(kScanChunk, P - off);
     SurrogateBatch* B = nullptr;
-    srw_status r = get_batch(s, round_up(rows, srw::kBM) < 65536 ? round_up(rows, srw::kBM) : round_up(rows, 65536), false, &B);
+    const int M = round_up(rows, srw::kScanRows);
+    srw_status r = get_batch(s, M < 65536 ? M : round_up(rows, 65536), false, &B);
     if (r != SRW_OK) return r;
     cudaError_t e = forward_hidden(s, theta + off * 5, rows, B, st);
     if (e == cudaSuccess) {
@@ -1266,9 +1504,9 @@ srw_status loglik_device(srw_surrogate s, const float* theta, long long P, T* ou
       g.E.rows_valid = rows;
       e = srw::run_gemm(g, s->sm_count, s->d_status, st);
     }
-    const int g_bn = B->fwd_scan.bn;
+    const int n_parts = 4 * srw::scan_groups(B->M, s->n_out_pad, s->sm_count);
     if (e == cudaSuccess) {
-      srw::scan_reduce_kernel<T><<<(rows + 255) / 256, 256, 0, st>>>(B->parts, s->n_out_pad / g_bn * 2, rows, s->h->d_cdata,
+      srw::scan_reduce_kernel<T><<<(rows + 255) / 256, 256, 0, st>>>(B->parts, n_parts, rows, s->h->d_cdata,
                                                                    out + off);
       e = srw::launch_result();
     }
@@ -1371,7 +1609,7 @@ srw_status srw_surrogate_create(srw_handle h, const float* centre, const float* 
   if (e == cudaSuccess) e = salloc(&s->d_step, 1);
   if (e == cudaSuccess) e = salloc(&s->mean, s->n_out_pad);
   if (e == cudaSuccess) e = salloc(&s->stdv, s->n_out_pad);
-  if (e == cudaSuccess) e = salloc(&s->binc, s->n_out_pad);
+  if (e == cudaSuccess) e = salloc(&s->binc, 4 * (size_t)s->n_out_pad);
   if (e == cudaSuccess) {  // identity standardization until training sets it
     std::vector<float> z(s->n_out_pad, 0.f), o(s->n_out_pad, 1.f);
     e = cudaMemcpy(s->mean, z.data(), sizeof(float) * z.size(), cudaMemcpyHostToDevice);
