@@ -21,7 +21,7 @@
 //              and accumulates them per point (double-float), one FP64 partial
 //              per (rec tile, point).
 //   warp 12    TMA producer: streams R hi (+ lo) tiles, BK x BN, swizzled.
-//   warp 13    MMA issuer (one thread) and TMEM owner.
+//   warp 13    MMA issuer (its elected lane) and TMEM owner.
 //   warp 14    TMA producer of the coefficient-spectra slice of each K block
 //              (BK x 8 floats), up to kShatSlots blocks ahead.
 //
@@ -578,60 +578,63 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
     }
   } else {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      int g = 0;
-      bool issued_any = false;
-      int tc = -1;
-      FOR_ITEMS(idx) {
-        ++tc;
-        if (aborted(&abort_flag)) break;
-        int m0, n0, gi;
-        const TcGroup G = work_at<GROUPED, BN>(L, idx, m0, n0, gi);
-        if (GROUPED && gi < 0) break;  // stop item: this CTA's list is done
-        const int2 kr = tile_walk<GROUPED, BN>(G, n0);
-        const uint32_t idesc = idesc_f16kind(kBM, GROUPED ? G.bn : BN, F16);
-        const int buf = tc % NB;
-        if (!ptx::mbar_wait(&acc_empty[buf], ((tc / NB) & 1) ^ 1, &abort_flag)) {
+    // the whole warp walks the items in uniform control flow; its elected lane issues
+    const uint32_t leader = elect_one();
+    int g = 0;
+    bool issued_any = false;
+    int tc = -1;
+    FOR_ITEMS(idx) {
+      ++tc;
+      int m0, n0, gi;
+      const TcGroup G = work_at<GROUPED, BN>(L, idx, m0, n0, gi);
+      if (GROUPED && gi < 0) break;  // stop item: this CTA's list is done
+      const int2 kr = tile_walk<GROUPED, BN>(G, n0);
+      const uint32_t idesc = idesc_f16kind(kBM, GROUPED ? G.bn : BN, F16);
+      const int buf = tc % NB;
+      if (!warp_wait(&acc_empty[buf], ((tc / NB) & 1) ^ 1, &abort_flag)) {
+        give_up();
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + (uint32_t)(buf * S::kAccCols);
+      const bool down = kr.y < 0;  // descending walk: the MMA steps inside a block run down too
+      bool ok = true;
+      for (int kk = 0; kk < kb_count<BK>(kr); ++kk, ++g) {
+        const int st = g % ST;
+        if (!warp_wait(&r_full[st], (g / ST) & 1, &abort_flag) ||
+            !warp_wait(&w_full[st], (g / ST) & 1, &abort_flag)) {
           give_up();
+          ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(buf * S::kAccCols);
-        const bool down = kr.y < 0;  // descending walk: the MMA steps inside a block run down too
-        bool ok = true;
-        for (int kk = 0; kk < kb_count<BK>(kr); ++kk, ++g) {
-          const int st = g % ST;
-          if (!ptx::mbar_wait(&r_full[st], (g / ST) & 1, &abort_flag) ||
-              !ptx::mbar_wait(&w_full[st], (g / ST) & 1, &abort_flag)) {
-            give_up();
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t ah = ptx::smem_addr(a_hi(st)), bh = ptx::smem_addr(b_hi(st));
-          const uint32_t al = ptx::smem_addr(a_lo(st)), bl = ptx::smem_addr(b_lo(st));
+        // 16 of K inside the swizzle atom are 32 bytes, 2 in the descriptors' address field
+        const int64_t step = down ? -2 : 2;
+        const uint64_t first = down ? (uint64_t)(2 * (BK / 16 - 1)) : 0;
+        const uint64_t ah = smem_desc_k<BK>(ptx::smem_addr(a_hi(st))) + first;
+        const uint64_t bh = smem_desc_k<BK>(ptx::smem_addr(b_hi(st))) + first;
+        const uint64_t al = smem_desc_k<BK>(ptx::smem_addr(a_lo(st))) + first;
+        const uint64_t bl = smem_desc_k<BK>(ptx::smem_addr(b_lo(st))) + first;
 #pragma unroll
-          for (int q = 0; q < BK / 16; ++q) {
-            const int ks = down ? BK / 16 - 1 - q : q;
-            const uint32_t off = (uint32_t)ks * 32u;  // 16 BF16 along K inside the swizzle atom
-            const uint32_t acc = (kk != 0) || q != 0;  // the item's first update initialises
-            mma_bf16(d_tmem, smem_desc_k<BK>(ah + off), smem_desc_k<BK>(bh + off), idesc, acc);
-            if (X3) {
-              mma_bf16(d_tmem, smem_desc_k<BK>(ah + off), smem_desc_k<BK>(bl + off), idesc, 1u);
-              mma_bf16(d_tmem, smem_desc_k<BK>(al + off), smem_desc_k<BK>(bh + off), idesc, 1u);
-            }
+        for (int q = 0; q < BK / 16; ++q) {
+          const uint64_t off = (uint64_t)(step * q);
+          const uint32_t acc = (kk != 0) || q != 0;  // the item's first update initialises
+          mma_bf16_warp(d_tmem, ah + off, bh + off, idesc, acc, leader);
+          if (X3) {
+            mma_bf16_warp(d_tmem, ah + off, bl + off, idesc, 1u, leader);
+            mma_bf16_warp(d_tmem, al + off, bh + off, idesc, 1u, leader);
           }
-          issued_any = true;
-          mma_commit(&empty[st]);  // frees the stage once these MMAs have read it
         }
-        if (!ok) break;
-        mma_commit(&acc_full[buf]);  // accumulator complete
+        issued_any = true;
+        mma_commit_warp(&empty[st], leader);  // frees the stage once these MMAs have read it
       }
-      // before TMEM is released every issued MMA must have finished
-      if (issued_any) {
-        mma_commit(&drain);
-        ptx::mbar_wait(&drain, 0, nullptr, 100000000ull);
-      }
+      if (!ok) break;
+      mma_commit_warp(&acc_full[buf], leader);  // accumulator complete
+    }
+    // before TMEM is released every issued MMA must have finished
+    if (issued_any) {
+      mma_commit_warp(&drain, leader);
+      ptx::mbar_wait(&drain, 0, nullptr, 100000000ull);
     }
   }
 
