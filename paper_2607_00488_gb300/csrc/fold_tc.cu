@@ -11,19 +11,31 @@
 //              takes K chunk w); it computes W from the coefficients (seven
 //              terms: the constant monomial is always in the reference fold)
 //              and the block's coefficient spectra (streamed into a
-//              shared-memory ring, read as warp-uniform loads), splits W into
-//              hi (+ lo) halves and writes it in the 128-byte-swizzled K-major
-//              layout the tensor core reads.
+//              shared-memory ring, read as warp-uniform loads) two K at a time
+//              in packed FP32, splits W into hi (+ lo) halves and writes it in
+//              the 128-byte-swizzled K-major layout the tensor core reads.
 //   warps 8-11 epilogue: thread = point; reads its accumulator row from
 //              tensor memory (TMEM lane = point, column = rec bin), adds the
-//              background and reference fold (one float4 of constants per
-//              bin), evaluates the Poisson terms with the mask multiplied out
+//              background and reference fold, evaluates the Poisson terms of
+//              two bins at a time in packed FP32 with the mask multiplied out
 //              and accumulates them per point (double-float), one FP64 partial
 //              per (rec tile, point).
 //   warp 12    TMA producer: streams R hi (+ lo) tiles, BK x BN, swizzled.
 //   warp 13    MMA issuer (its elected lane) and TMEM owner.
 //   warp 14    TMA producer of the coefficient-spectra slice of each K block
 //              (BK x 8 floats), up to kShatSlots blocks ahead.
+//
+// What bounds it (a stage of 128 x 64 x 256 on the 65,536-point solar set,
+// cycles): the tensor core needs 12 x 128, 71 % of it with the FP16 split's
+// zeros left out; the W producers ~1300 of latencies (loads, sums,
+// conversions, stores, fence) in a two-stage ring, so their halves of K are
+// handed over separately and refilled while the other half's MMAs run; the
+// epilogue's 256 columns took 2200 a stage in scalar form (it was the longest
+// role of the FP16 split, whose items have 31 stages), about half of that in
+// pairs.  A stage takes ~1950.  Measured and not kept: sixteen producer warps
+// of two rows (the spectra loads double and the shared-memory port with them:
+// 989 us), eight epilogue warps of branchy terms (998 us), copying only the
+// nonzero rows in boxes of 64 (1024 us).
 //
 // The fold is taken of W(theta) - W_ref (the reference point's FP64 fold
 // R W_ref enters the epilogue with the background), so the BF16 rounding
@@ -39,7 +51,14 @@
 //
 // Each rec tile runs only the range of K blocks in which its split response
 // has nonzero elements (kbr, from create time); the skipped blocks hold
-// zeros in both halves, so their products are exact zeros.
+// zeros in both halves, so their products are exact zeros.  Inside the range
+// the response is still mostly a band: per block the rows with nonzero hi and
+// with nonzero lo elements are known (kbn, in 16 rows) and the MMAs cover only
+// those columns of the accumulator; a block without lo elements skips that
+// half's copy.  What is left out adds exact zeros, so the result is the
+// same bit for bit.  On the solar set 71 % of the executed blocks' columns
+// remain with the FP16 split (its lo half ends 15 sigma before the hi half on
+// the low tail) and 92 % with the BF16 split.
 //
 // Grouped launches (several detector configurations with their own binning,
 // response, data and points in one persistent grid) use the same kernel: each
@@ -56,6 +75,7 @@
 #include <vector>
 
 #include "dfloat.cuh"
+#include "f32x2.cuh"
 #include "poisson.cuh"
 #include "ptx.cuh"
 #include "srw_internal.h"
@@ -115,13 +135,8 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
     hi = pack_bf16x2(a, b);
     h2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hi));
   }
-  uint64_t r;
-  asm("sub.rn.f32x2 %0, %1, %2;"
-      : "=l"(r)
-      : "l"((uint64_t)__float_as_uint(a) | ((uint64_t)__float_as_uint(b) << 32)),
-        "l"((uint64_t)__float_as_uint(h2.x) | ((uint64_t)__float_as_uint(h2.y) << 32)));
-  const float ra = __uint_as_float((uint32_t)r), rb = __uint_as_float((uint32_t)(r >> 32));
-  lo = F16 ? pack_f16x2(ra, rb) : pack_bf16x2(ra, rb);
+  const float2 r = unpk(sub2(pk(a, b), pk(h2.x, h2.y)));
+  lo = F16 ? pack_f16x2(r.x, r.y) : pack_bf16x2(r.x, r.y);
 }
 
 // Power of two s with s * bound in [2^13, 2^14): the FP16 scale of values
@@ -177,6 +192,16 @@ __device__ __forceinline__ int kb_at(int2 kr, int kk) {
   return kr.y >= 0 ? R * kr.x + kk : R * kr.x + (R - 1) - kk;
 }
 
+// Rows of a block (rec tile x 64 true bins) that hold nonzero elements, in
+// units of 16: hi in [h0, h1), lo in [l0, l1), one byte each.
+struct BlockRows {
+  uint32_t v;
+  __device__ __forceinline__ int h0() const { return (int)(v & 255u); }
+  __device__ __forceinline__ int h1() const { return (int)((v >> 8) & 255u); }
+  __device__ __forceinline__ int l0() const { return (int)((v >> 16) & 255u); }
+  __device__ __forceinline__ int l1() const { return (int)(v >> 24); }
+};
+
 constexpr int kMaxGroups = 4096;  // configurations of one grouped launch
 constexpr int kPrefetch = 2;      // R blocks prefetched into L2 this many stages ahead
 constexpr double kL2ResidentBytes = 64.0 * 1024 * 1024;  // responses up to this size stay in L2 (129 MB)
@@ -216,6 +241,32 @@ struct TcLaunch {
 // therefore stores CTA b's k-th item at slot k * gridDim.x + b, and each list
 // ends with a stop item (group < 0).
 #define FOR_ITEMS(idx) for (int idx = (int)blockIdx.x; idx < L.n_items; idx += (int)gridDim.x)
+
+// Poisson terms of two bins from their accumulators (poisson_term_f32_dm, in
+// packed FP32 where the two are alike): mu - n = acc / (s_p r_j) + (b + R W_ref
+// - n), the power-of-two scales of both operands coming out exactly.  ts
+// collects the terms in the order of the bins, mneg and least the smallest
+// active mu and the smallest |mu|.
+template <bool F16>
+__device__ __forceinline__ void epilogue_pair(uint64_t v, float sinv, uint64_t n, uint64_t y, uint64_t z, uint64_t w,
+                                              float& ts, float& mneg, float& least) {
+  const uint64_t dm = F16 ? fma2(v, mul2(pk(sinv, sinv), w), y) : add2(v, y);
+  const uint64_t mu = add2(n, dm), s = add2(n, mu);
+  const float2 mu1 = unpk(mu), s1 = unpk(s), n1 = unpk(n), z1 = unpk(z);
+  // u = (mu - n) / (mu + n) = -v of poisson_term_f32_dm; rounding is symmetric
+  const uint64_t u = mul2(dm, pk(reciprocal(s1.x), reciprocal(s1.y))), u2 = mul2(u, u);
+  uint64_t p = fma2(u2, pk(1.f / 9.f, 1.f / 9.f), pk(1.f / 7.f, 1.f / 7.f));
+  p = fma2(u2, p, pk(1.f / 5.f, 1.f / 5.f));
+  p = fma2(u2, p, pk(1.f / 3.f, 1.f / 3.f));
+  const float2 a = unpk(fma2(dm, u, mul2(mul2(mul2(mul2(n, pk(-2.f, -2.f)), u), u2), p)));
+  const float l0 = logf(fmaxf(quotient(n1.x, mu1.x), 1e-30f)), l1 = logf(fmaxf(quotient(n1.y, mu1.y), 1e-30f));
+  const float2 b = unpk(fma2(n, pk(l0, l1), sub2(mu, n)));
+  const float2 v1 = unpk(u), m = unpk(mul2(mu, z));
+  ts = fmaf(fabsf(v1.x) < 0.1f ? a.x : b.x, z1.x, ts);
+  ts = fmaf(fabsf(v1.y) < 0.1f ? a.y : b.y, z1.y, ts);
+  mneg = fminf(mneg, fminf(m.x, m.y));
+  least = fminf(least, fminf(fabsf(mu1.x), fabsf(mu1.y)));
+}
 
 // Configuration (by value) and tile origin of work item idx (gi < 0: a stop
 // item of a grouped launch).  A single-
@@ -265,11 +316,12 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
   // (a round trip through an integer makes them generic loads: slower, and on
   // the long scoreboard)
   unsigned char* smem = dsmem_raw + ((1024u - (ptx::smem_addr(dsmem_raw) & 1023u)) & 1023u);
-  __shared__ __align__(8) uint64_t r_full[ST], w_full[ST], empty[ST], acc_full[NB], acc_empty[NB], drain;
+  __shared__ __align__(8) uint64_t r_full[ST], w_full[ST][2], a_empty[ST][2], b_empty[ST], acc_full[NB], acc_empty[NB], drain;
   __shared__ __align__(8) uint64_t s_full[kShatSlots], s_empty[kShatSlots], never;
   __shared__ uint32_t tmem_slot;
   __shared__ unsigned abort_flag;
   __shared__ uint32_t map_fenced[GROUPED ? kMaxGroups / 32 : 1];  // maps already acquired by the R producer
+  __shared__ uint32_t rows_of[ST];  // nonzero rows of each stage's block (see BlockRows)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned* status = L.status;
@@ -289,8 +341,11 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
   if (threadIdx.x == 0) {
     for (int s = 0; s < ST; ++s) {
       ptx::mbar_init(&r_full[s], 1);
-      ptx::mbar_init(&w_full[s], kWWarps / KS::kGroups);
-      ptx::mbar_init(&empty[s], 1);
+      for (int f = 0; f < 2; ++f) {
+        ptx::mbar_init(&w_full[s][f], kWWarps / KS::kGroups / 2);
+        ptx::mbar_init(&a_empty[s][f], 1);
+      }
+      ptx::mbar_init(&b_empty[s], 1);
     }
     for (int b = 0; b < NB; ++b) {
       ptx::mbar_init(&acc_full[b], 1);
@@ -325,6 +380,7 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
     const int rg = lane;
     const int ch = warp % KS::kChunks;  // 16-byte chunk = 8 consecutive k
     const int wg = warp / KS::kChunks;
+    const int fh = 2 * ch / KS::kChunks;  // half of the stage's K
     int g = 0;            // global K-block counter (stage ring position)
     FOR_ITEMS(idx) {
       if (__any_sync(0xffffffffu, aborted(&abort_flag))) break;
@@ -335,7 +391,7 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
       const int2 kr = tile_walk<GROUPED, BN>(G, n0);
       // the coefficients of this thread's four points, computed once per point
       // by the pre-pass (not once per W warp and item)
-      float c[4][kNB - 1];
+      uint64_t c[4][kNB - 1];  // each twice, for the packed products
 #pragma unroll
       for (int rr = 0; rr < 4; ++rr) {
         const int p = m0 + rg + 32 * rr;
@@ -344,8 +400,8 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
           a = __ldg(L.coef + 2 * ((size_t)G.p_off + p));
           b = __ldg(L.coef + 2 * ((size_t)G.p_off + p) + 1);
         }
-        c[rr][0] = a.x; c[rr][1] = a.y; c[rr][2] = a.z; c[rr][3] = a.w;
-        c[rr][4] = b.x; c[rr][5] = b.y; c[rr][6] = b.z;
+        c[rr][0] = pk(a.x, a.x); c[rr][1] = pk(a.y, a.y); c[rr][2] = pk(a.z, a.z); c[rr][3] = pk(a.w, a.w);
+        c[rr][4] = pk(b.x, b.x); c[rr][5] = pk(b.y, b.y); c[rr][6] = pk(b.z, b.z);
       }
       bool ok = true;
       for (int kk = 0; kk < kb_count<BK>(kr); ++kk, ++g) {
@@ -353,34 +409,26 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
         const int st = g % ST, sl = g % kShatSlots;
         // the A buffers of this stage are free once the MMAs of its previous
         // use have completed; the coefficient spectra come through their own ring
-        if (!warp_wait(&empty[st], ((g / ST) & 1) ^ 1, &abort_flag) ||
+        if (!warp_wait(&a_empty[st][fh], ((g / ST) & 1) ^ 1, &abort_flag) ||
             !warp_wait(&s_full[sl], (g / kShatSlots) & 1, &abort_flag)) {
           give_up();
           ok = false;
           break;
         }
-        const float4* sh = shat_s(sl) + ch * 16;  // 8 k x 8 floats
+        const ulonglong2* sh = reinterpret_cast<const ulonglong2*>(shat_s(sl)) + ch * 16;  // 4 pairs of k x 8 spectra
         uint32_t h[4][4], l[4][4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          float w[4][2];
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float4 s0 = sh[(q * 2 + e) * 2], s1 = sh[(q * 2 + e) * 2 + 1];
-            const float sv[kNB] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-#pragma unroll
-            for (int rr = 0; rr < 4; ++rr) {
-              float a = c[rr][0] * sv[0];
-#pragma unroll
-              for (int bb = 1; bb < kNB; ++bb)  // the constant monomial (6) is always in the reference fold
-                if (bb != 6) a = fmaf(c[rr][bb < 6 ? bb : 6], sv[bb], a);
-              w[rr][e] = a;
-            }
-          }
+          const ulonglong2 s01 = sh[4 * q], s23 = sh[4 * q + 1], s45 = sh[4 * q + 2], s6 = sh[4 * q + 3];
+          const uint64_t sv[kNB - 1] = {s01.x, s01.y, s23.x, s23.y, s45.x, s45.y, s6.x};
 #pragma unroll
           for (int rr = 0; rr < 4; ++rr) {
-            if (X3) split2<F16>(w[rr][0], w[rr][1], h[rr][q], l[rr][q]);
-            else h[rr][q] = pack_bf16x2(w[rr][0], w[rr][1]);
+            uint64_t a = mul2(c[rr][0], sv[0]);
+#pragma unroll
+            for (int bb = 1; bb < kNB - 1; ++bb) a = fma2(c[rr][bb], sv[bb], a);
+            const float2 w = unpk(a);
+            if (X3) split2<F16>(w.x, w.y, h[rr][q], l[rr][q]);
+            else h[rr][q] = pack_bf16x2(w.x, w.y);
           }
         }
         // the four rows share the swizzle phase (rows 32 apart)
@@ -395,7 +443,7 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
         ptx::fence_proxy_async_smem();  // generic-proxy writes -> visible to the tensor core
         __syncwarp();
         if (lane == 0) {
-          ptx::mbar_arrive(&w_full[st]);
+          ptx::mbar_arrive(&w_full[st][fh]);
           ptx::mbar_arrive(&s_empty[sl]);
         }
       }
@@ -441,52 +489,52 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
       float mneg = 0.f;       // smallest mu of the active bins (below 0: outside the domain)
 #pragma unroll 1
       for (int c0 = 0; c0 < bn; c0 += 16) {
-        // per-column constants first (warp-uniform loads), then the accumulator row
-        float4 dj[16];
-        if (parts != nullptr) {
-#pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const int j = n0 + c0 + k;
-            // {n_j (0 where masked), b_j + R W_ref - n_j, mask, 1/r_j}; padding columns add nothing
-            dj[k] = j < n_rec ? __ldg(G.nb4 + j) : make_float4(0.f, 1.f, 0.f, 0.f);
-          }
-        } else {  // folded spectra only (no data needed): the row scales and the reference fold
-#pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const int j = n0 + c0 + k;
-            dj[k] = j < n_rec ? make_float4(0.f, 0.f, __ldg(G.muref + j), F16 ? __ldg(G.rinv + j) : 0.f)
-                              : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-        }
         float v[16];
         tmem_ld16(tbase + (uint32_t)c0, v);
-        if (musig_out != nullptr && p < P) {  // batched folded spectra (row p)
-          float* row = musig_out + (size_t)(G.p_off + p) * n_rec + n0 + c0;
-          // scaled, rounded, then the reference fold added
+        if (parts == nullptr) {
+          // folded spectra (row p, no data needed): scaled, rounded, then the reference fold added
+          if (p < P) {
+            float* row = musig_out + (size_t)(G.p_off + p) * n_rec + n0 + c0;
 #pragma unroll
-          for (int k = 0; k < 16; ++k) v[k] = __fadd_rn(F16 ? __fmul_rn(v[k], sinv * dj[k].w) : v[k], dj[k].z);
-          if ((n_rec & 3) == 0 && n0 + c0 + 16 <= n_rec && (reinterpret_cast<uint64_t>(musig_out) & 15u) == 0) {
+            for (int k = 0; k < 16; ++k) {
+              const int j = n0 + c0 + k;
+              const float ref = j < n_rec ? __ldg(G.muref + j) : 0.f;
+              const float w = F16 && j < n_rec ? __ldg(G.rinv + j) : 0.f;
+              v[k] = __fadd_rn(F16 ? __fmul_rn(v[k], sinv * w) : v[k], ref);
+            }
+            if ((n_rec & 3) == 0 && n0 + c0 + 16 <= n_rec && (reinterpret_cast<uint64_t>(musig_out) & 15u) == 0) {
 #pragma unroll
-            for (int k = 0; k < 16; k += 4)  // rows of 16-byte multiples: a thread's 64 bytes in four stores
-              *reinterpret_cast<float4*>(row + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
-          } else {
+              for (int k = 0; k < 16; k += 4)  // rows of 16-byte multiples: a thread's 64 bytes in four stores
+                *reinterpret_cast<float4*>(row + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+            } else {
 #pragma unroll
-            for (int k = 0; k < 16; ++k)
-              if (n0 + c0 + k < n_rec) row[k] = v[k];
+              for (int k = 0; k < 16; ++k)
+                if (n0 + c0 + k < n_rec) row[k] = v[k];
+            }
           }
+          continue;
         }
-        if (parts != nullptr) {
-          float ts = 0.f;
+        // the 16 columns' constants, rows of n, b + R W_ref - n, mask and 1/r (warp-uniform loads), in pairs
+        const ulonglong2* cp = reinterpret_cast<const ulonglong2*>(G.nb4 + n0 + c0);
+        float ts = 0.f, least = 1.f;
+#pragma unroll
+        for (int k = 0; k < 16; k += 4) {
+          const ulonglong2 cn = __ldg(cp + k / 4), cy = __ldg(cp + 4 + k / 4), cz = __ldg(cp + 8 + k / 4);
+          const ulonglong2 cw = F16 ? __ldg(cp + 12 + k / 4) : make_ulonglong2(0ull, 0ull);
+          epilogue_pair<F16>(pk(v[k], v[k + 1]), sinv, cn.x, cy.x, cz.x, cw.x, ts, mneg, least);
+          epilogue_pair<F16>(pk(v[k + 2], v[k + 3]), sinv, cn.y, cy.y, cz.y, cw.y, ts, mneg, least);
+        }
+        if (least < 1e-30f) {  // quotients by a subnormal mu need the scaled division
+          const float* cf = reinterpret_cast<const float*>(cp);
+          ts = 0.f;
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
-            // mu - n (the power-of-two scales of both operands come out exactly)
-            const float dm = F16 ? fmaf(v[k], sinv * dj[k].w, dj[k].y) : v[k] + dj[k].y;
-            ts = fmaf(poisson_term_f32_dm(dm, dj[k].x), dj[k].z, ts);
-            mneg = fminf(mneg, (dj[k].x + dm) * dj[k].z);
+            const float n = cf[k], dm = F16 ? fmaf(v[k], sinv * cf[48 + k], cf[16 + k]) : v[k] + cf[16 + k];
+            ts = fmaf(poisson_term_f32_dm(dm, n), cf[32 + k], ts);
           }
-          if (isinf(ts) || isnan(ts)) infinite = true;
-          else acc = df_add(acc, ts);
         }
+        if (isinf(ts) || isnan(ts)) infinite = true;
+        else acc = df_add(acc, ts);
       }
       if (mneg < 0.f) infinite = true;
       tc_fence_before();
@@ -507,7 +555,6 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
         const TcGroup G = work_at<GROUPED, BN>(L, idx, m0, n0, gi);
         if (GROUPED && gi < 0) break;  // stop item: this CTA's list is done
         const int2 kr = tile_walk<GROUPED, BN>(G, n0);
-        const uint32_t bytes = (uint32_t)((X3 ? 2 : 1) * (GROUPED ? G.bn : BN) * BK * 2);
         const CUtensorMap* mh = &map_hi;
         const CUtensorMap* ml = &map_lo;
         if (GROUPED) {
@@ -519,22 +566,34 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
             map_fenced[gi >> 5] |= 1u << (gi & 31);
           }
         }
-        for (int kk = 0; kk < kb_count<BK>(kr); ++kk, ++g) {
+        const int bn = GROUPED ? G.bn : BN, cnt = kb_count<BK>(kr);
+        const uint32_t* kbn = G.kbn + (size_t)(n0 / bn) * (G.k_pad / kBK);
+        BlockRows next{__ldg(kbn + kb_at<BK>(kr, 0) / KS::kPerBlock)};
+        for (int kk = 0; kk < cnt; ++kk, ++g) {
           const int kb = kb_at<BK>(kr, kk);
           const int st = g % ST;
-          if (!ptx::mbar_wait(&empty[st], ((g / ST) & 1) ^ 1, &abort_flag)) {
+          BlockRows cur = next;
+          if (kk + 1 < cnt) next = BlockRows{__ldg(kbn + kb_at<BK>(kr, kk + 1) / KS::kPerBlock)};
+          if (kk == 0) cur.v = (cur.v & 0xffff0000u) | ((uint32_t)(bn / 16) << 8);  // initialises every column
+          if (!ptx::mbar_wait(&b_empty[st], ((g / ST) & 1) ^ 1, &abort_flag)) {
             give_up();
             ok = false;
             break;
           }
-          SRW_CHECK(status, kb >= 0 && kb < G.k_pad / BK && n0 >= 0 && n0 < G.n_tiles * (GROUPED ? G.bn : BN));
-          ptx::mbar_arrive_expect_tx(&r_full[st], bytes);
+          SRW_CHECK(status, kb >= 0 && kb < G.k_pad / BK && n0 >= 0 && n0 < G.n_tiles * bn && cur.h1() * 16 <= bn &&
+                                cur.l1() * 16 <= bn);
+          rows_of[st] = cur.v;
+          // a block without nonzero lo elements needs no lo half.  (Copying only
+          // the nonzero rows, in boxes of 64, was slower: 947 -> 1024 us for the
+          // 65,536-point scan, with eight copies a stage instead of two.)
+          const bool lo = X3 && cur.l1() > 0;
+          ptx::mbar_arrive_expect_tx(&r_full[st], (uint32_t)((lo ? 2 : 1) * bn * BK * 2));
           tma_load_2d(b_hi(st), mh, kb * BK, n0, &r_full[st]);
-          if (X3) tma_load_2d(b_lo(st), ml, kb * BK, n0, &r_full[st]);
+          if (lo) tma_load_2d(b_lo(st), ml, kb * BK, n0, &r_full[st]);
           // warm L2 with the block kPrefetch stages ahead: with a two-stage ring
           // a response that does not stay in L2 (many configurations, or one
           // large one) would otherwise expose the HBM latency at every stage
-          if (L.prefetch && kk + kPrefetch < kb_count<BK>(kr)) {
+          if (L.prefetch && kk + kPrefetch < cnt) {
             const int kbp = kb_at<BK>(kr, kk + kPrefetch);
             tma_prefetch_2d(mh, kbp * BK, n0);
             if (X3) tma_prefetch_2d(ml, kbp * BK, n0);
@@ -589,7 +648,7 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
       const TcGroup G = work_at<GROUPED, BN>(L, idx, m0, n0, gi);
       if (GROUPED && gi < 0) break;  // stop item: this CTA's list is done
       const int2 kr = tile_walk<GROUPED, BN>(G, n0);
-      const uint32_t idesc = idesc_f16kind(kBM, GROUPED ? G.bn : BN, F16);
+      const uint32_t idesc = idesc_f16kind(kBM, 0, F16);  // the columns are the block's
       const int buf = tc % NB;
       if (!warp_wait(&acc_empty[buf], ((tc / NB) & 1) ^ 1, &abort_flag)) {
         give_up();
@@ -601,32 +660,50 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
       bool ok = true;
       for (int kk = 0; kk < kb_count<BK>(kr); ++kk, ++g) {
         const int st = g % ST;
-        if (!warp_wait(&r_full[st], (g / ST) & 1, &abort_flag) ||
-            !warp_wait(&w_full[st], (g / ST) & 1, &abort_flag)) {
+        if (!warp_wait(&r_full[st], (g / ST) & 1, &abort_flag)) {
           give_up();
           ok = false;
           break;
         }
-        tc_fence_after();
-        // 16 of K inside the swizzle atom are 32 bytes, 2 in the descriptors' address field
-        const int64_t step = down ? -2 : 2;
-        const uint64_t first = down ? (uint64_t)(2 * (BK / 16 - 1)) : 0;
-        const uint64_t ah = smem_desc_k<BK>(ptx::smem_addr(a_hi(st))) + first;
-        const uint64_t bh = smem_desc_k<BK>(ptx::smem_addr(b_hi(st))) + first;
-        const uint64_t al = smem_desc_k<BK>(ptx::smem_addr(a_lo(st))) + first;
-        const uint64_t bl = smem_desc_k<BK>(ptx::smem_addr(b_lo(st))) + first;
+        // the block's nonzero rows, left by the R producer with the copies
+        const BlockRows rows{__shfl_sync(0xffffffffu, rows_of[st], 0)};
+        const int h0 = rows.h0(), nh = rows.h1() - h0, l0 = rows.l0(), nl = rows.l1() - l0;
+        const uint32_t id_h = idesc + ((uint32_t)nh << 18), id_l = idesc + ((uint32_t)nl << 18);  // N / 8 at bit 17
+        const uint32_t d_h = d_tmem + (uint32_t)(16 * h0), d_l = d_tmem + (uint32_t)(16 * l0);
+        // 16 of K inside the swizzle atom are 32 bytes, 2 in the descriptors' address field; 16 rows 32 BK bytes
+        const uint64_t ah = smem_desc_k<BK>(ptx::smem_addr(a_hi(st)));
+        const uint64_t bh = smem_desc_k<BK>(ptx::smem_addr(b_hi(st))) + (uint64_t)(2 * BK * h0);
+        const uint64_t al = smem_desc_k<BK>(ptx::smem_addr(a_lo(st)));
+        const uint64_t bl = smem_desc_k<BK>(ptx::smem_addr(b_lo(st))) + (uint64_t)(2 * BK * l0);
+        // the W tile comes and goes in halves of its K: with two stages in
+        // shared memory the producers of a half refill it while the MMAs of the
+        // other one run, instead of waiting for the whole stage's
 #pragma unroll
-        for (int q = 0; q < BK / 16; ++q) {
-          const uint64_t off = (uint64_t)(step * q);
-          const uint32_t acc = (kk != 0) || q != 0;  // the item's first update initialises
-          mma_bf16_warp(d_tmem, ah + off, bh + off, idesc, acc, leader);
-          if (X3) {
-            mma_bf16_warp(d_tmem, ah + off, bl + off, idesc, 1u, leader);
-            mma_bf16_warp(d_tmem, al + off, bh + off, idesc, 1u, leader);
+        for (int q2 = 0; q2 < 2; ++q2) {
+          const int f = down ? 1 - q2 : q2;
+          if (!warp_wait(&w_full[st][f], (g / ST) & 1, &abort_flag)) {
+            give_up();
+            ok = false;
+            break;
           }
+          tc_fence_after();
+          if (nh > 0) {
+#pragma unroll
+            for (int q = 0; q < BK / 32; ++q) {
+              const uint64_t off = 2ull * (uint32_t)(f * (BK / 32) + (down ? BK / 32 - 1 - q : q));
+              const uint32_t acc = (kk != 0) || q2 != 0 || q != 0;  // the item's first update initialises
+              mma_bf16_warp(d_h, ah + off, bh + off, id_h, acc, leader);
+              if (X3) {
+                if (nl > 0) mma_bf16_warp(d_l, ah + off, bl + off, id_l, 1u, leader);
+                mma_bf16_warp(d_h, al + off, bh + off, id_h, 1u, leader);
+              }
+            }
+          }
+          issued_any = true;
+          mma_commit_warp(&a_empty[st][f], leader);  // frees the half once these MMAs have read it
         }
-        issued_any = true;
-        mma_commit_warp(&empty[st], leader);  // frees the stage once these MMAs have read it
+        if (!ok) break;
+        mma_commit_warp(&b_empty[st], leader);
       }
       if (!ok) break;
       mma_commit_warp(&acc_full[buf], leader);  // accumulator complete
@@ -644,8 +721,7 @@ fold_tc_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
   if (warp == kMmaWarp) tmem_dealloc(tmem_base, S::kTmemCols);
 }
 
-// R (FP32, n_rec x ld) -> BF16 hi + lo (rec_pad x k_pad, zero padding); and
-// shat (FP32 [8][k_pad]) -> k-major [k_pad][8] for the W producers.
+// R (FP32, n_rec x ld) -> BF16 hi + lo (rec_pad x k_pad, zero padding); .
 __global__ void split_r_kernel(const float* __restrict__ R, int n_rec, int ld, int rec_pad, int k_pad,
                                __nv_bfloat16* __restrict__ rhi, __nv_bfloat16* __restrict__ rlo) {
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -718,31 +794,46 @@ __global__ void group_coef_kernel(const TcGroup* __restrict__ groups, const floa
     point_coef(theta + ((size_t)G.p_off + p) * 5, G, f16 != 0, out + 2 * ((size_t)G.p_off + p));
 }
 
+// shat (FP32 [8][k_pad]) -> pairs of true bins for the packed products:
+// [k / 2][spectrum 0-5, 7, pad][k % 2].
 __global__ void shat_k8_kernel(const float* __restrict__ shat, int k_pad, float* __restrict__ out) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= k_pad) return;
 #pragma unroll
-  for (int b = 0; b < kNB; ++b) out[(size_t)k * kNB + b] = shat[(size_t)b * k_pad + k];
+  for (int b = 0; b < kNB; ++b)
+    out[(size_t)(k / 2) * 2 * kNB + 2 * b + (k & 1)] =
+        b == kNB - 1 ? 0.f : shat[(size_t)(b < 6 ? b : 7) * k_pad + k];
 }
 
-// Nonzero flags of the (rec tile, K block) pairs of one split: block (kb, t)
-// reads the bn x 64 elements of hi and lo in 16-byte pieces (+-0 counts as
-// zero: it adds nothing).  The host turns the flags into each tile's range.
-__global__ void kb_flags_kernel(const uint4* __restrict__ hi, const uint4* __restrict__ lo, int n_rec, int k_pad,
-                                int bn, unsigned char* __restrict__ flags) {
+// Nonzero rows of the (rec tile, K block) pairs of one split (BlockRows, 0
+// where none): block (kb, t) reads the bn x 64 elements of hi and lo in
+// 16-byte pieces (+-0 counts as zero: it adds nothing), one bit per 16 rows.
+// The host takes each tile's range of K blocks from them.
+__global__ void kb_rows_kernel(const uint4* __restrict__ hi, const uint4* __restrict__ lo, int n_rec, int k_pad,
+                               int bn, uint32_t* __restrict__ rows) {
+  __shared__ uint32_t bits[2];
   const int kb = blockIdx.x, t = blockIdx.y;
   const int pieces = k_pad / 8;  // 16-byte pieces per row
-  bool nz = false;
+  if (threadIdx.x < 2) bits[threadIdx.x] = 0u;
+  __syncthreads();
   for (int q = threadIdx.x; q < bn * (kBK / 8); q += blockDim.x) {
-    const int r = t * bn + q / (kBK / 8);
+    const int rl = q / (kBK / 8), r = t * bn + rl;
     if (r < n_rec) {
       const size_t i = (size_t)r * pieces + (size_t)kb * (kBK / 8) + (q % (kBK / 8));
       const uint4 a = hi[i], b = lo[i];
-      nz |= ((a.x | a.y | a.z | a.w | b.x | b.y | b.z | b.w) & 0x7fff7fffu) != 0u;
+      if ((a.x | a.y | a.z | a.w) & 0x7fff7fffu) atomicOr(&bits[0], 1u << (rl / 16));
+      if ((b.x | b.y | b.z | b.w) & 0x7fff7fffu) atomicOr(&bits[1], 1u << (rl / 16));
     }
   }
-  nz = __syncthreads_or(nz);
-  if (threadIdx.x == 0) flags[(size_t)t * gridDim.x + kb] = nz ? 1 : 0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    // a product needs hi rows (of either operand order) wherever lo has one
+    const uint32_t h = bits[0] | bits[1], l = bits[1];
+    uint32_t v = 0u;
+    if (h) v |= (uint32_t)(__ffs((int)h) - 1) | (uint32_t)(32 - __clz((int)h)) << 8;
+    if (l) v |= (uint32_t)(__ffs((int)l) - 1) << 16 | (uint32_t)(32 - __clz((int)l)) << 24;
+    rows[(size_t)t * gridDim.x + kb] = v;
+  }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -866,15 +957,15 @@ cudaError_t tc_prepare(srw_ctx* h) {
   TcMaps* maps = new (std::nothrow) TcMaps();
   if (!maps) return cudaErrorMemoryAllocation;
   for (int ki = 0; ki < 2; ++ki)
-  for (int bi = 0; bi < 2; ++bi) {
-    const int bk = ki ? 32 : 64;
-    cudaError_t e = tc_encode_maps(h, bi ? 256 : 128, false, &maps->hi[ki][bi], &maps->lo[ki][bi], bk);
-    if (e == cudaSuccess) e = tc_encode_maps(h, bi ? 256 : 128, true, &maps->hi16[ki][bi], &maps->lo16[ki][bi], bk);
-    if (e != cudaSuccess) {
-      delete maps;
-      return e;
+    for (int bi = 0; bi < 2; ++bi) {
+      const int bk = ki ? 32 : 64;
+      cudaError_t e = tc_encode_maps(h, bi ? 256 : 128, false, &maps->hi[ki][bi], &maps->lo[ki][bi], bk);
+      if (e == cudaSuccess) e = tc_encode_maps(h, bi ? 256 : 128, true, &maps->hi16[ki][bi], &maps->lo16[ki][bi], bk);
+      if (e != cudaSuccess) {
+        delete maps;
+        return e;
+      }
     }
-  }
   h->tmap = maps;
   return cudaSuccess;
 }
@@ -930,11 +1021,9 @@ static bool descending_is_better(const std::vector<float>& R, int ld, int n_rec,
 // The device copy holds the walk {first block, +-count} (see kb_at).
 cudaError_t tc_block_ranges(srw_ctx* h, const std::vector<float>& R, cudaStream_t s) {
   const int n_kb = h->k_pad / kBK;
-  unsigned char* d_flags = nullptr;
   const int max_tiles = (h->n_rec + 127) / 128;
-  cudaError_t e = dev_malloc(&d_flags, (size_t)max_tiles * n_kb);
-  if (e != cudaSuccess) return e;
-  std::vector<unsigned char> flags((size_t)max_tiles * n_kb);
+  cudaError_t e = cudaSuccess;
+  std::vector<uint32_t> flags((size_t)max_tiles * n_kb);
   // direction per group of 256 rows (both tile widths use it, so that every
   // output element accumulates the same updates in the same order whichever
   // width a launch uses; skipped blocks only ever add exact zeros)
@@ -944,9 +1033,13 @@ cudaError_t tc_block_ranges(srw_ctx* h, const std::vector<float>& R, cudaStream_
       const int bn = bi ? 256 : 128, n_tiles = (h->n_rec + bn - 1) / bn;
       const uint4* hi = reinterpret_cast<const uint4*>(f16 ? (const void*)h->d_rhi16 : (const void*)h->d_rhi);
       const uint4* lo = reinterpret_cast<const uint4*>(f16 ? (const void*)h->d_rlo16 : (const void*)h->d_rlo);
-      kb_flags_kernel<<<dim3(n_kb, n_tiles), 256, 0, s>>>(hi, lo, h->n_rec, h->k_pad, bn, d_flags);
+      const size_t row_bytes = sizeof(uint32_t) * (size_t)n_tiles * n_kb;
+      uint32_t*& d_rows = h->d_kbn[f16][bi];
+      if ((e = dev_malloc(&d_rows, row_bytes)) != cudaSuccess) break;
+      h->device_bytes += row_bytes;
+      kb_rows_kernel<<<dim3(n_kb, n_tiles), 256, 0, s>>>(hi, lo, h->n_rec, h->k_pad, bn, d_rows);
       if ((e = launch_result()) != cudaSuccess) break;
-      if ((e = cudaMemcpyAsync(flags.data(), d_flags, (size_t)n_tiles * n_kb, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+      if ((e = cudaMemcpyAsync(flags.data(), d_rows, row_bytes, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
           (e = cudaStreamSynchronize(s)) != cudaSuccess)
         break;
       std::vector<int2>& r = h->kbr_h[f16][bi];
@@ -972,7 +1065,6 @@ cudaError_t tc_block_ranges(srw_ctx* h, const std::vector<float>& R, cudaStream_
       h->device_bytes += sizeof(int2) * n_tiles;
       e = cudaMemcpy(h->d_kbr[f16][bi], walk.data(), sizeof(int2) * n_tiles, cudaMemcpyHostToDevice);
     }
-  cudaFree(d_flags);
   return e;
 }
 
@@ -988,6 +1080,7 @@ double tc_block_fraction(const srw_ctx* h, int bn, bool f16) {
 TcGroup tc_group_of(const srw_ctx* h, int bn, bool f16) {
   TcGroup G{};
   G.kbr = h->d_kbr[f16 ? 1 : 0][bn == 256 ? 1 : 0];
+  G.kbn = h->d_kbn[f16 ? 1 : 0][bn == 256 ? 1 : 0];
   G.map_hi = G.map_lo = nullptr;
   G.shat_k8 = reinterpret_cast<const float4*>(h->d_shat_k8);
   G.nb4 = h->d_nb4;

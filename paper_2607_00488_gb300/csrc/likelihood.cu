@@ -318,14 +318,27 @@ __global__ void data_prepare_kernel(const double* __restrict__ bkg, int n_bkg, i
   b64[j] = b;
 }
 
+// Constants of the tensor-core epilogue: per 16 bins the rows n, b + R W_ref -
+// n, mask and 1/r (16 floats each).
+__device__ __forceinline__ void store_nb4(float4* nb4, int j, float n, float y, float z, float w) {
+  float* o = reinterpret_cast<float*>(nb4) + (size_t)(j / 16) * 64 + j % 16;
+  o[0] = n;
+  o[16] = y;
+  o[32] = z;
+  o[48] = w;
+}
+
 // Per-bin constants of the batched epilogues: reference fold + background,
 // in FP64 (SIMT fold) and as floats with the count and the mask (tensor fold).
 __global__ void data_ref_kernel(const double* __restrict__ n64, const double* __restrict__ b64,
-                                const double* __restrict__ muref, const unsigned char* __restrict__ mask, int n_rec,
+                                const double* __restrict__ muref, const unsigned char* __restrict__ mask, int n_rec, int rec_pad,
                                 const float* __restrict__ rinv, double* __restrict__ bref64, float4* __restrict__ simt_c,
                                 float2* __restrict__ nb2, float4* __restrict__ nb4) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n_rec) return;
+  if (j >= n_rec) {  // padding columns of the tensor-core tiles: mu = 1, n = 0, outside the sum
+    if (nb4 && j < rec_pad) store_nb4(nb4, j, 0.f, 1.f, 0.f, 0.f);
+    return;
+  }
   const double br = b64[j] + muref[j];
   bref64[j] = br;
   const bool on = mask == nullptr || mask[j] != 0;
@@ -334,8 +347,9 @@ __global__ void data_ref_kernel(const double* __restrict__ n64, const double* __
   simt_c[2 * j + 1] = make_float4(on ? 1.f : 0.f, 0.f, 0.f, 0.f);
   nb2[j] = make_float2(on ? (float)n64[j] : -1.f, (float)br);
   // tensor-core epilogue: mu - n is formed from b + R W_ref - n, rounded once from FP64
-  if (nb4) nb4[j] = make_float4(on ? (float)n64[j] : 0.f, (float)(on ? br - n64[j] : br), on ? 1.f : 0.f,
-                                rinv ? rinv[j] : 1.f);
+  if (nb4)
+    store_nb4(nb4, j, !on || n64[j] == 0.0 ? 0.f : (float)fmax(n64[j], 1e-30), (float)(on ? br - n64[j] : br),
+              on ? 1.f : 0.f, rinv ? rinv[j] : 1.f);
 }
 
 // C = 2 sum_j M_j [n_j - n_j ln n_j + lnGamma(n_j + 1)], one block.
@@ -528,7 +542,7 @@ cudaError_t launch_set_data(srw_ctx* h, const double* d_bkg, int n_bkg, cudaStre
 
 cudaError_t launch_data_ref(srw_ctx* h, cudaStream_t s) {
   const int thr = 256;
-  data_ref_kernel<<<(h->n_rec + thr - 1) / thr, thr, 0, s>>>(h->d_n64, h->d_b64, h->d_muref64, h->d_mask, h->n_rec,
+  data_ref_kernel<<<(h->rec_pad + thr - 1) / thr, thr, 0, s>>>(h->d_n64, h->d_b64, h->d_muref64, h->d_mask, h->n_rec, h->rec_pad,
                                                              h->d_rinv, h->d_bref64, h->d_simt_c, h->d_nb2, h->d_nb4);
   cudaError_t e = launch_result();
   if (e == cudaSuccess && h->d_lin) e = launch_linear_consts(h, s);

@@ -28,6 +28,7 @@
 
 #include "dfloat.cuh"
 #include "f32x2.cuh"
+#include "poisson.cuh"
 #include "srw_internal.h"
 
 namespace srw {
@@ -109,14 +110,6 @@ __device__ __forceinline__ void deviations(const float* th, dfloat s, const Coef
     c[b] = d.hi + d.lo;
   }
   g = Couplings{gle.hi + gle.lo, gre.hi + gre.lo, glt.hi + glt.lo, grt.hi + grt.lo, th[4]};
-}
-
-// a / b where b is 0, infinite, NaN or at least 1e-30 in magnitude: the fast
-// division without its scaling of subnormal divisors.
-__device__ __forceinline__ float quotient(float a, float b) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
-  return __fmul_rn(a, r);
 }
 
 // n / mu of N points in a bin with data; the scaled division where some point

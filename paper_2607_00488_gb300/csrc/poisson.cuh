@@ -65,6 +65,15 @@ __device__ __forceinline__ dfloat poisson_term_df(dfloat mu, dfloat n) {
   return df_add(df_add(mu, dfloat{-n.hi, -n.lo}), df_mul(n, l));
 }
 
+// a / b where b is 0, infinite, NaN or at least 1e-30 in magnitude: the fast
+// division without its scaling of subnormal divisors.
+__device__ __forceinline__ float reciprocal(float b) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+  return r;
+}
+__device__ __forceinline__ float quotient(float a, float b) { return __fmul_rn(a, reciprocal(b)); }
+
 // FP32 term of the tensor-core epilogue, branch-free and without per-element
 // special cases.  With v = (n - mu)/(n + mu), ln(n/mu) = 2 atanh(v), hence
 //   t = (n - mu) v + 2 n (v^3/3 + v^5/5 + v^7/7 + v^9/9 + ...)
@@ -78,19 +87,7 @@ __device__ __forceinline__ dfloat poisson_term_df(dfloat mu, dfloat n) {
 // 0 * ln(1e-30) = 0, so t = mu (mu = 0 included, where n / mu is NaN and the
 // floor applies); mu = 0 with n > 0 gives +inf through ln(inf).  mu < 0 is
 // left to the caller (it tracks the smallest mu of the active bins).
-__device__ __forceinline__ float poisson_term_f32_tc(float mu, float n) {
-  const float d = n - mu, s = n + mu;
-  const float v = __fdividef(d, s);
-  const float v2 = v * v;
-  float p = fmaf(v2, 1.f / 9.f, 1.f / 7.f);
-  p = fmaf(v2, p, 1.f / 5.f);
-  p = fmaf(v2, p, 1.f / 3.f);
-  const float ts = fmaf(d, v, 2.f * n * v * v2 * p);
-  const float tl = fmaf(n, logf(fmaxf(__fdividef(n, mu), 1e-30f)), -d);  // mu - n = -d exactly
-  return fabsf(v) < 0.1f ? ts : tl;
-}
-
-// The same term from dm = mu - n (and n), for callers that form mu - n
+// It is formed from dm = mu - n (and n), for callers that form mu - n
 // directly: an FP32 mu of 1e5 counts carries an absolute rounding error of
 // ~6e-3, while mu - n near the data is a few hundred, so its FP32 value is
 // ~1e3 times more precise and the series branch then loses nothing to it.
@@ -98,7 +95,6 @@ __device__ __forceinline__ float poisson_term_f32_tc(float mu, float n) {
 // enters the logarithm: then mu's rounding error e enters t only as
 // (1 - n/mu) e, as in the exact expression (dt/dmu = 1 - n/mu); with the
 // unrounded dm it would enter as -(n/mu) e, about e itself.
-// Same branches, floor and special cases as poisson_term_f32_tc.
 __device__ __forceinline__ float poisson_term_f32_dm(float dm, float n) {
   const float mu = n + dm, s = n + mu;
   const float v = __fdividef(-dm, s);

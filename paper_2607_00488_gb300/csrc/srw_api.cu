@@ -134,7 +134,10 @@ static void release(srw_ctx* h) {
   dfree(h->d_node_a); dfree(h->d_node_w); dfree(h->d_node_c); dfree(h->d_node_wlo); dfree(h->d_shat_lo); dfree(h->d_shat_k8); dfree(h->d_node64); dfree(h->d_bin_count); dfree(h->d_bin_f);
   dfree(h->d_bin_l); dfree(h->d_bin64); dfree(h->d_basis); dfree(h->d_ssm64); dfree(h->d_esm64);
   for (int f = 0; f < 2; ++f)
-    for (int b = 0; b < 2; ++b) dfree(h->d_kbr[f][b]);
+    for (int b = 0; b < 2; ++b) {
+      dfree(h->d_kbr[f][b]);
+      dfree(h->d_kbn[f][b]);
+    }
   dfree(h->d_ssm32); dfree(h->d_esm32); dfree(h->d_shat); dfree(h->d_R); dfree(h->d_rhi); dfree(h->d_rlo); dfree(h->d_rhi16); dfree(h->d_rlo16); dfree(h->d_rinv); dfree(h->d_coef); dfree(h->d_linM); dfree(h->d_lin); dfree(h->d_linp);
   dfree(h->d_n64); dfree(h->d_b64); dfree(h->d_muref64); dfree(h->d_bref64); dfree(h->d_simt_c); dfree(h->d_muref32); dfree(h->d_nb2); dfree(h->d_nb4); dfree(h->d_mask); dfree(h->d_cdata);
   dfree(h->d_W); dfree(h->d_S); dfree(h->d_musig); dfree(h->d_mu); dfree(h->d_part); dfree(h->d_ticket);
@@ -841,7 +844,7 @@ srw_status srw_set_data(srw_handle h, const double* counts, const double* bkg, i
   if (!h->d_b64) SRW_CUDA(h, dalloc(h, &h->d_b64, n_rec), "alloc data");
   if (!h->d_simt_c) SRW_CUDA(h, dalloc(h, &h->d_simt_c, 2 * (size_t)n_rec), "alloc data");
   if (!h->d_nb2) SRW_CUDA(h, dalloc(h, &h->d_nb2, n_rec), "alloc data");
-  if (!h->d_nb4) SRW_CUDA(h, dalloc(h, &h->d_nb4, n_rec), "alloc data");
+  if (!h->d_nb4) SRW_CUDA(h, dalloc(h, &h->d_nb4, h->rec_pad), "alloc data");
   if (!h->d_cdata) SRW_CUDA(h, dalloc(h, &h->d_cdata, 1), "alloc data");
   if (!h->d_bref64) SRW_CUDA(h, dalloc(h, &h->d_bref64, n_rec), "alloc data");
   if (mask && !h->d_mask) SRW_CUDA(h, dalloc(h, &h->d_mask, n_rec), "alloc mask");

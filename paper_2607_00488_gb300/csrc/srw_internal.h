@@ -105,8 +105,8 @@ struct CoefRef {
 struct TcGroup {
   const CUtensorMap* map_hi;   // R hi / lo maps, box 64 K x bn rows (grouped launches; global memory)
   const CUtensorMap* map_lo;
-  const float4* shat_k8;       // [k_pad][8] coefficient spectra, k-major
-  const float4* nb4;           // [n_rec] {n_j (0 where masked), b_j + R W_ref - n_j, mask 1/0, 1/r_j (FP16 row scale)}
+  const float4* shat_k8;       // [k_pad / 2][8][2] coefficient spectra in pairs of true bins
+  const float4* nb4;           // [rec_pad / 16][4][16 floats] n_j (0 where masked), b_j + R W_ref - n_j, mask 1/0, 1/r_j (FP16 row scale)
   const double* c_data;        // data constant of -2 ln L (device scalar)
   long long parts_off;         // partial sums of the group: parts + parts_off, [n_tiles][P]
   int n_rec, k_pad, P, p_off;  // p_off: first point of the group in the launch's theta / out
@@ -116,6 +116,7 @@ struct TcGroup {
   const float* rinv;           // SRW_FP16X3: [n_rec] inverse power-of-two row scales of R
   const float* muref;          // [n_rec] R W_ref (folded spectra)
   const int2* kbr;             // [n_tiles] K-block walk {first block, +-count} over the tile's nonzero response
+  const uint32_t* kbn;         // [n_tiles][k_pad / 64] nonzero rows of each block (BlockRows in fold_tc.cu)
   float wmax[kNB];             // SRW_FP16X3: max_i |shat_b,i| (bound of the weighted-spectrum deviations)
 };
 
@@ -169,7 +170,7 @@ struct srw_ctx {
   float* d_esm32 = nullptr;
   float* d_shat = nullptr;     // [8][k_pad] FP32 pre-weighted basis (W = sum_b c_b shat_b)
   float* d_shat_lo = nullptr;  // [8][k_pad] FP32 residuals of shat
-  float* d_shat_k8 = nullptr;  // [k_pad][8] FP32 shat, k-major (tensor-core W producers)
+  float* d_shat_k8 = nullptr;  // [k_pad / 2][8][2] FP32 shat in pairs of true bins (tensor-core W producers)
   float* d_R = nullptr;        // [n_rec][ld_r]
   __nv_bfloat16* d_rhi = nullptr;  // [rec_pad][k_pad]
   __nv_bfloat16* d_rlo = nullptr;
@@ -177,6 +178,7 @@ struct srw_ctx {
   __half* d_rlo16 = nullptr;
   float* d_rinv = nullptr;         // [n_rec] inverse row scales of the FP16 split
   int2* d_kbr[2][2] = {};          // [FP16 split?][bn == 256] K-block range of each rec tile
+  uint32_t* d_kbn[2][2] = {};      // [..][..] nonzero rows of every (rec tile, K block)
   std::vector<int2> kbr_h[2][2];   // host copies (grouped scheduling, work accounting)
   float wmax[8] = {};              // max_i |shat_b,i|
   float4* d_coef = nullptr;        // [P][2] per-point W-producer coefficients and FP16 scales (batched scratch)
@@ -190,7 +192,7 @@ struct srw_ctx {
   double* d_b64 = nullptr;
   float4* d_simt_c = nullptr;  // [2 n_rec] FP32 fold epilogue: {n, n lo, b + R W_ref, lo}, {mask, 0, 0, 0}
   float2* d_nb2 = nullptr;     // {n_j or -1 where masked, b_j + R W_ref} (surrogate epilogue)
-  float4* d_nb4 = nullptr;     // {n_j (0 where masked), b_j + R W_ref - n_j, mask 1/0, 1/r_j} (tensor-core epilogue)
+  float4* d_nb4 = nullptr;     // n_j (0 where masked), b_j + R W_ref - n_j, mask 1/0, 1/r_j per 16 bins (tensor-core epilogue)
   unsigned char* d_mask = nullptr;
   double* d_cdata = nullptr;
 
