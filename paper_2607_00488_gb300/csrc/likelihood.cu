@@ -501,10 +501,11 @@ cudaError_t launch_fold_point(const srw_ctx* h, const float* W, float* musig_out
   return launch_result();
 }
 
-cudaError_t launch_fold_point_after(const srw_ctx* h, const float* W, double* out, cudaStream_t s) {
+cudaError_t launch_fold_point_after(const srw_ctx* h, const float* W, float* musig_out, float* mu_out, double* out,
+                                    cudaStream_t s, bool delta) {
   const size_t smem = gv_smem(h);
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
-  const double* muref = h->d_muref64;
+  const double* muref = delta ? h->d_muref64 : nullptr;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(fold_point_grid(h));
   cfg.blockDim = dim3(kGvThreads);
@@ -518,7 +519,7 @@ cudaError_t launch_fold_point_after(const srw_ctx* h, const float* W, double* ou
   const cudaError_t e = cudaLaunchKernelEx(&cfg, fold_point_kernel, (const float*)h->d_R, h->n_rec, h->ld_r,
                                            gv_rows_per_block(h), W, muref, (const double*)h->d_n64,
                                            (const double*)h->d_b64, (const unsigned char*)h->d_mask,
-                                           (const double*)h->d_cdata, (float*)nullptr, (float*)nullptr, h->d_part,
+                                           (const double*)h->d_cdata, musig_out, mu_out, h->d_part,
                                            h->d_ticket, out, h->d_status, inject_timeout(),
                                            (const int4*)(h->gv_blocks > 0 ? h->d_gv_seg : nullptr),
                                            (const int*)(h->gv_blocks > 0 ? h->d_gv_segs : nullptr),

@@ -19,28 +19,15 @@
 // Nodes are sorted by T_max descending, so the nodes that can reach bin i
 // are a prefix [0, bin_count[i]).
 
-#include <cooperative_groups.h>
-
 #include "dfloat.cuh"
 #include "srw_internal.h"
-
-namespace cg = cooperative_groups;
 
 namespace srw {
 namespace {
 
 constexpr int kBasisThreads = 256;
-constexpr int kSpecThreads = 256;
-constexpr int kSpecCluster = 4;   // blocks per bin group (thread-block cluster)
-constexpr int kBinsPerBlock = 8;
 
 __device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ __forceinline__ float warp_sum_f(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
@@ -111,165 +98,334 @@ basis_fp64_kernel(ModelView m, double gl_mu, double gr_mu, double kappa, double*
   }
 }
 
-// Coupling products of the reference point, hi/lo, in the order used by the
-// spectrum kernel: gLe^2 gLm^2 gLt^2 gRe^2 gRm^2 gRt^2 gLe.gRe gLm.gRm gLt.gRt kappa mu^2.
+// ---------------------------------------------------------------------------
+// G1: single-point spectrum + weights (the per-theta "physics update"), from
+// the cross-section integrals of every node at this theta.
+//
+// Nodes are sorted by T_max, so the nodes that cover bin i whole are a prefix
+// [0, full_i), and over a whole bin the integrals are polynomials in the bin's
+// edges whose coefficients depend on the node alone.  With r = 1/E and the
+// node's coupling-weighted a0 = sum w P gL^2, a1 = sum w P gR^2,
+// a2 = sum w P gL gR and a3 = w kappa mu^2,
+//   S_i = I0_i [X - p_i Y + q_i Z] + L_i V + sum of the clipped nodes,
+//   X = sum (a0 + a1 - a3 r), Y = sum r (a1 + a2 m_e r / 2), Z = sum a1 r^2, V = sum a3
+// over the prefix, with {I0, p, q, L} = {b - a, a + b, (a^2 + a b + b^2) / 3,
+// log(b / a)} of the bin (midpoint mode: {dt, 2 tc, tc^2, dt / tc}).  So one
+// scan over the nodes serves every bin: n_nodes + n_t terms instead of
+// n_nodes x n_t.  Expanding (1 - T/E)^2 cancels to about
+// (m_e / (m_e + 2E))^2 of its terms (2e-4 at the hep endpoint), which is why
+// the sums are FP64; the nodes that end inside bin i, [full_i, count_i), are
+// summed apart (a scan that starts again with every bin, in tiles of 32), so
+// that a bin without nodes stays an exact zero.
+//
+// Two kernels, the second and the fold behind it launched programmatically.
+// moments_kernel: one block of two warps per chunk of nodes writes the prefix
+// sums inside its chunk and the chunk's totals (at most kMaxChunks, chunks of 32
+// nodes up to 8192 nodes).  bins_kernel: every block scans the totals again, one
+// warp per quantity, and evaluates kBinsPerBlock bins.  Both are bound by the
+// chain of FP64 instructions of a warp (64 cycles each on an SM sub-partition,
+// dependent or not, measured), so the work is spread thin: small chunks and
+// blocks, the quantities of a chunk over two warps.
+//
+// Solar set (8003 nodes), device time per call of back-to-back calls, against a
+// kernel over all (node, bin) pairs in FP32 (clusters of four blocks per eight
+// bins): S at 4096 bins 34.8 -> 10.3 us, expected counts 49.2 -> 20.4 us; S at
+// 257 bins 10.2 -> 10.3 us.  Letting bins_kernel start at the top of
+// moments_kernel instead of at its end gave 20.5 us (S at 4096 bins), an
+// ordinary launch 12.4 us.  A line (1 node, 256 bins) takes the one-kernel form,
+// 7.5 -> 7.4 us, expected counts 13.0 -> 9.6 us; with the two kernels S took
+// 10.2 us.
+// ---------------------------------------------------------------------------
+constexpr int kMaxChunks = kSpecChunks;
+constexpr int kBinsPerBlock = 16;
+constexpr int kLanesPerBin = 8;  // clipped nodes of a bin
+constexpr int kBinThreads = kBinsPerBlock * kLanesPerBin;
+static_assert(kBinThreads == 4 * 32, "one warp per scanned quantity");
+constexpr int kTotalsPerLane = kMaxChunks / 32;
+
 struct GRef {
-  float v[2][10];
+  double v[10];
+  double gl_e, gl_mu;  // 1/2 + sin^2, -1/2 + sin^2
 };
 
-// ---------------------------------------------------------------------------
-// G1: single-point FP32 spectrum + weights (the per-theta "physics update").
-// Each block owns kBinsPerBlock consecutive recoil bins and streams the
-// contributing nodes once (coalesced float4 loads), computing the coupling-
-// weighted per-node coefficients and the closed-form bin integrals for all
-// of its bins.  Outputs (any may be null):
+// Products of the couplings (eq. g_tilde), one per thread k < 10; nu_mu is
+// unshifted.  Order: gLe^2 gLm^2 gLt^2 gRe^2 gRm^2 gRt^2 gLe.gRe gLm.gRm gLt.gRt
+// kappa mu^2; delta mode: minus those of the reference point.
+__device__ __forceinline__ void couplings(int k, const float* __restrict__ theta, double sin2w, double kappa,
+                                          const GRef& gref, int delta, double* c) {
+  if (k >= 10) return;
+  // an SM sub-partition takes 64 cycles for any FP64 instruction of a warp, so
+  // every thread picks its own two factors first and adds and multiplies once
+  const double gl_e = gref.gl_e, gl_mu = gref.gl_mu;
+  double x, y;
+  if (k == 9) {
+    x = kappa;
+    y = (double)theta[4] * (double)theta[4];
+  } else {
+    const int kx = k < 6 ? k : k - 6, ky = k < 6 ? k : k - 3;  // gLe gLm gLt gRe gRm gRt
+    const float tx = kx == 0 ? theta[0] : kx == 2 ? theta[2] : kx == 3 ? theta[1] : kx == 5 ? theta[3] : 0.f;
+    const float ty = ky == 0 ? theta[0] : ky == 2 ? theta[2] : ky == 3 ? theta[1] : ky == 5 ? theta[3] : 0.f;
+    x = (kx == 0 ? gl_e : kx < 3 ? gl_mu : sin2w) + (double)tx;
+    y = (ky == 0 ? gl_e : ky < 3 ? gl_mu : sin2w) + (double)ty;
+  }
+  x *= y;
+  if (delta) x -= gref.v[k];
+  c[k] = x;
+}
+
+// A node's tables: {w P_e, w P_mu, w P_tau, w}, {1/E, clipped I0, I1, J, MM}
+// and the bin that clips it; zeros beyond the last node.
+struct Node {
+  double w[4], q[5];
+  int k;
+};
+
+__device__ __forceinline__ Node load_node(const ModelView& m, int n, int n_end) {
+  Node d;
+  const bool in = n < n_end;
+  const size_t N = m.n_nodes;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) d.w[k] = in ? m.node64[(k + 1) * N + n] : 0.0;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) d.q[k] = in ? m.node_q[k * N + n] : 0.0;
+  d.k = in ? m.node_k[n] : -1;
+  return d;
+}
+
+// Prefix sums over the warp's 32 nodes (one per lane): X, Y, Z, V, and the
+// clipped-bin terms over the nodes that end in the same bin.
+struct Sums {
+  double x, y, z, v, q;
+};
+
+// kPart 0: X, Y and V; 1: Z and the clipped terms; 2: all of them.  Only lanes
+// below count need their sums.
+template <int kPart>
+__device__ __forceinline__ Sums scan_nodes(const Node& d, const double* c, int lane, int count = 32) {
+  Sums s = {};
+  const double r = d.q[0];
+  const double a0 = fma(d.w[0], c[0], fma(d.w[1], c[1], d.w[2] * c[2]));
+  const double a1 = fma(d.w[0], c[3], fma(d.w[1], c[4], d.w[2] * c[5]));
+  const double a2 = fma(d.w[0], c[6], fma(d.w[1], c[7], d.w[2] * c[8])) * (kMe * r * r);  // times m_e / E^2
+  const double v = d.w[3] * c[9], a1r = a1 * r;
+  if (kPart != 1) {
+    s.v = v;
+    s.x = fma(-v, r, a0 + a1);
+    s.y = fma(0.5, a2, a1r);
+  }
+  if (kPart != 0) {
+    s.z = a1r * r;
+    s.q = fma(a0, d.q[1], fma(a1, d.q[3], fma(-a2, d.q[2], v * d.q[4])));
+  }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    if (o >= count) break;
+    if (kPart != 1) {
+      const double px = __shfl_up_sync(0xffffffffu, s.x, o), py = __shfl_up_sync(0xffffffffu, s.y, o);
+      const double pv = __shfl_up_sync(0xffffffffu, s.v, o);
+      if (lane >= o) {
+        s.x += px;
+        s.y += py;
+        s.v += pv;
+      }
+    }
+    if (kPart != 0) {
+      const double pz = __shfl_up_sync(0xffffffffu, s.z, o), pq = __shfl_up_sync(0xffffffffu, s.q, o);
+      const int pk = __shfl_up_sync(0xffffffffu, d.k, o);
+      if (lane >= o) {
+        s.z += pz;
+        if (pk == d.k) s.q += pq;
+      }
+    }
+  }
+  return s;
+}
+
+// Warp 0 takes X, Y and V of the chunk, warp 1 Z and the clipped terms: half
+// the chain of FP64 instructions, on two sub-partitions.
+__global__ void __launch_bounds__(64)
+moments_kernel(ModelView m, const float* __restrict__ theta, double sin2w, double kappa, GRef gref, int delta,
+               int chunk_nodes, double* __restrict__ totals, double* __restrict__ pre, double* __restrict__ clip) {
+  __shared__ double cs[2][10];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+  double* c = cs[part];
+  const int n0 = blockIdx.x * chunk_nodes, n1 = min(m.n_nodes, n0 + chunk_nodes);
+  Node next = load_node(m, n0 + lane, n1);  // ahead of the couplings
+  couplings(lane, theta, sin2w, kappa, gref, delta, c);
+  __syncwarp();
+  double cx = 0.0, cy = 0.0, cz = 0.0, cv = 0.0;  // carry of the chunk's earlier tiles
+  for (int base = n0; base < n1; base += 32) {
+    const int n = base + lane;
+    const bool more = base + 32 < n1;
+    const Node d = next;
+    if (more) next = load_node(m, n + 32, n1);
+    if (part == 0) {
+      Sums s = scan_nodes<0>(d, c, lane);
+      if (base != n0) {
+        s.x += cx;
+        s.y += cy;
+        s.v += cv;
+      }
+      if (n < n1) {
+        pre[4 * (size_t)n] = s.x;
+        pre[4 * (size_t)n + 1] = s.y;
+        pre[4 * (size_t)n + 3] = s.v;
+      }
+      cx = more ? __shfl_sync(0xffffffffu, s.x, 31) : s.x;
+      cy = more ? __shfl_sync(0xffffffffu, s.y, 31) : s.y;
+      cv = more ? __shfl_sync(0xffffffffu, s.v, 31) : s.v;
+    } else {
+      Sums s = scan_nodes<1>(d, c, lane);
+      if (base != n0) s.z += cz;
+      if (n < n1) {
+        pre[4 * (size_t)n + 2] = s.z;
+        clip[n] = s.q;
+      }
+      cz = more ? __shfl_sync(0xffffffffu, s.z, 31) : s.z;
+    }
+  }
+  // the dependents start here, not at the top: started early, they cost more than they hide
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (lane == 31) {
+    double* t = totals + blockIdx.x;
+    if (part == 0) {
+      t[0] = cx;
+      t[kMaxChunks] = cy;
+      t[3 * kMaxChunks] = cv;
+    } else {
+      t[2 * kMaxChunks] = cz;
+    }
+  }
+}
+
+// Outputs (any may be null):
 //   S_out[i]   = S_i(theta)
 //   W_out[i]   = S_i(theta) / S_SM,i * E_SM,i   (E_SM,i where S_SM,i == 0)
 //   ssm_out[i] = S_i(theta)                     (used once at create, theta = 0)
-// ---------------------------------------------------------------------------
-__global__ void __cluster_dims__(kSpecCluster, 1, 1) __launch_bounds__(kSpecThreads)
-spectrum_point_kernel(ModelView m, const float* __restrict__ theta, dfloat sin2w, dfloat kappa, GRef gref,
-                      int delta, float* __restrict__ S_out, float* __restrict__ W_out, float* __restrict__ ssm_out) {
-  // coupling products as hi + lo float pairs: a single FP32 rounding of a
-  // coupling would bias every bin of this theta by the same relative amount
-  __shared__ float coef[2][10];
-  __shared__ float4 sbin[kBinsPerBlock];
-  __shared__ float sbl[kBinsPerBlock];
-  __shared__ float red[kSpecThreads / 32][kBinsPerBlock];
-  __shared__ float blocksum[kBinsPerBlock];
-
-  // grid: kSpecCluster blocks (one cluster) per group of kBinsPerBlock bins;
-  // the blocks of a cluster split the group's node range
-  cg::cluster_group cluster = cg::this_cluster();
-  const int crank = (int)cluster.block_rank();
-  const int first = (blockIdx.x / kSpecCluster) * kBinsPerBlock;
-  if (threadIdx.x < 10) {
-    // couplings (eq. g_tilde) in double-float arithmetic, one product per
-    // thread; nu_mu is unshifted
-    const int k = threadIdx.x;
-    const dfloat gle = df_add(df_add(dfloat{0.5f, 0.f}, sin2w), theta[0]);
-    const dfloat gre = df_add(sin2w, theta[1]);
-    const dfloat glt = df_add(df_add(dfloat{-0.5f, 0.f}, sin2w), theta[2]);
-    const dfloat grt = df_add(sin2w, theta[3]);
-    const dfloat glm = df_add(dfloat{-0.5f, 0.f}, sin2w), grm = sin2w;
-    // order: gLe^2 gLm^2 gLt^2 gRe^2 gRm^2 gRt^2 gLe.gRe gLm.gRm gLt.gRt kappa mu^2
-    const dfloat x = k == 0 ? gle : k == 1 ? glm : k == 2 ? glt : k == 3 ? gre : k == 4 ? grm : k == 5 ? grt
-                   : k == 6 ? gle : k == 7 ? glm : k == 8 ? glt : kappa;
-    const dfloat y = k == 0 ? gle : k == 1 ? glm : k == 2 ? glt : k == 3 ? gre : k == 4 ? grm : k == 5 ? grt
-                   : k == 6 ? gre : k == 7 ? grm : k == 8 ? grt : two_prod(theta[4], theta[4]);
-    const dfloat c = df_mul(x, y);
-    // delta mode: monomials of theta minus those of the reference point
-    const dfloat d = delta ? df_add(c, dfloat{-gref.v[0][k], -gref.v[1][k]}) : c;
-    coef[0][k] = d.hi;
-    coef[1][k] = d.lo;
+// kFew: at most kBinThreads nodes (a few lines): every block sums them itself,
+// one tile of 32 a warp, and there is no first kernel (n_chunks tiles of 32).
+// Otherwise totals, pre and clip are written by the grid this one waits for; they
+// are not __restrict__: a load that may be taken for constant can move above the wait.
+template <bool kFew>
+__global__ void __launch_bounds__(kBinThreads)
+bins_kernel(ModelView m, const float* theta, double sin2w, double kappa, GRef gref, int delta, int n_chunks,
+            int chunk_nodes, const double* totals, const double2* pre, const double* clip, float* S_out, float* W_out,
+            float* ssm_out) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  __shared__ double base[4][kFew ? 4 : kMaxChunks];  // sums of the chunks before this one, from its lane's first
+  __shared__ double lbase[4][kFew ? 1 : 32];         // sums of the chunks before the lane's first
+  __shared__ double sclip[kBinsPerBlock];
+  __shared__ double2 spre[kFew ? 2 * kBinThreads : 1];
+  __shared__ double sq[kFew ? kBinThreads : 1], c[kFew ? 10 : 1];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  // what does not depend on theta, ahead of the wait
+  const int first = blockIdx.x * kBinsPerBlock;
+  const int iq = first + t / kLanesPerBin, ib = first + t;
+  const int2 nq = iq < m.n_t ? m.bin_n[iq] : make_int2(0, 0);
+  int full = 0;
+  double2 b0 = {0.0, 0.0}, b1 = {0.0, 0.0};
+  float den = 0.f, esm = 0.f;
+  if (t < kBinsPerBlock && ib < m.n_t) {
+    full = m.bin_n[ib].x;
+    b0 = m.bin_q[2 * (size_t)ib];
+    b1 = m.bin_q[2 * (size_t)ib + 1];
+    if (W_out) {
+      den = m.ssm32[ib];
+      esm = m.esm32[ib];
+    }
   }
-  if (threadIdx.x < kBinsPerBlock) {
-    const int i = first + threadIdx.x;
-    sbin[threadIdx.x] = i < m.n_t ? m.bin_f[i] : make_float4(1.f, 1.f, 0.f, 0.f);
-    sbl[threadIdx.x] = i < m.n_t ? m.bin_l[i] : 0.f;
+  double2 p0 = {0.0, 0.0}, p1 = {0.0, 0.0};
+  if constexpr (kFew) {
+    const Node d = load_node(m, t, m.n_nodes);
+    couplings(t, theta, sin2w, kappa, gref, delta, c);
+    __syncthreads();
+    if (warp < n_chunks) {
+      const Sums s = scan_nodes<2>(d, c, lane, m.n_nodes - 32 * warp);
+      spre[2 * t] = make_double2(s.x, s.y);
+      spre[2 * t + 1] = make_double2(s.z, s.v);
+      sq[t] = s.q;
+    }
+    __syncthreads();
+    if (t < 4) {
+      double run = 0.0;
+      for (int k = 0; k < n_chunks; ++k) {
+        base[t][k] = run;
+        const double2 e = spre[2 * min(32 * k + 31, m.n_nodes - 1) + t / 2];  // the tile's total
+        run += t & 1 ? e.y : e.x;
+      }
+    }
+    if (full > 0) {
+      p0 = spre[2 * (full - 1)];
+      p1 = spre[2 * (full - 1) + 1];
+    }
+    clip = sq;
+  } else {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    double tot[kTotalsPerLane];
+#pragma unroll
+    for (int k = 0; k < kTotalsPerLane; ++k) {
+      const int i = lane * kTotalsPerLane + k;
+      tot[k] = i < n_chunks ? totals[warp * kMaxChunks + i] : 0.0;
+    }
+    if (full > 0) {  // t < kBinsPerBlock
+      p0 = pre[2 * (size_t)(full - 1)];
+      p1 = pre[2 * (size_t)(full - 1) + 1];
+    }
+    double run = tot[0];
+    base[warp][lane * kTotalsPerLane] = 0.0;
+#pragma unroll
+    for (int k = 1; k < kTotalsPerLane; ++k) {
+      base[warp][lane * kTotalsPerLane + k] = run;
+      run += tot[k];
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double u = __shfl_up_sync(0xffffffffu, run, o);
+      if (lane >= o) run += u;
+    }
+    run = __shfl_up_sync(0xffffffffu, run, 1);
+    lbase[warp][lane] = lane == 0 ? 0.0 : run;
   }
+  // clipped nodes [x, y) of the bin: the sums left at the last of them in each
+  // tile of 32 nodes
+  double q = 0.0;
+  if (nq.x < nq.y) {
+    for (int k = nq.x / 32 + t % kLanesPerBin; 32 * k < nq.y; k += 4 * kLanesPerBin) {
+      double e[4];  // all in flight before the first is added
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = k + u * kLanesPerBin;
+        e[u] = 32 * i < nq.y ? clip[min(nq.y, 32 * (i + 1)) - 1] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (32 * (k + u * kLanesPerBin) < nq.y) q += e[u];
+    }
+  }
+#pragma unroll
+  for (int o = kLanesPerBin / 2; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+  if (t % kLanesPerBin == 0) sclip[t / kLanesPerBin] = q;
   __syncthreads();
-
-  float ch[10], cl[10];
-#pragma unroll
-  for (int k = 0; k < 10; ++k) {
-    ch[k] = coef[0][k];
-    cl[k] = coef[1][k];
-  }
-  float acc[kBinsPerBlock];
-#pragma unroll
-  for (int bb = 0; bb < kBinsPerBlock; ++bb) acc[bb] = 0.f;
-
-  const int count = first < m.n_t ? m.bin_count[first] : 0;
-  // software pipeline: the next node's tables load while this node computes
-  constexpr int kStride = kSpecThreads * kSpecCluster;
-  const int n0 = crank * kSpecThreads + threadIdx.x;
-  float4 na_n, nw_n, nl_n;
-  if (n0 < count) {
-    na_n = m.node_a[n0];
-    nw_n = m.node_w[n0];
-    nl_n = m.node_wlo[n0];
-  }
-  for (int n = n0; n < count; n += kStride) {
-    const float4 na = na_n;  // E, 1/E, k_n, m_e/E^2
-    const float4 nw = nw_n;  // w P_e, w P_mu, w P_tau, w
-    const float4 nl = nl_n;
-    if (n + kStride < count) {
-      na_n = m.node_a[n + kStride];
-      nw_n = m.node_w[n + kStride];
-      nl_n = m.node_wlo[n + kStride];
+  if (t >= kBinsPerBlock || ib >= m.n_t) return;
+  double v = sclip[t];
+  if (full > 0) {
+    const int k = (full - 1) / chunk_nodes;
+    double X = base[0][k] + p0.x, Y = base[1][k] + p0.y, Z = base[2][k] + p1.x, V = base[3][k] + p1.y;
+    if constexpr (!kFew) {
+      const int l = k / kTotalsPerLane;
+      X += lbase[0][l];
+      Y += lbase[1][l];
+      Z += lbase[2][l];
+      V += lbase[3][l];
     }
-    const float inv_e = na.y;
-    const int kn = __float_as_int(na.z);
-    // per-node coupling-weighted coefficients, hi*hi + (hi*lo + lo*hi): the
-    // node weights and couplings enter without a shared FP32 rounding
-    const float a0 = fmaf(nw.x, ch[0], fmaf(nw.y, ch[1], nw.z * ch[2])) +
-                     (fmaf(nw.x, cl[0], fmaf(nw.y, cl[1], nw.z * cl[2])) +
-                      fmaf(nl.x, ch[0], fmaf(nl.y, ch[1], nl.z * ch[2])));
-    const float a1 = fmaf(nw.x, ch[3], fmaf(nw.y, ch[4], nw.z * ch[5])) +
-                     (fmaf(nw.x, cl[3], fmaf(nw.y, cl[4], nw.z * cl[5])) +
-                      fmaf(nl.x, ch[3], fmaf(nl.y, ch[4], nl.z * ch[5])));
-    const float a2 = (fmaf(nw.x, ch[6], fmaf(nw.y, ch[7], nw.z * ch[8])) +
-                      (fmaf(nw.x, cl[6], fmaf(nw.y, cl[7], nw.z * cl[8])) +
-                       fmaf(nl.x, ch[6], fmaf(nl.y, ch[7], nl.z * ch[8])))) * na.w;
-    const float a3 = fmaf(nw.w, ch[9], fmaf(nw.w, cl[9], nl.w * ch[9]));
-    if (m.midpoint) {
-#pragma unroll
-      for (int bb = 0; bb < kBinsPerBlock; ++bb) {
-        if (first + bb < kn) {
-          const float tc = sbin[bb].x, dt = sbin[bb].y;
-          const float y = fmaf(-tc, inv_e, 1.f);
-          acc[bb] += dt * (a0 + a1 * y * y - a2 * tc + a3 * (1.f / tc - inv_e));
-        }
-      }
-    } else {
-      float4 nc = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (kn - first < kBinsPerBlock) nc = m.node_c[n];  // this block holds the clipped bin
-#pragma unroll
-      for (int bb = 0; bb < kBinsPerBlock; ++bb) {
-        const int i = first + bb;
-        if (i < kn) {  // complete bin [a, b]
-          const float4 bf = sbin[bb];  // a, b, I0, I1
-          const float u = fmaf(-bf.x, inv_e, 1.f), v = fmaf(-bf.y, inv_e, 1.f);
-          const float j = bf.z * fmaf(u, u, fmaf(u, v, v * v)) * (1.f / 3.f);
-          acc[bb] += fmaf(a0, bf.z, fmaf(a1, j, fmaf(-a2, bf.w, a3 * fmaf(-bf.z, inv_e, sbl[bb]))));
-        } else if (i == kn) {  // bin clipped at T_max(E): integrals precomputed in FP64
-          acc[bb] += fmaf(a0, nc.x, fmaf(a1, nc.z, fmaf(-a2, nc.y, a3 * nc.w)));
-        }
-      }
-    }
+    v += fma(b0.x, fma(b1.x, Z, fma(-b0.y, Y, X)), b1.y * V);
   }
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int bb = 0; bb < kBinsPerBlock; ++bb) {
-    const float v = warp_sum_f(acc[bb]);
-    if (lane == 0) red[warp][bb] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < kBinsPerBlock) {
-    float s = 0.f;
-    for (int w = 0; w < kSpecThreads / 32; ++w) s += red[w][threadIdx.x];
-    blocksum[threadIdx.x] = s;
-  }
-  // combine the cluster's partial sums in rank order through distributed shared memory
-  cluster.sync();
-  if (crank == 0 && threadIdx.x < kBinsPerBlock) {
-    const int i = first + threadIdx.x;
-    float s = 0.f;
-    for (int c = 0; c < kSpecCluster; ++c) s += cluster.map_shared_rank(blocksum, c)[threadIdx.x];
-    if (i < m.n_t) {
-      if (S_out) S_out[i] = s;
-      if (ssm_out) ssm_out[i] = s;
-      if (W_out) {
-        // W = S/S_SM E_SM (E_SM where S_SM = 0); in delta mode S is the
-        // deviation from the reference point and so is W (0 where S_SM = 0)
-        const float den = m.ssm32[i];
-        W_out[i] = den != 0.f ? (s / den) * m.esm32[i] : (delta ? 0.f : m.esm32[i]);
-      }
-    }
-  }
-  cluster.sync();  // keep every block's shared memory alive until rank 0 has read it
+  const float s = (float)v;
+  if (S_out) S_out[ib] = s;
+  if (ssm_out) ssm_out[ib] = s;
+  // W = S/S_SM E_SM (E_SM where S_SM = 0); in delta mode S is the deviation
+  // from the reference point and so is W (0 where S_SM = 0)
+  if (W_out) W_out[ib] = den != 0.f ? (s / den) * esm : (delta ? 0.f : esm);
 }
 
 // ---------------------------------------------------------------------------
@@ -448,16 +604,36 @@ cudaError_t launch_basis_fp64(const srw_ctx* h, cudaStream_t s) {
 cudaError_t launch_spectrum_point(const srw_ctx* h, const float* theta, float* S_out, float* W_out, float* ssm_out,
                                   cudaStream_t s, bool delta) {
   const ModelView m = model_view(h);
-  const int grid = (h->n_t + kBinsPerBlock - 1) / kBinsPerBlock * kSpecCluster;
   GRef g;
-  for (int k = 0; k < 10; ++k) {
-    g.v[0][k] = h->gref[0][k];
-    g.v[1][k] = h->gref[1][k];
+  for (int k = 0; k < 10; ++k) g.v[k] = (double)h->gref[0][k] + (double)h->gref[1][k];
+  g.gl_e = 0.5 + h->sin2w;
+  g.gl_mu = -0.5 + h->sin2w;
+  const int d = delta && h->use_ref ? 1 : 0;
+  const int chunk = ((h->n_nodes - 1) / (32 * kMaxChunks) + 1) * 32, n_chunks = (h->n_nodes + chunk - 1) / chunk;
+  double* totals = h->d_spec;
+  double* pre = totals + 4 * kMaxChunks;
+  double* clip = totals + 4 * kMaxChunks + 4 * (size_t)h->n_nodes;
+  const int grid = (h->n_t + kBinsPerBlock - 1) / kBinsPerBlock;
+  if (h->n_nodes <= kBinThreads) {
+    bins_kernel<true><<<grid, kBinThreads, 0, s>>>(m, theta, h->sin2w, h->kappa, g, d, n_chunks, 32, nullptr, nullptr,
+                                                   nullptr, S_out, W_out, ssm_out);
+    return launch_result();
   }
-  delta = delta && h->use_ref;
-  spectrum_point_kernel<<<grid, kSpecThreads, 0, s>>>(m, theta, df_from_double(h->sin2w), df_from_double(h->kappa),
-                                                        g, delta ? 1 : 0, S_out, W_out, ssm_out);
-  return launch_result();
+  moments_kernel<<<n_chunks, 64, 0, s>>>(m, theta, h->sin2w, h->kappa, g, d, chunk, totals, pre, clip);
+  cudaError_t e = launch_result();
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kBinThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, bins_kernel<false>, m, theta, h->sin2w, h->kappa, g, d, n_chunks, chunk,
+                         (const double*)totals, reinterpret_cast<const double2*>(pre), (const double*)clip, S_out, W_out, ssm_out);
+  return e != cudaSuccess ? e : launch_result();
 }
 
 // Builds S_SM (FP64), lambda, E_SM and shat.  Requires d_basis.

@@ -38,14 +38,12 @@ ModelView model_view(const srw_ctx* h) {
   m.midpoint = h->midpoint;
   m.t_min = (float)h->t_min;
   m.t_min64 = h->t_min;
-  m.node_a = h->d_node_a;
-  m.node_w = h->d_node_w;
-  m.node_c = h->d_node_c;
-  m.node_wlo = h->d_node_wlo;
   m.node64 = h->d_node64;
+  m.node_q = h->d_node_q;
+  m.node_k = h->d_node_k;
   m.bin_count = h->d_bin_count;
-  m.bin_f = h->d_bin_f;
-  m.bin_l = h->d_bin_l;
+  m.bin_n = h->d_bin_n;
+  m.bin_q = h->d_bin_q;
   m.bin64 = h->d_bin64;
   m.ssm32 = h->d_ssm32;
   m.esm32 = h->d_esm32;
@@ -74,12 +72,6 @@ template <class T>
 static void dfree(T*& p) {
   if (p) cudaFree((void*)p);
   p = nullptr;
-}
-
-static float int_bits_as_float(int v) {
-  float f;
-  std::memcpy(&f, &v, sizeof f);
-  return f;
 }
 
 static void split_df(double x, float* hi, float* lo) {
@@ -131,8 +123,8 @@ static void destroy_graphs(srw_ctx* h) {
 static void release(srw_ctx* h) {
   destroy_graphs(h);
   tc_release(h);
-  dfree(h->d_node_a); dfree(h->d_node_w); dfree(h->d_node_c); dfree(h->d_node_wlo); dfree(h->d_shat_lo); dfree(h->d_shat_k8); dfree(h->d_node64); dfree(h->d_bin_count); dfree(h->d_bin_f);
-  dfree(h->d_bin_l); dfree(h->d_bin64); dfree(h->d_basis); dfree(h->d_ssm64); dfree(h->d_esm64);
+  dfree(h->d_node64); dfree(h->d_node_q); dfree(h->d_node_k); dfree(h->d_shat_lo); dfree(h->d_shat_k8); dfree(h->d_bin_count); dfree(h->d_bin_n);
+  dfree(h->d_bin_q); dfree(h->d_spec); dfree(h->d_bin64); dfree(h->d_basis); dfree(h->d_ssm64); dfree(h->d_esm64);
   for (int f = 0; f < 2; ++f)
     for (int b = 0; b < 2; ++b) {
       dfree(h->d_kbr[f][b]);
@@ -274,8 +266,8 @@ static srw_status run_graph(srw_ctx* h, int path, int precision, int P, const vo
 // nodes reaching bin i are the prefix k_n >= i.
 static cudaError_t upload_tables(srw_ctx* h, const srw_binning* bin, const srw_source* sources, int n_sources,
                                  cudaStream_t s) {
-  dfree(h->d_node_a); dfree(h->d_node_w); dfree(h->d_node_c); dfree(h->d_node_wlo); dfree(h->d_node64);
-  dfree(h->d_bin_count); dfree(h->d_bin_f); dfree(h->d_bin_l); dfree(h->d_bin64);
+  dfree(h->d_node64); dfree(h->d_node_q); dfree(h->d_node_k); dfree(h->d_bin_count); dfree(h->d_bin_n); dfree(h->d_bin_q);
+  dfree(h->d_bin64);
   const int n_t = bin->n_t;
   const double t_min = h->t_min, f_tau = h->f_tau;
   int N = 0;
@@ -299,15 +291,10 @@ static cudaError_t upload_tables(srw_ctx* h, const srw_binning* bin, const srw_s
   std::vector<int> order(N);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return tmax[a] > tmax[b]; });
-  std::vector<float4> node_a(N), node_w(N), node_c(N), node_wlo(N);
-  std::vector<double> node64(5 * (size_t)N);
+  std::vector<double> node64(5 * (size_t)N), node_q(5 * (size_t)N, 0.0);
   for (int q = 0; q < N; ++q) {
     const int o = order[q];
     const double e = E[o];
-    const double wq[4] = {w[o] * pe[o], w[o] * pm[o], w[o] * pt[o], w[o]};
-    node_w[q] = make_float4((float)wq[0], (float)wq[1], (float)wq[2], (float)wq[3]);
-    node_wlo[q] = make_float4((float)(wq[0] - (double)node_w[q].x), (float)(wq[1] - (double)node_w[q].y),
-                              (float)(wq[2] - (double)node_w[q].z), (float)(wq[3] - (double)node_w[q].w));
     node64[q] = e;
     node64[(size_t)N + q] = w[o] * pe[o];
     node64[2 * (size_t)N + q] = w[o] * pm[o];
@@ -315,31 +302,23 @@ static cudaError_t upload_tables(srw_ctx* h, const srw_binning* bin, const srw_s
     node64[4 * (size_t)N + q] = w[o];
   }
   // ---- bins
-  std::vector<float4> bin_f(n_t);
-  std::vector<float> bin_l(n_t);
-  std::vector<double> bin64(2 * (size_t)n_t);
+  std::vector<double> bin_q(4 * (size_t)n_t, 0.0), bin64(2 * (size_t)n_t);
   std::vector<double> edge_hi(n_t), edge_c(n_t);
+  std::vector<char> below(n_t, 0);  // bins below the threshold: no width
   for (int i = 0; i < n_t; ++i) {
-    const double lo = bin->t_edges[i], hi = bin->t_edges[i + 1];
+    const double lo = bin->t_edges[i], hi = bin->t_edges[i + 1], tc = 0.5 * (lo + hi);
     bin64[i] = lo;
     bin64[(size_t)n_t + i] = hi;
     edge_hi[i] = hi;
-    edge_c[i] = 0.5 * (lo + hi);
-    if (h->midpoint) {
-      const double tc = 0.5 * (lo + hi);
-      // bins whose centre is below the threshold carry zero width
-      bin_f[i] = make_float4((float)tc, tc >= t_min ? (float)(hi - lo) : 0.f, 0.f, 0.f);
-      bin_l[i] = 0.f;
-    } else {
-      const double a = std::max(lo, t_min);
-      if (!(hi > a)) {
-        bin_f[i] = make_float4(1.f, 1.f, 0.f, 0.f);  // below threshold: zero-width bin
-        bin_l[i] = 0.f;
-        continue;
-      }
-      bin_f[i] = make_float4((float)a, (float)hi, (float)(hi - a), (float)(0.5 * (hi - a) * (a + hi)));
-      bin_l[i] = (float)std::log1p((hi - a) / a);
-    }
+    edge_c[i] = tc;
+    const double a = std::max(lo, t_min), d = h->midpoint ? hi - lo : hi - a;
+    below[i] = h->midpoint ? !(tc >= t_min) : !(hi > a);
+    if (below[i]) continue;
+    double* o = bin_q.data() + 4 * (size_t)i;
+    o[0] = d;
+    o[1] = h->midpoint ? 2.0 * tc : a + hi;
+    o[2] = h->midpoint ? tc * tc : (a * a + a * hi + hi * hi) / 3.0;
+    o[3] = h->midpoint ? d / tc : std::log1p(d / a);
   }
   std::vector<int> kn(N);
   for (int q = 0; q < N; ++q) {
@@ -352,14 +331,15 @@ static cudaError_t upload_tables(srw_ctx* h, const srw_binning* bin, const srw_s
     else
       k = (int)(std::upper_bound(ref.begin(), ref.end(), tm) - ref.begin());
     kn[q] = k;
-    node_a[q] = make_float4((float)e, (float)(1.0 / e), int_bits_as_float(k), (float)(kMe / (e * e)));
-    node_c[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    node_q[q] = 1.0 / e;
     if (!h->midpoint && k < n_t) {
       const double a = std::max(bin->t_edges[k], t_min), b = tm;
       if (b > a) {
         const double d = b - a, u = 1.0 - a / e, v = 1.0 - b / e;
-        node_c[q] = make_float4((float)d, (float)(0.5 * d * (a + b)), (float)(d * (u * u + u * v + v * v) / 3.0),
-                                (float)(std::log1p(d / a) - d / e));
+        node_q[(size_t)N + q] = d;
+        node_q[2 * (size_t)N + q] = 0.5 * d * (a + b);
+        node_q[3 * (size_t)N + q] = d * (u * u + u * v + v * v) / 3.0;
+        node_q[4 * (size_t)N + q] = std::log1p(d / a) - d / e;
       }
     }
   }
@@ -367,30 +347,31 @@ static cudaError_t upload_tables(srw_ctx* h, const srw_binning* bin, const srw_s
   std::vector<int> bin_count(n_t + 1, 0);
   for (int q = 0; q < N; ++q) bin_count[std::min(kn[q], n_t)] += 1;
   for (int i = n_t - 1; i >= 0; --i) bin_count[i] += bin_count[i + 1];
+  std::vector<int2> bin_n(n_t);
+  for (int i = 0; i < n_t; ++i) {
+    if (below[i]) bin_n[i] = make_int2(0, 0);
+    else bin_n[i] = make_int2(bin_count[i + 1], h->midpoint ? bin_count[i + 1] : bin_count[i]);
+  }
   bin_count.resize(n_t);
   for (int i = 0; i < n_t; ++i)
-    if (!h->midpoint && !(bin->t_edges[i + 1] > std::max(bin->t_edges[i], t_min))) bin_count[i] = 0;
+    if (!h->midpoint && below[i]) bin_count[i] = 0;
 
   cudaError_t e;
 #define TAB(call) \
   if ((e = (call)) != cudaSuccess) return e
-  TAB(dalloc(h, &h->d_node_a, N));
-  TAB(dalloc(h, &h->d_node_w, N));
-  TAB(dalloc(h, &h->d_node_c, N));
-  TAB(dalloc(h, &h->d_node_wlo, N));
   TAB(dalloc(h, &h->d_node64, 5 * (size_t)N));
+  TAB(dalloc(h, &h->d_node_q, 5 * (size_t)N));
+  TAB(dalloc(h, &h->d_node_k, N));
   TAB(dalloc(h, &h->d_bin_count, n_t));
-  TAB(dalloc(h, &h->d_bin_f, n_t));
-  TAB(dalloc(h, &h->d_bin_l, n_t));
+  TAB(dalloc(h, &h->d_bin_n, n_t));
+  TAB(dalloc(h, &h->d_bin_q, 2 * (size_t)n_t));
   TAB(dalloc(h, &h->d_bin64, 2 * (size_t)n_t));
-  TAB(cudaMemcpyAsync(h->d_node_a, node_a.data(), sizeof(float4) * N, cudaMemcpyHostToDevice, s));
-  TAB(cudaMemcpyAsync(h->d_node_w, node_w.data(), sizeof(float4) * N, cudaMemcpyHostToDevice, s));
-  TAB(cudaMemcpyAsync(h->d_node_c, node_c.data(), sizeof(float4) * N, cudaMemcpyHostToDevice, s));
-  TAB(cudaMemcpyAsync(h->d_node_wlo, node_wlo.data(), sizeof(float4) * N, cudaMemcpyHostToDevice, s));
   TAB(cudaMemcpyAsync(h->d_node64, node64.data(), sizeof(double) * node64.size(), cudaMemcpyHostToDevice, s));
   TAB(cudaMemcpyAsync(h->d_bin_count, bin_count.data(), sizeof(int) * n_t, cudaMemcpyHostToDevice, s));
-  TAB(cudaMemcpyAsync(h->d_bin_f, bin_f.data(), sizeof(float4) * n_t, cudaMemcpyHostToDevice, s));
-  TAB(cudaMemcpyAsync(h->d_bin_l, bin_l.data(), sizeof(float) * n_t, cudaMemcpyHostToDevice, s));
+  TAB(cudaMemcpyAsync(h->d_node_q, node_q.data(), sizeof(double) * node_q.size(), cudaMemcpyHostToDevice, s));
+  TAB(cudaMemcpyAsync(h->d_node_k, kn.data(), sizeof(int) * N, cudaMemcpyHostToDevice, s));
+  TAB(cudaMemcpyAsync(h->d_bin_n, bin_n.data(), sizeof(int2) * n_t, cudaMemcpyHostToDevice, s));
+  TAB(cudaMemcpyAsync(h->d_bin_q, bin_q.data(), sizeof(double) * bin_q.size(), cudaMemcpyHostToDevice, s));
   TAB(cudaMemcpyAsync(h->d_bin64, bin64.data(), sizeof(double) * bin64.size(), cudaMemcpyHostToDevice, s));
 #undef TAB
   return cudaStreamSynchronize(s);  // the host tables go out of scope
@@ -459,8 +440,8 @@ static srw_status build_joint(srw_ctx* h, const srw_binning* bin, const srw_sour
                        cudaMemcpyDeviceToHost, s), "basis download");
     JC(cudaStreamSynchronize(s), "basis sync");
   }
-  dfree(h->d_node_a); dfree(h->d_node_w); dfree(h->d_node_c); dfree(h->d_node_wlo); dfree(h->d_node64);
-  dfree(h->d_bin_count); dfree(h->d_bin_f); dfree(h->d_bin_l); dfree(h->d_bin64); dfree(h->d_basis);
+  dfree(h->d_node64); dfree(h->d_node_q); dfree(h->d_node_k); dfree(h->d_bin_count); dfree(h->d_bin_n); dfree(h->d_bin_q);
+  dfree(h->d_bin64); dfree(h->d_basis);
   int total_nodes = 0;
   for (int k = 0; k < n_src; ++k) total_nodes += sources[k].n_nodes;
   h->n_nodes = total_nodes;
@@ -718,6 +699,7 @@ static srw_status create_impl(const srw_binning* bin, const srw_source* sources,
   if (!jr) {
     CREATE_CUDA(upload_tables(h, bin, sources, n_sources, s), "node tables");
     CREATE_CUDA(alloc_axis(h, s), "alloc");
+    CREATE_CUDA(dalloc(h, &h->d_spec, 4 * (size_t)kSpecChunks + 5 * (size_t)h->n_nodes), "alloc spectrum workspace");
     CREATE_CUDA(cudaMemcpy2DAsync(h->d_R, (size_t)h->ld_r * sizeof(float), R, (size_t)n_t * sizeof(float),
                                   (size_t)n_t * sizeof(float), n_rec, cudaMemcpyHostToDevice, s), "upload R");
     if (h->has_esm_input)
@@ -894,8 +876,8 @@ srw_status srw_spectrum(srw_handle h, const float* theta, int stage, float* out,
       SRW_CUDA(h, launch_basis_eval(h, th, stage, dst, s), "spectrum kernel");
     } else {
       SRW_CUDA(h, launch_weights_from_basis(h, th, h->d_W, s), "weights kernel");
-      SRW_CUDA(h, launch_fold_point(h, h->d_W, stage == 2 ? dst : nullptr, stage == 3 ? dst : nullptr, nullptr, s, true),
-               "fold kernel");
+      SRW_CUDA(h, launch_fold_point_after(h, h->d_W, stage == 2 ? dst : nullptr, stage == 3 ? dst : nullptr, nullptr, s,
+                                          true), "fold kernel");
     }
   } else if (stage == 0) {
     SRW_CUDA(h, launch_spectrum_point(h, th, dst, nullptr, nullptr, s), "spectrum kernel");
@@ -904,8 +886,9 @@ srw_status srw_spectrum(srw_handle h, const float* theta, int stage, float* out,
     float* Wbuf = (stage == 1 && dev) ? out : h->d_W;
     SRW_CUDA(h, launch_spectrum_point(h, th, nullptr, Wbuf, nullptr, s, stage >= 2), "spectrum kernel");
     // the spectrum kernel forms a deviation only with a reference point set
-    if (stage == 2) SRW_CUDA(h, launch_fold_point(h, h->d_W, dst, nullptr, nullptr, s, h->use_ref != 0), "fold kernel");
-    if (stage == 3) SRW_CUDA(h, launch_fold_point(h, h->d_W, nullptr, dst, nullptr, s, h->use_ref != 0), "fold kernel");
+    if (stage >= 2)
+      SRW_CUDA(h, launch_fold_point_after(h, h->d_W, stage == 2 ? dst : nullptr, stage == 3 ? dst : nullptr, nullptr, s,
+                                          h->use_ref != 0), "fold kernel");
   }
   if (!dev) {
     SRW_CUDA(h, cudaMemcpyAsync(out, dst, sizeof(float) * n_out, cudaMemcpyDeviceToHost, s), "download");
@@ -950,7 +933,7 @@ static srw_status loglik_impl(srw_handle h, const float* theta, int P, double* o
         cudaError_t e = h->joint ? launch_weights_from_basis(h, th + 5 * (size_t)p, h->d_W, cs)
                                  : launch_spectrum_point(h, th + 5 * (size_t)p, nullptr, h->d_W, nullptr, cs, true);
         if (e != cudaSuccess) return e;
-        if ((e = launch_fold_point(h, h->d_W, nullptr, nullptr, o + p, cs, h->joint || h->use_ref)) != cudaSuccess)
+        if ((e = launch_fold_point_after(h, h->d_W, nullptr, nullptr, o + p, cs, h->joint || h->use_ref)) != cudaSuccess)
           return e;
       }
       return cudaSuccess;
@@ -989,7 +972,7 @@ static srw_status loglik_impl(srw_handle h, const float* theta, int P, double* o
       // weights kernel runs
       cudaError_t e = launch_weights_from_basis(h, th, h->d_W, cs);
       if (e != cudaSuccess) return e;
-      return launch_fold_point_after(h, h->d_W, o, cs);
+      return launch_fold_point_after(h, h->d_W, nullptr, nullptr, o, cs, true);
     });
   } else {
     const int n_parts_max = precision == SRW_FP32 ? fold_simt_parts(h, P) : (h->rec_pad / 128);

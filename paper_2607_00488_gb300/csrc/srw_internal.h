@@ -55,20 +55,21 @@ constexpr bool kDebugChecks = false;
 constexpr int kCanaryDoubles = 64;
 constexpr unsigned long long kCanaryBits = 0x7ff4dead5ca1ab1eull;  // a signalling-NaN pattern
 
+// Chunks of nodes whose totals the single-point spectrum scans.
+constexpr int kSpecChunks = 256;
+
 // Device-side view of the theta-independent model tables.
 struct ModelView {
   int n_t, n_rec, n_nodes, k_pad, ld_r, midpoint;
   float t_min;
   double t_min64;
   // nodes sorted by T_max descending
-  const float4* node_a;  // {E, 1/E, k_n (int bits), m_e/E^2}; k_n = #bins with T_hi <= T_max(E)
-  const float4* node_w;  // {w P_e, w P_mu, w P_tau, w}
-  const float4* node_wlo;  // FP32 residuals of node_w (node_w + node_wlo = FP64 value)
-  const float4* node_c;  // FP64-exact integrals over the clipped bin k_n: {I0, I1, J, MM}
-  const double* node64;  // [5][n_nodes]: E, w P_e, w P_mu, w P_tau, w (FP64, same order)
+  const double* node64;  // [5][n_nodes]: E, w P_e, w P_mu, w P_tau, w
+  const double* node_q;  // [5][n_nodes]: 1/E, and over the bin clipped at T_max(E): I0, I1, J, MM
+  const int* node_k;     // [n_nodes]: k_n, the number of bins below T_max(E)
   const int* bin_count;  // per bin: nodes [0, count) may contribute
-  const float4* bin_f;   // {a = max(T_lo, t_min), b = T_hi, I0 = b - a, I1 = (b-a)(a+b)/2}
-  const float* bin_l;    // log(b/a) per bin (from FP64)
+  const int2* bin_n;     // per bin: nodes [0, x) cover it whole, [x, y) end inside it
+  const double2* bin_q;  // [n_t][2]: {I0, p}, {q, L} of the whole bin (see spectrum.cu)
   const double* bin64;   // [2][n_t]: T_lo, T_hi (FP64)
   const float* ssm32;    // [n_t] S_SM from the FP32 spectrum kernel (weights denominator)
   const float* esm32;    // [n_t] E_SM baseline
@@ -154,14 +155,13 @@ struct srw_ctx {
   size_t device_bytes = 0;
 
   // model tables
-  float4* d_node_a = nullptr;
-  float4* d_node_w = nullptr;
-  float4* d_node_c = nullptr;
-  float4* d_node_wlo = nullptr;
   double* d_node64 = nullptr;
+  double* d_node_q = nullptr;
+  int* d_node_k = nullptr;
   int* d_bin_count = nullptr;
-  float4* d_bin_f = nullptr;
-  float* d_bin_l = nullptr;
+  int2* d_bin_n = nullptr;
+  double2* d_bin_q = nullptr;
+  double* d_spec = nullptr;  // workspace of the single-point spectrum: chunk totals, prefix sums, clipped terms
   double* d_bin64 = nullptr;
   double* d_basis = nullptr;   // [8][n_t] FP64 coefficient spectra
   double* d_ssm64 = nullptr;   // [n_t] FP64 S_SM
@@ -326,7 +326,8 @@ cudaError_t launch_fold_point(const srw_ctx* h, const float* W, float* musig_out
                               cudaStream_t s, bool delta = false);
 // The single-point fold (delta mode) as a programmatic dependent of the
 // preceding kernel on s: it starts while that kernel runs and waits for W.
-cudaError_t launch_fold_point_after(const srw_ctx* h, const float* W, double* out, cudaStream_t s);
+cudaError_t launch_fold_point_after(const srw_ctx* h, const float* W, float* musig_out, float* mu_out, double* out,
+                                    cudaStream_t s, bool delta);
 cudaError_t launch_reduce_parts(const srw_ctx* h, const double* parts, int n_parts, int P, double* out,
                                 cudaStream_t s);
 

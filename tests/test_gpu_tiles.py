@@ -95,3 +95,28 @@ def test_rank8_and_profiled_rounds(srw, n_rec, p):
             if k < len(prof):
                 p1, a1 = lk.loglik_profiled(theta[k:k + 1], 0.05)
                 assert p1[0] == prof[k] and a1[0] == alpha[k]
+
+
+# The single-point spectrum sums up to 128 nodes in the bins' blocks, more in
+# chunks of 32 (longer ones from 8193 nodes on), and the bins 32 to a block; some bins lie below the threshold, some
+# hold many clipped nodes, the topmost none.  S is an FP64 sum rounded to FP32
+# (6e-8); its terms cancel to (m_e / (m_e + 2E))^2 >= 2e-4, so 1e-7 holds with
+# room for the FP64 rounding of up to 2e4 terms.
+@pytest.mark.parametrize("midpoint", [False, True])
+@pytest.mark.parametrize("n_nodes,n_t", [(1, 1), (31, 33), (32, 32), (33, 31), (128, 7), (129, 7), (1000, 5), (8192, 64),
+                                         (8193, 257), (20000, 100)])
+def test_spectrum_node_chunks_and_bin_blocks(srw, n_nodes, n_t, midpoint):
+    rng = np.random.default_rng(n_nodes + n_t)
+    e = rng.uniform(0.2, 16.0, n_nodes)
+    src = [{"name": "s", "e": e, "w": rng.uniform(0.1, 1.0, n_nodes), "pee": rng.uniform(0.3, 0.6, n_nodes)}]
+    t_edges = np.linspace(0.0, 17.0, n_t + 1)
+    wl = line_workload(n_t, 8)
+    wl.update(sources=src, t_edges=t_edges, t_min=0.3 if n_t > 1 else 1e-3)
+    theta = np.array([[0.11, -0.07, 0.21, 0.05, 1.3], [0.0, 0.0, 0.0, 0.0, 0.0]], np.float32)
+    with srw.Likelihood(wl, midpoint=midpoint, e_true_sm=np.ones(n_t)) as lk:  # one centre above T_max: S_SM = 0
+        for t in theta:
+            want = O.recoil_spectrum(src, t_edges, t.astype(np.float64), wl["t_min"], wl["sin2w"], wl["f_tau"],
+                                     midpoint=midpoint)
+            got = lk.spectrum(t, 0)
+            np.testing.assert_allclose(got, want, rtol=1e-7, atol=0)
+            np.testing.assert_array_equal(got == 0, want == 0)
