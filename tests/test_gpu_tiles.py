@@ -120,3 +120,58 @@ def test_spectrum_node_chunks_and_bin_blocks(srw, n_nodes, n_t, midpoint):
             got = lk.spectrum(t, 0)
             np.testing.assert_allclose(got, want, rtol=1e-7, atol=0)
             np.testing.assert_array_equal(got == 0, want == 0)
+
+
+# Tensor-core fold: per (rec tile, block of 64 true bins) only the rows of R with
+# nonzero split elements are multiplied.  Bands that start and end anywhere,
+# single elements at a block's corners, empty rows and an empty tile.  Bound:
+# the dropped lo x lo product and the splits' residuals (2^-15 / 2^-21 of each
+# product of R with W - W_ref), FP32 accumulation over n_t terms, one rounding
+# of the result and of the FP32 spectra.
+@pytest.mark.parametrize("prec,split", [("bf16x3", 2.0**-15), ("fp16x3", 2.0**-21)])
+@pytest.mark.parametrize("n_t,n_rec,form", [(300, 300, "band"), (65, 257, "corners"), (257, 520, "gap"), (129, 16, "band")])
+def test_tensor_fold_rows_left_out(srw, n_t, n_rec, form, prec, split):
+    wl = line_workload(n_t, n_rec)
+    r = wl["R"].copy()
+    i, j = np.arange(n_t)[None, :], np.arange(n_rec)[:, None]
+    if form == "band":
+        keep = np.abs(i / n_t - j / n_rec - 0.07) < 0.06
+    elif form == "corners":
+        keep = ((i % 64 == 0) | (i % 64 == 63) | (i == n_t - 1)) & ((j % 16 == 0) | (j % 16 == 15) | (j == n_rec - 1))
+        r = np.maximum(r, 1e-6)
+    else:
+        keep = (j < 250) | (j >= 513)  # rows 256..511, a whole tile, are empty
+    wl["R"] = np.ascontiguousarray(np.where(keep, r, 0.0), dtype=r.dtype)
+    m, counts = model_and_counts(wl)
+    theta = workloads.fit_region_points(130, seed=n_t)
+    basis = O.coefficient_spectra(m.sources, m.t_edges, m.t_min)
+    shat = np.where(m.s_sm != 0, basis * (m.e_sm / np.where(m.s_sm != 0, m.s_sm, 1.0)), 0.0)
+    c = np.array([O.coupling_coefficients(t) for t in theta.astype(np.float64)])
+    dw = (c - O.coupling_coefficients(np.zeros(5))) @ shat
+    _, mu = values(m, oracle_matrix(m), theta)
+    bound = (split + n_t * 2.0**-24) * (np.abs(dw) @ m.r.T) + 2.0**-22 * mu
+    with srw.Likelihood(wl, counts) as lk:
+        spec = lk.spectrum_batch(theta, srw.PRECISIONS[prec])
+    assert np.all(np.abs(spec - (mu - m.bkg_sum)) <= bound)
+
+
+# Surrogate: the scan takes 256 points a unit and the GEMM tiles narrow for few
+# rows; every output adds the same products in the same order, so a point's
+# outputs and value do not depend on the size of the batch that holds it.
+@pytest.mark.parametrize("n_rec", [1, 255, 257, 600])
+def test_surrogate_batch_sizes(srw, n_rec):
+    from workloads.mlp import BOX_CENTRE, BOX_HALF, init_weights, round_to_bf16
+    wl = line_workload(64, n_rec)
+    _, counts = model_and_counts(wl)
+    params = [(round_to_bf16(W), round_to_bf16(b)) for W, b in init_weights(n_rec, seed=5)]
+    theta = workloads.theta_box(40000, 43)
+    with srw.Likelihood(wl, counts) as lk:
+        s = srw.Surrogate(lk, params, BOX_CENTRE, BOX_HALF)
+        try:
+            y, v = s.forward(theta[:20000]), s.loglik(theta)
+            assert np.all(np.isfinite(v))
+            for p in (1, 127, 129, 255, 256, 257, 4096):
+                np.testing.assert_array_equal(s.forward(theta[:p]), y[:p])
+                np.testing.assert_array_equal(s.loglik(theta[:p]), v[:p])
+        finally:
+            s.close()
