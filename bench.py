@@ -543,7 +543,8 @@ def fold_roofline(srw, lk, info, prec, prec_name, P, fold_ms, peaks, peak_src):
     """Roofline of the batched fold: useful flops 2 N_rec N_T per point (the
     dense contraction, whatever the kernel skips or repeats) over the kernel's
     own device time, against the measured burst peak; beside it the executed
-    tensor-core work (products x executed (rec tile, K block) pairs)."""
+    tensor-core work (products x executed (rec tile, K block) pairs, whole
+    blocks: their all-zero rows are left out of the MMAs, so this can exceed 1)."""
     fold_s = statistics.mean(fold_ms) * 1e-3
     work = lk.fold_work(prec)
     dense = 2.0 * info["n_rec"] * info["n_t"] * P
