@@ -198,7 +198,7 @@ srw_status srw_set_data(srw_handle h, const double* counts, const double* bkg, i
  *   stage 1: W_i = w_i(theta) E_SM,i, the reweighted true spectrum (n_t floats)
  *   stage 2: sum_i R_ji W_i, the folded signal                   (n_rec floats)
  *   stage 3: mu_j = M_j (signal_j + background_j)                (n_rec floats)
- * Computed by the single-point kernels (FP32). */
+ * Computed by the single-point kernels (spectrum in FP64, rounded to FP32; FP32 fold). */
 srw_status srw_spectrum(srw_handle h, const float* theta, int stage, float* out, int where, void* stream);
 
 /* -2 ln L (without pull terms) for P parameter points.
@@ -219,7 +219,7 @@ srw_status srw_loglik(srw_handle h, const float* theta, int P, double* out, int 
 
 /* The plain single-point FP32 path applied to P points one after another, as
  * the paper's pipeline does it (Sec. IV.B): per point the cross-section
- * integrals are recomputed over all (node, bin) pairs by the spectrum kernel,
+ * integrals of every node are recomputed and summed by the spectrum kernels,
  * then one HBM-streaming fold; launches in order, replayed from a captured
  * CUDA graph per call signature, like srw_loglik. */
 srw_status srw_loglik_points(srw_handle h, const float* theta, int P, double* out, int where, void* stream);

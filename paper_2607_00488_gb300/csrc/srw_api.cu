@@ -704,7 +704,7 @@ static srw_status create_impl(const srw_binning* bin, const srw_source* sources,
                                   (size_t)n_t * sizeof(float), n_rec, cudaMemcpyHostToDevice, s), "upload R");
     if (h->has_esm_input)
       CREATE_CUDA(cudaMemcpyAsync(h->d_esm64, opt->e_true_sm, sizeof(double) * n_t, cudaMemcpyHostToDevice, s), "upload");
-    // ---- G0 coefficient spectra (FP64), S_SM, E_SM, shat; then S_SM of the FP32 kernel
+    // ---- G0 coefficient spectra (FP64), S_SM, E_SM, shat; then S_SM as the single-point spectrum forms it
     CREATE_CUDA(launch_basis_fp64(h, s), "basis kernel");
     CREATE_CUDA(launch_build_shat(h, s), "shat kernels");
     CREATE_CUDA(launch_spectrum_point(h, h->d_theta0, nullptr, nullptr, h->d_ssm32, s), "SM spectrum kernel");

@@ -71,7 +71,7 @@ struct ModelView {
   const int2* bin_n;     // per bin: nodes [0, x) cover it whole, [x, y) end inside it
   const double2* bin_q;  // [n_t][2]: {I0, p}, {q, L} of the whole bin (see spectrum.cu)
   const double* bin64;   // [2][n_t]: T_lo, T_hi (FP64)
-  const float* ssm32;    // [n_t] S_SM from the FP32 spectrum kernel (weights denominator)
+  const float* ssm32;    // [n_t] S_SM from the single-point spectrum kernels (weights denominator)
   const float* esm32;    // [n_t] E_SM baseline
   const float* R;        // [n_rec][ld_r] FP32, zero padded
 };
