@@ -65,8 +65,9 @@ __device__ __forceinline__ dfloat poisson_term_df(dfloat mu, dfloat n) {
   return df_add(df_add(mu, dfloat{-n.hi, -n.lo}), df_mul(n, l));
 }
 
-// a / b where b is 0, infinite, NaN or at least 1e-30 in magnitude: the fast
-// division without its scaling of subnormal divisors.
+// a / b as the product with PTX's approximate reciprocal (rcp.approx.ftz: 1 ulp,
+// a subnormal b counts as 0), for b that is 0, infinite, NaN or at least 1e-30 in
+// magnitude.
 __device__ __forceinline__ float reciprocal(float b) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
