@@ -92,7 +92,7 @@ template <int MI, int NI>
 __global__ void __launch_bounds__(THR, MI * NI == 4 ? 2 : 4)
 fold_simt_kernel(const float* __restrict__ theta, int P, dfloat sin2w, CoefRef cref, const float* __restrict__ shk,
                  int k_pad, const float* __restrict__ Rt, int n_rec, const float4* __restrict__ consts,
-                 double* __restrict__ parts, float* __restrict__ musig_out, const float* __restrict__ muref,
+                 const double* __restrict__ n64, const double* __restrict__ b64, double* __restrict__ parts, float* __restrict__ musig_out, const float* __restrict__ muref,
                  unsigned* __restrict__ status, const int4* __restrict__ order) {
   using S = SimtShape<MI, NI>;
   constexpr int BM = S::BM, BN = S::BN;
@@ -257,7 +257,11 @@ fold_simt_kernel(const float* __restrict__ theta, int P, dfloat sin2w, CoefRef c
     for (int r = 0; r < 4 * MI; ++r) {
       const float2 s2 = unpk(sum[r][c / 2]), c2 = unpk(comp[r][c / 2]);
       const dfloat dev = two_sum((c & 1) ? s2.y : s2.x, (c & 1) ? -c2.y : -c2.x);
-      const dfloat t = poisson_term_df(df_add(dev, dfloat{nb.z, nb.w}), dfloat{nb.x, nb.y});
+      dfloat t;
+      if (!poisson_term_df(df_add(dev, dfloat{nb.z, nb.w}), dfloat{nb.x, nb.y}, &t)) {
+        const double x = poisson_term_f64(((double)dev.hi + (double)dev.lo) + b64[j], n64[j]);
+        t = isfinite(x) ? df_from_double(x) : dfloat{(float)x, 0.f};
+      }
       if (isinf(t.hi)) inf[r] = true;
       else d[r] = df_add(d[r], t);
     }
@@ -326,8 +330,8 @@ void launch_shape(const srw_ctx* h, const float* theta, int P, double* parts, cu
   using S = SimtShape<MI, NI>;
   const dim3 grid((P + S::BM - 1) / S::BM, (h->n_rec + S::BN - 1) / S::BN);
   fold_simt_kernel<MI, NI><<<grid, THR, 0, s>>>(theta, P, df_from_double(h->sin2w), h->cref, h->d_simt_sh, h->k_pad,
-                                                h->d_simt_r, h->n_rec, h->d_simt_c, parts, musig_out, h->d_muref32,
-                                                h->d_status, order);
+                                                h->d_simt_r, h->n_rec, h->d_simt_c, h->d_n64, h->d_bref64, parts,
+                                                musig_out, h->d_muref32, h->d_status, order);
 }
 
 // The small tile where the large ones do not give every SM a block.

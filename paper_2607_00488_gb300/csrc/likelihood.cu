@@ -342,7 +342,9 @@ __global__ void data_ref_kernel(const double* __restrict__ n64, const double* __
   const double br = b64[j] + muref[j];
   bref64[j] = br;
   const bool on = mask == nullptr || mask[j] != 0;
-  const dfloat nd = df_from_double(n64[j]), bd = df_from_double(br);
+  dfloat nd = df_from_double(n64[j]);
+  const dfloat bd = df_from_double(br);
+  if (n64[j] != 0.0 && nd.hi == 0.f) nd = {1e-38f, 0.f};  // below FP32, but data (the term takes n64)
   simt_c[2 * j] = make_float4(nd.hi, nd.lo, bd.hi, bd.lo);
   simt_c[2 * j + 1] = make_float4(on ? 1.f : 0.f, 0.f, 0.f, 0.f);
   nb2[j] = make_float2(on ? (float)n64[j] : -1.f, (float)br);

@@ -27,17 +27,18 @@ __device__ __forceinline__ double poisson_term_f64(double mu, double n) {
 // ~sqrt(2) of mu and v = (n' - mu)/(n' + mu),
 //   ln(n/mu) = k ln 2 + 2 atanh(v) = k ln 2 + 2 v (1 + v^2 (1/3 + v^2 q(v^2))),
 // |v| < 0.18; q in FP32 (its part of the bracket is below 0.007, so its
-// rounding is below 1e-9 v^3), the rest in double-float.  Same domain rules as
-// poisson_term_f64; a mu too small for FP32 quotients takes that function.
-__device__ __forceinline__ dfloat poisson_term_df(dfloat mu, dfloat n) {
-  if (n.hi == 0.f && !(mu.hi < 0.f)) return mu;
-  if (!(mu.hi > 1e-30f)) {
-    const double t = poisson_term_f64((double)mu.hi + (double)mu.lo, (double)n.hi + (double)n.lo);
-    return isfinite(t) ? df_from_double(t) : dfloat{(float)t, 0.f};
+// rounding is below 1e-9 v^3), the rest in double-float.  False, and no term,
+// outside 1e-30 < mu, n with n / mu within 2^+-96 (n = 0 with mu >= 0 is
+// inside), where n', mu and their low parts are normal FP32 numbers; NaN and
+// infinities are outside as well.  The caller then takes poisson_term_f64.
+__device__ __forceinline__ bool poisson_term_df(dfloat mu, dfloat n, dfloat* t) {
+  if (n.hi == 0.f && mu.hi >= 0.f) {
+    *t = mu;
+    return true;
   }
   const float r = __fdividef(n.hi, mu.hi) * 1.41421356f;
-  int k = (__float_as_int(r) >> 23) - 127;  // r > 0: n / mu in 2^k [0.707, 1.415)
-  k = max(-100, min(100, k));
+  const int k = (__float_as_int(r) >> 23) - 127;  // r > 0: n / mu in 2^k [0.707, 1.415)
+  if (!(mu.hi > 1e-30f) || !(n.hi > 1e-30f) || abs(k) > 96) return false;
   const float p2 = __int_as_float((127 - k) << 23);
   const dfloat ns = {n.hi * p2, n.lo * p2};
   const dfloat d = df_add(ns, dfloat{-mu.hi, -mu.lo}), s = df_add(ns, mu);
@@ -62,7 +63,8 @@ __device__ __forceinline__ dfloat poisson_term_df(dfloat mu, dfloat n) {
   dfloat kl = two_prod(kf, ln2.hi);
   kl = fast_two_sum(kl.hi, fmaf(kf, ln2.lo, kl.lo));
   l = df_add(kl, l);
-  return df_add(df_add(mu, dfloat{-n.hi, -n.lo}), df_mul(n, l));
+  *t = df_add(df_add(mu, dfloat{-n.hi, -n.lo}), df_mul(n, l));
+  return true;
 }
 
 // a / b as the product with PTX's approximate reciprocal (rcp.approx.ftz: 1 ulp,

@@ -1,0 +1,91 @@
+"""Values at the ends of what the evaluators take, and in batches of other sizes.
+
+Bins with almost no expectation beside their data, counts below FP32's range,
+empty bins beside ordinary ones, batches on either side of the tile and unit
+rules (a point's value may not depend on the batch that holds it), very many
+reconstructed bins, and a surrogate pass whose device wait runs out.
+"""
+
+import numpy as np
+import pytest
+
+import oracle as O
+import workloads
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def srw():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2607_00488_gb300 as pkg
+    pkg.srw_fault_inject("none")
+    yield pkg
+    pkg.srw_fault_inject("none")
+
+
+def line(n_t, n_rec, exposure=2.0e4):
+    """One 7Be line on [0, 1] MeV, smeared onto n_rec bins of [0, 1.3] MeV."""
+    t_edges, rec_edges = np.linspace(0.0, 1.0, n_t + 1), np.linspace(0.0, 1.3, n_rec + 1)
+    r = workloads.solar.response_matrix(t_edges, rec_edges, res=0.06, tail_frac=1e-3)
+    return {"name": "line", "t_edges": t_edges, "rec_edges": rec_edges, "sources": workloads.solar.be7_sources(), "R": r,
+            "bkg": np.full((1, n_rec), 0.1 * exposure / n_rec), "exposure": exposure, "t_min": 1e-3, "sin2w": 0.23121,
+            "f_tau": 0.5}
+
+
+def oracle_of(wl, counts=None):
+    m = O.OracleModel.from_workload(wl)
+    m.set_data(np.zeros(wl["R"].shape[0]), wl["bkg"])
+    if counts is None:
+        counts = workloads.poisson_counts(m.mu(np.zeros(5)), 3)
+    m.set_data(counts, wl["bkg"])
+    return m, counts
+
+
+def with_bins(n_t, n_rec, bins):
+    """The line with given expectations (no background) and counts in some bins: {bin: (mu, n)}."""
+    wl = line(n_t, n_rec)
+    r, bkg = wl["R"].copy(), wl["bkg"].copy()
+    m, counts = oracle_of(wl)
+    total = float(m.e_sm.sum())
+    for j, (mu, n) in bins.items():
+        r[j, :] = np.float32(mu / total)
+        bkg[:, j] = 0.0
+        counts[j] = n
+    wl.update(R=r, bkg=bkg, e_true_sm=m.e_sm)
+    return wl, counts
+
+
+# A count beside an expectation of 1e-30 .. 1e-24: n / mu beyond 2^100.  FP32
+# products: |d(-2 ln L)| <= 1e-4 in the fit region (the library's bar; a relative
+# error of 2^-24 of the deviation from the reference moves the three terms by at
+# most 2 x 3 x 1e3 x 2^-24 x 0.1 = 4e-5), and 2^-50 of the sum for its rounding.
+@pytest.mark.parametrize("p", [3, 10000])
+@pytest.mark.parametrize("n,mu", [(10.0, 1.1e-30), (100.0, 1.5e-30), (100.0, 1e-29), (100.0, 1e-28), (1e3, 1e-26),
+                                  (1e3, 1e-24), (3.0, 1e-31)])
+def test_fp32_batch_counts_without_expectation(srw, n, mu, p):
+    wl, counts = with_bins(64, 130, {0: (mu, n), 70: (mu, n), 129: (mu, n)})
+    m = O.OracleModel.from_workload(wl, e_true_sm=wl["e_true_sm"])
+    m.set_data(counts, wl["bkg"])
+    theta = workloads.fit_region_points(p, seed=7)
+    pick = np.unique(np.linspace(0, p - 1, 5).astype(int))
+    want = m.neg2lnl_batch(theta[pick].astype(np.float64))
+    with srw.Likelihood(wl, counts, e_true_sm=wl["e_true_sm"]) as lk:
+        got = lk.loglik(theta, srw.SRW_FP32)[pick]
+    np.testing.assert_allclose(got, want, rtol=2.0**-50, atol=1e-4)
+
+
+# A count below FP32's range in a bin that expects nothing: outside the domain.
+@pytest.mark.parametrize("n", [1.0, 1e-40, 1e-50])
+def test_fp32_batch_tiny_count_is_data(srw, n):
+    wl, counts = with_bins(64, 130, {70: (0.0, n)})
+    out = torch.zeros(3, dtype=torch.float64, device="cuda")
+    theta = torch.from_numpy(workloads.fit_region_points(3, seed=7)).cuda()
+    with srw.Likelihood(wl, counts, e_true_sm=wl["e_true_sm"]) as lk:
+        lk.loglik(theta, srw.SRW_FP32, out=out)
+        torch.cuda.synchronize()
+        assert np.all(np.isposinf(out.cpu().numpy()))
