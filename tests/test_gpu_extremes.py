@@ -79,6 +79,25 @@ def test_fp32_batch_counts_without_expectation(srw, n, mu, p):
     np.testing.assert_allclose(got, want, rtol=2.0**-50, atol=1e-4)
 
 
+# FP32 products at the reference point, where the fold's deviation is exactly 0:
+# what is left is the Poisson term of mu = b + R W_ref (FP64) in double-float.
+# Its bound is 1.4e-13 (n + mu), twice that for -2 ln L; 2e-14 (n + mu) more for
+# mu and the data constant, sums of a few hundred FP64 terms in either program.
+def test_fp32_batch_poisson_term_at_the_reference(srw):
+    wl = line(40, 1, exposure=3.0e3)
+    m, _ = oracle_of(wl)
+    mu = float(m.mu(np.zeros(5))[0])
+    theta = np.zeros((2, 5), np.float32)
+    worst = 0.0
+    for ratio in np.concatenate([np.linspace(0.70, 0.75, 12), np.linspace(1.3, 1.42, 12), [0.01, 0.3, 1.001, 7.0, 60.0]]):
+        counts = np.array([np.floor(mu * ratio) + 1.0])
+        m.set_data(counts, wl["bkg"])
+        with srw.Likelihood(wl, counts) as lk:
+            got = lk.loglik(theta, srw.SRW_FP32)
+        worst = max(worst, np.max(np.abs(got - m.neg2lnl(theta[0]))) / (counts[0] + mu))
+    assert worst <= 3.0e-13
+
+
 # A count below FP32's range in a bin that expects nothing: outside the domain.
 @pytest.mark.parametrize("n", [1.0, 1e-40, 1e-50])
 def test_fp32_batch_tiny_count_is_data(srw, n):
