@@ -87,13 +87,17 @@ __device__ __forceinline__ void coefficients(const float* th, dfloat s, const Co
 // 16-byte copies bring in three K tiles ahead (the row-major R went through
 // registers and was transposed by four 4-byte stores per load).  order: {first
 // and end K tile holding nonzero response, rec tile, 0}, longest range first,
-// so that the last wave holds the short ones.
+// so that the last wave holds the short ones.  The range is that of the 128
+// bins around a tile in both shapes, which then add the same terms in the same
+// order (a range per 64 bins, with warps that sit out the rest of the large
+// tile's, cost the large tile 7 %).
 template <int MI, int NI>
 __global__ void __launch_bounds__(THR, MI * NI == 4 ? 2 : 4)
 fold_simt_kernel(const float* __restrict__ theta, int P, dfloat sin2w, CoefRef cref, const float* __restrict__ shk,
                  int k_pad, const float* __restrict__ Rt, int n_rec, const float4* __restrict__ consts,
-                 const double* __restrict__ n64, const double* __restrict__ b64, double* __restrict__ parts, float* __restrict__ musig_out, const float* __restrict__ muref,
-                 unsigned* __restrict__ status, const int4* __restrict__ order) {
+                 const double* __restrict__ n64, const double* __restrict__ b64, double* __restrict__ parts,
+                 float* __restrict__ musig_out, const float* __restrict__ muref, unsigned* __restrict__ status,
+                 const int4* __restrict__ order) {
   using S = SimtShape<MI, NI>;
   constexpr int BM = S::BM, BN = S::BN;
   __shared__ __align__(16) float ring[kRing][BK][S::kRow];
@@ -239,62 +243,71 @@ fold_simt_kernel(const float* __restrict__ theta, int P, dfloat sin2w, CoefRef c
   if (parts == nullptr) return;
   // Epilogue: Poisson terms over this block's rec bins per point, in double-
   // float: FP64 (a warp's instruction takes the SM's unit 16 cycles) spent
-  // 0.7 ms of a 4096-point call's 2.7 ms on the logarithms here.
-  dfloat d[4 * MI];
-  bool inf[4 * MI];
+  // 0.7 ms of a 4096-point call's 2.7 ms on the logarithms here.  A sum over 16
+  // bins (four a thread, then its four neighbours) is in double-float, the four
+  // of 64 bins are added in FP64 in the order of the bins and are one partial
+  // sum: the same in every tile shape, so that a point's value does not depend
+  // on the batch that holds it.
+  // the ring is free (its last copies landed above)
+  float2(*psum)[BM] = reinterpret_cast<float2(*)[BM]>(&ring[0][0][0]);  // [16 bins][point]
+  int(*pinf)[BM] = reinterpret_cast<int(*)[BM]>(&ring[1][0][0]);
+  static_assert(sizeof(float2) * 4 * NI * BM <= sizeof(ring[0]), "sums of four warps in a ring slot");
+  __syncthreads();
 #pragma unroll
-  for (int r = 0; r < 4 * MI; ++r) {
-    d[r] = {0.f, 0.f};
-    inf[r] = false;
-  }
-#pragma unroll
-  for (int c = 0; c < 4 * NI; ++c) {
-    const int j = jw + 16 * (c / 4) + (c & 3);
-    if (j >= n_rec) continue;
-    const float4 nb = __ldg(consts + 2 * j), mk = __ldg(consts + 2 * j + 1);  // {n, n lo, b, b lo}, {mask, ...}
-    if (mk.x == 0.f) continue;
+  for (int i = 0; i < NI; ++i) {
+    dfloat d[4 * MI];
+    bool inf[4 * MI];
 #pragma unroll
     for (int r = 0; r < 4 * MI; ++r) {
-      const float2 s2 = unpk(sum[r][c / 2]), c2 = unpk(comp[r][c / 2]);
-      const dfloat dev = two_sum((c & 1) ? s2.y : s2.x, (c & 1) ? -c2.y : -c2.x);
-      dfloat t;
-      if (!poisson_term_df(df_add(dev, dfloat{nb.z, nb.w}), dfloat{nb.x, nb.y}, &t)) {
-        const double x = poisson_term_f64(((double)dev.hi + (double)dev.lo) + b64[j], n64[j]);
-        t = isfinite(x) ? df_from_double(x) : dfloat{(float)x, 0.f};
+      d[r] = {0.f, 0.f};
+      inf[r] = false;
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int j = jw + 16 * i + c;
+      if (j >= n_rec) continue;
+      const float4 nb = __ldg(consts + 2 * j), mk = __ldg(consts + 2 * j + 1);  // {n, n lo, b, b lo}, {mask, ...}
+      if (mk.x == 0.f) continue;
+#pragma unroll
+      for (int r = 0; r < 4 * MI; ++r) {
+        const float2 s2 = unpk(sum[r][2 * i + c / 2]), c2 = unpk(comp[r][2 * i + c / 2]);
+        const dfloat dev = two_sum((c & 1) ? s2.y : s2.x, (c & 1) ? -c2.y : -c2.x);
+        dfloat t;
+        if (!poisson_term_df(df_add(dev, dfloat{nb.z, nb.w}), dfloat{nb.x, nb.y}, &t)) {
+          const double x = poisson_term_f64(((double)dev.hi + (double)dev.lo) + b64[j], n64[j]);
+          t = isfinite(x) ? df_from_double(x) : dfloat{(float)x, 0.f};
+        }
+        if (isinf(t.hi)) inf[r] = true;
+        else d[r] = df_add(d[r], t);
       }
-      if (isinf(t.hi)) inf[r] = true;
-      else d[r] = df_add(d[r], t);
+    }
+#pragma unroll
+    for (int r = 0; r < 4 * MI; ++r) {
+#pragma unroll
+      for (int o = 1; o <= 2; o <<= 1) {
+        d[r] = df_add(d[r], df_shfl_xor(d[r], o));
+        inf[r] = __shfl_xor_sync(0xffffffffu, (int)inf[r], o) || inf[r];
+      }
+      if (ln == 0) {
+        const int q = (r / 4) * 32 + lm * 4 + (r & 3);
+        psum[warp * NI + i][q] = make_float2(d[r].hi, d[r].lo);
+        pinf[warp * NI + i][q] = inf[r];
+      }
     }
   }
-  // the ring is free (its last copies landed above): the warps' sums per point
-  float2(*psum)[BM] = reinterpret_cast<float2(*)[BM]>(&ring[0][0][0]);
-  int(*pinf)[BM] = reinterpret_cast<int(*)[BM]>(&ring[1][0][0]);
-  static_assert(sizeof(float2) * 4 * BM <= sizeof(ring[0]), "sums of four warps in a ring slot");
   __syncthreads();
+  for (int x = tid; x < NI * BM; x += THR) {
+    const int q = x % BM, u = x / BM;  // 64 bins from j0 + 64 u on
+    if (m0 + q >= P || j0 + 64 * u >= n_rec) continue;
+    double s = 0.0;
+    bool any = false;
 #pragma unroll
-  for (int r = 0; r < 4 * MI; ++r) {
-#pragma unroll
-    for (int o = 1; o <= 2; o <<= 1) {
-      d[r] = df_add(d[r], df_shfl_xor(d[r], o));
-      inf[r] = __shfl_xor_sync(0xffffffffu, (int)inf[r], o) || inf[r];
+    for (int w = 0; w < 4; ++w) {
+      s += (double)psum[4 * u + w][q].x + (double)psum[4 * u + w][q].y;
+      any |= pinf[4 * u + w][q] != 0;
     }
-    if (ln == 0) {
-      const int q = (r / 4) * 32 + lm * 4 + (r & 3);
-      psum[warp][q] = make_float2(d[r].hi, d[r].lo);
-      pinf[warp][q] = inf[r];
-    }
+    parts[(size_t)(od.z * NI + u) * P + m0 + q] = any ? __longlong_as_double(0x7ff0000000000000LL) : s;
   }
-  __syncthreads();
-  for (int q = tid; q < BM; q += THR)
-    if (m0 + q < P) {
-      double s = 0.0;
-      bool any = false;
-      for (int w = 0; w < 4; ++w) {
-        s += (double)psum[w][q].x + (double)psum[w][q].y;
-        any |= pinf[w][q] != 0;
-      }
-      parts[(size_t)od.z * P + m0 + q] = any ? __longlong_as_double(0x7ff0000000000000LL) : s;
-    }
 }
 
 // Rt[tile][k][128] from the row-major R (zero beyond n_rec), and shk[k][16].
@@ -342,48 +355,44 @@ bool small_tile(const srw_ctx* h, int P) {
 
 }  // namespace
 
-int fold_simt_parts(const srw_ctx* h, int P) {
-  const int bn = small_tile(h, P) ? 64 : 128;
-  return (h->n_rec + bn - 1) / bn;
-}
+int fold_simt_parts(int n_rec) { return (n_rec + 63) / 64; }
 
 cudaError_t launch_fold_simt(const srw_ctx* h, const float* theta, int P, double* parts, cudaStream_t s,
                              int* n_parts, float* musig_out) {
   if (small_tile(h, P)) launch_shape<1, 1>(h, theta, P, parts, s, musig_out, h->d_simt_kr + (h->n_rec + 127) / 128);
   else launch_shape<2, 2>(h, theta, P, parts, s, musig_out, h->d_simt_kr);
-  if (n_parts) *n_parts = fold_simt_parts(h, P);
+  if (n_parts) *n_parts = fold_simt_parts(h->n_rec);
   return launch_result();
 }
 
-// Per rec tile of 128 and of 64 bins the K tiles [first, end) between its
-// first and last nonzero column of R (FP32, exact zeros outside; a tile
-// without any nonzero element gets an empty range), longest first; and the
-// kernel's copies of R and of the coefficient spectra.
+// Per 128 rec bins the K tiles [first, end) between their first and last
+// nonzero column of R (FP32, exact zeros outside; an empty range without any
+// nonzero element), for the 128-bin and then for the 64-bin tiles, longest
+// first; and the kernel's copies of R and of the coefficient spectra.
 cudaError_t simt_prepare(srw_ctx* h, const std::vector<float>& R, cudaStream_t s) {
   const int n_kt = h->k_pad / BK, cols = std::min(h->ld_r, h->k_pad);
   std::vector<int4> kr;
-  for (int bn = 128; bn >= 64; bn -= 64) {
-    const size_t first_of = kr.size();
-    for (int t = 0; t * bn < h->n_rec; ++t) {
-      int first = cols, last = -1;
-      for (int j = t * bn; j < std::min(h->n_rec, (t + 1) * bn); ++j) {
-        const float* row = R.data() + (size_t)j * h->ld_r;
-        for (int k = 0; k < first; ++k)
-          if (row[k] != 0.f) {
-            first = k;
-            break;
-          }
-        for (int k = cols - 1; k > last; --k)
-          if (row[k] != 0.f) {
-            last = k;
-            break;
-          }
-      }
-      kr.push_back(last < 0 ? make_int4(0, 0, t, 0) : make_int4(first / BK, std::min(n_kt, last / BK + 1), t, 0));
+  for (int t = 0; t * 128 < h->n_rec; ++t) {
+    int first = cols, last = -1;
+    for (int j = t * 128; j < std::min(h->n_rec, (t + 1) * 128); ++j) {
+      const float* row = R.data() + (size_t)j * h->ld_r;
+      for (int k = 0; k < first; ++k)
+        if (row[k] != 0.f) {
+          first = k;
+          break;
+        }
+      for (int k = cols - 1; k > last; --k)
+        if (row[k] != 0.f) {
+          last = k;
+          break;
+        }
     }
-    std::stable_sort(kr.begin() + first_of, kr.end(),
-                     [](const int4& a, const int4& b) { return a.y - a.x > b.y - b.x; });
+    kr.push_back(last < 0 ? make_int4(0, 0, t, 0) : make_int4(first / BK, std::min(n_kt, last / BK + 1), t, 0));
   }
+  std::stable_sort(kr.begin(), kr.end(), [](const int4& a, const int4& b) { return a.y - a.x > b.y - b.x; });
+  for (size_t q = 0, n128 = kr.size(); q < n128; ++q)
+    for (int t = 2 * kr[q].z; t < 2 * kr[q].z + 2; ++t)
+      if (t * 64 < h->n_rec) kr.push_back(make_int4(kr[q].x, kr[q].y, t, 0));
   const int nt = (h->n_rec + kTile - 1) / kTile;
   const size_t bytes[3] = {sizeof(int4) * kr.size(), sizeof(float) * (size_t)nt * kTile * h->k_pad,
                            sizeof(float) * 16 * (size_t)h->k_pad};

@@ -268,7 +268,7 @@ srw_status build_simt(srw_group g) {
   std::vector<GroupPart> gp(g->n);
   long long off = 0;
   for (int i = 0; i < g->n; ++i) {
-    const int np = srw::fold_simt_parts(g->hs[i], g->P[i]);
+    const int np = srw::fold_simt_parts(g->hs[i]->n_rec);
     gp[i] = GroupPart{off, np, g->P[i], g->p_off[i], 0, g->hs[i]->d_cdata};
     off += (long long)np * g->P[i];
   }

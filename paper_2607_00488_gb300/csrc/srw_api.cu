@@ -992,7 +992,7 @@ static srw_status loglik_impl(srw_handle h, const float* theta, int P, double* o
       if (e == cudaSuccess) e = cudaEventRecord(h->ev_fold[1], s);
       if (e != cudaSuccess) return cuda_fail(h, e, "profiled single-point fold");
     } else {
-      const int n_parts_max = precision == SRW_FP32 ? fold_simt_parts(h, P) : (h->rec_pad / 128);
+      const int n_parts_max = precision == SRW_FP32 ? fold_simt_parts(h->n_rec) : (h->rec_pad / 128);
       st = ensure_bparts(h, (size_t)n_parts_max * P);
       if (st == SRW_OK && precision != SRW_FP32) st = ensure_coef(h, P);
       if (st != SRW_OK) return st;
@@ -1019,7 +1019,7 @@ static srw_status loglik_impl(srw_handle h, const float* theta, int P, double* o
       return launch_fold_point_after(h, h->d_W, nullptr, nullptr, o, cs, true);
     });
   } else {
-    const int n_parts_max = precision == SRW_FP32 ? fold_simt_parts(h, P) : (h->rec_pad / 128);
+    const int n_parts_max = precision == SRW_FP32 ? fold_simt_parts(h->n_rec) : (h->rec_pad / 128);
     st = ensure_bparts(h, (size_t)n_parts_max * P);
     if (st == SRW_OK && precision != SRW_FP32) st = ensure_coef(h, P);
     if (st != SRW_OK) return st;

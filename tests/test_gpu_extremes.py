@@ -108,3 +108,18 @@ def test_fp32_batch_tiny_count_is_data(srw, n):
         lk.loglik(theta, srw.SRW_FP32, out=out)
         torch.cuda.synchronize()
         assert np.all(np.isposinf(out.cpu().numpy()))
+
+
+# FP32 products: the tile that a batch gets depends on its size, the value of a
+# point does not.
+@pytest.mark.parametrize("n_t,n_rec,p", [(100, 64, 9800), (64, 129, 4900), (260, 200, 4900), (33, 1111, 1200),
+                                         (300, 2050, 640)])
+def test_fp32_value_independent_of_the_batch(srw, n_t, n_rec, p):
+    wl = line(n_t, n_rec)
+    _, counts = oracle_of(wl)
+    theta = workloads.theta_box(p, 11)
+    with srw.Likelihood(wl, counts) as lk:
+        want, spec = lk.loglik(theta, srw.SRW_FP32), lk.spectrum_batch(theta, srw.SRW_FP32)
+        for k in (2, 31, 33, 65, 300):
+            np.testing.assert_array_equal(lk.loglik(theta[:k], srw.SRW_FP32), want[:k])
+            np.testing.assert_array_equal(lk.spectrum_batch(theta[:k], srw.SRW_FP32), spec[:k])
