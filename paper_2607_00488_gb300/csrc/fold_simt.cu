@@ -311,10 +311,11 @@ fold_simt_kernel(const float* __restrict__ theta, int P, dfloat sin2w, CoefRef c
 }
 
 // Rt[tile][k][128] from the row-major R (zero beyond n_rec), and shk[k][16].
+// One block per 32 x 32 elements in one grid dimension (the others end at 65,535).
 __global__ void simt_layout_kernel(const float* __restrict__ R, int n_rec, int ld, int k_pad,
                                    float* __restrict__ Rt) {
   __shared__ float s[32][33];
-  const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32;  // 32 true bins x 32 rec bins
+  const int k0 = (int)(blockIdx.x % (k_pad / 32)) * 32, r0 = (int)(blockIdx.x / (k_pad / 32)) * 32;
   for (int i = threadIdx.y; i < 32; i += 8) {
     const int j = r0 + i, k = k0 + threadIdx.x;
     s[i][threadIdx.x] = j < n_rec && k < ld ? R[(size_t)j * ld + k] : 0.f;
@@ -401,8 +402,8 @@ cudaError_t simt_prepare(srw_ctx* h, const std::vector<float>& R, cudaStream_t s
   if (!h->d_simt_r && (e = dev_malloc(&h->d_simt_r, bytes[1])) != cudaSuccess) return e;
   if (!h->d_simt_sh && (e = dev_malloc(&h->d_simt_sh, bytes[2])) != cudaSuccess) return e;
   h->device_bytes += bytes[0] + bytes[1] + bytes[2];
-  simt_layout_kernel<<<dim3(h->k_pad / 32, nt * (kTile / 32)), dim3(32, 8), 0, s>>>(h->d_R, h->n_rec, h->ld_r,
-                                                                                    h->k_pad, h->d_simt_r);
+  simt_layout_kernel<<<(unsigned)nt * (kTile / 32) * (h->k_pad / 32), dim3(32, 8), 0, s>>>(h->d_R, h->n_rec, h->ld_r,
+                                                                                           h->k_pad, h->d_simt_r);
   simt_spectra_kernel<<<(h->k_pad + 255) / 256, 256, 0, s>>>(h->d_shat, h->d_shat_lo, h->k_pad, h->d_simt_sh);
   if ((e = launch_result()) != cudaSuccess) return e;
   return cudaMemcpyAsync(h->d_simt_kr, kr.data(), bytes[0], cudaMemcpyHostToDevice, s) == cudaSuccess

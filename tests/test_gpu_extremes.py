@@ -123,3 +123,26 @@ def test_fp32_value_independent_of_the_batch(srw, n_t, n_rec, p):
         for k in (2, 31, 33, 65, 300):
             np.testing.assert_array_equal(lk.loglik(theta[:k], srw.SRW_FP32), want[:k])
             np.testing.assert_array_equal(lk.spectrum_batch(theta[:k], srw.SRW_FP32), spec[:k])
+
+
+# Two million reconstructed bins: more rows than a grid's y dimension holds in tiles of 32.
+def test_fp32_batch_with_very_many_bins(srw):
+    from scipy.special import gammaln, xlogy
+    n_rec, n_t = 2100001, 2
+    rng = np.random.default_rng(1)
+    r = rng.uniform(0.5, 1.5, (n_rec, n_t)).astype(np.float32) / np.float32(n_rec)
+    wl = line(n_t, 8)
+    wl.update(R=r[:8], e_true_sm=np.full(n_t, 1.0e6))
+    m = O.OracleModel.from_workload(wl, e_true_sm=wl["e_true_sm"])  # spectra only: the fold is one product here
+    bkg = rng.uniform(0.5, 1.0, (1, n_rec))
+    ref = r.astype(np.float64) @ m.weighted_true(np.zeros(5)) + bkg[0]
+    counts = rng.poisson(ref).astype(np.float64)
+    wl.update(R=r, rec_edges=np.linspace(0.0, 1.3, n_rec + 1), bkg=bkg)
+    theta = workloads.fit_region_points(2, seed=3)
+    with srw.Likelihood(wl, counts, e_true_sm=wl["e_true_sm"]) as lk:
+        got = lk.loglik(theta, srw.SRW_FP32)
+    for t, v in zip(theta, got):
+        mu = r.astype(np.float64) @ m.weighted_true(t.astype(np.float64)) + bkg[0]
+        want = 2.0 * np.sum(mu - xlogy(counts, mu) + gammaln(counts + 1.0))
+        # FP32 products of R with the deviation from the reference: 2^-23 of each
+        assert abs(v - want) <= 2.0 * np.sum(np.abs(1.0 - counts / mu) * np.abs(mu - ref)) * 2.0**-23
