@@ -369,7 +369,7 @@ cudaError_t launch_fold_simt(const srw_ctx* h, const float* theta, int P, double
 // Per 128 rec bins the K tiles [first, end) between their first and last
 // nonzero column of R (FP32, exact zeros outside; an empty range without any
 // nonzero element), for the 128-bin and then for the 64-bin tiles, longest
-// first; and the kernel's copies of R and of the coefficient spectra.
+// first; and the copies of simt_ready.
 cudaError_t simt_prepare(srw_ctx* h, const std::vector<float>& R, cudaStream_t s) {
   const int n_kt = h->k_pad / BK, cols = std::min(h->ld_r, h->k_pad);
   std::vector<int4> kr;
@@ -394,21 +394,44 @@ cudaError_t simt_prepare(srw_ctx* h, const std::vector<float>& R, cudaStream_t s
   for (size_t q = 0, n128 = kr.size(); q < n128; ++q)
     for (int t = 2 * kr[q].z; t < 2 * kr[q].z + 2; ++t)
       if (t * 64 < h->n_rec) kr.push_back(make_int4(kr[q].x, kr[q].y, t, 0));
-  const int nt = (h->n_rec + kTile - 1) / kTile;
-  const size_t bytes[3] = {sizeof(int4) * kr.size(), sizeof(float) * (size_t)nt * kTile * h->k_pad,
-                           sizeof(float) * 16 * (size_t)h->k_pad};
   cudaError_t e = cudaSuccess;
-  if (!h->d_simt_kr && (e = dev_malloc(&h->d_simt_kr, bytes[0])) != cudaSuccess) return e;
-  if (!h->d_simt_r && (e = dev_malloc(&h->d_simt_r, bytes[1])) != cudaSuccess) return e;
-  if (!h->d_simt_sh && (e = dev_malloc(&h->d_simt_sh, bytes[2])) != cudaSuccess) return e;
-  h->device_bytes += bytes[0] + bytes[1] + bytes[2];
-  simt_layout_kernel<<<(unsigned)nt * (kTile / 32) * (h->k_pad / 32), dim3(32, 8), 0, s>>>(h->d_R, h->n_rec, h->ld_r,
-                                                                                           h->k_pad, h->d_simt_r);
-  simt_spectra_kernel<<<(h->k_pad + 255) / 256, 256, 0, s>>>(h->d_shat, h->d_shat_lo, h->k_pad, h->d_simt_sh);
-  if ((e = launch_result()) != cudaSuccess) return e;
-  return cudaMemcpyAsync(h->d_simt_kr, kr.data(), bytes[0], cudaMemcpyHostToDevice, s) == cudaSuccess
-             ? cudaStreamSynchronize(s)
-             : cudaErrorUnknown;
+  if (!h->d_simt_kr && (e = dev_malloc(&h->d_simt_kr, sizeof(int4) * kr.size())) != cudaSuccess) return e;
+  h->device_bytes += sizeof(int4) * kr.size();
+  e = cudaMemcpyAsync(h->d_simt_kr, kr.data(), sizeof(int4) * kr.size(), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return e;
+  e = simt_ready(h);
+  return e == cudaErrorMemoryAllocation ? cudaSuccess : e;  // only the FP32 batch reads the copies: it tries again
+}
+
+// The kernel's copies of R (as large as R) and of the coefficient spectra,
+// made with the handle, or by the first FP32 batch where there was no room.
+cudaError_t simt_ready(srw_ctx* h) {
+  if (h->d_simt_r && h->d_simt_sh) return cudaSuccess;
+  const int nt = (h->n_rec + kTile - 1) / kTile;
+  const size_t bytes[2] = {sizeof(float) * (size_t)nt * kTile * h->k_pad, sizeof(float) * 16 * (size_t)h->k_pad};
+  cudaStream_t s = h->own_stream;
+  float *r = nullptr, *sh = nullptr;
+  cudaError_t e = dev_malloc(&sh, bytes[1]);
+  if (e == cudaSuccess) e = dev_malloc(&r, bytes[0]);
+  if (e == cudaSuccess) {
+    simt_layout_kernel<<<(unsigned)nt * (kTile / 32) * (h->k_pad / 32), dim3(32, 8), 0, s>>>(h->d_R, h->n_rec, h->ld_r,
+                                                                                             h->k_pad, r);
+    simt_spectra_kernel<<<(h->k_pad + 255) / 256, 256, 0, s>>>(h->d_shat, h->d_shat_lo, h->k_pad, sh);
+    e = launch_result();
+    const cudaError_t es = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = es;
+  }
+  if (e != cudaSuccess) {
+    if (r) cudaFree(r);
+    if (sh) cudaFree(sh);
+    cudaGetLastError();  // a failed allocation is not the next launch's error
+    return e;
+  }
+  h->d_simt_r = r;
+  h->d_simt_sh = sh;
+  h->device_bytes += bytes[0] + bytes[1];
+  return cudaSuccess;
 }
 
 }  // namespace srw

@@ -297,6 +297,7 @@ srw_status run(srw_group g, const float* th, double* o, int precision, cudaStrea
     }
     srw_status st = ensure_parts(g, g->simt_parts);
     if (st != SRW_OK) return st;
+    for (int i = 0; i < g->n; ++i) G_CUDA(g, srw::simt_ready(g->hs[i]), "FP32 fold layout");
     size_t off = 0;
     for (int i = 0; i < g->n; ++i) {
       if (g->P[i] == 0) continue;

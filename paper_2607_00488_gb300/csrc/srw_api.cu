@@ -996,6 +996,7 @@ static srw_status loglik_impl(srw_handle h, const float* theta, int P, double* o
       st = ensure_bparts(h, (size_t)n_parts_max * P);
       if (st == SRW_OK && precision != SRW_FP32) st = ensure_coef(h, P);
       if (st != SRW_OK) return st;
+      if (precision == SRW_FP32) SRW_CUDA(h, simt_ready(h), "FP32 fold layout");
       int n_parts = 0;
       cudaError_t e = cudaSuccess;
       if (precision == SRW_FP32) {
@@ -1023,6 +1024,7 @@ static srw_status loglik_impl(srw_handle h, const float* theta, int P, double* o
     st = ensure_bparts(h, (size_t)n_parts_max * P);
     if (st == SRW_OK && precision != SRW_FP32) st = ensure_coef(h, P);
     if (st != SRW_OK) return st;
+    if (precision == SRW_FP32) SRW_CUDA(h, simt_ready(h), "FP32 fold layout");
     const FoldConfig cfg = h->cfg[precision];
     st = run_graph(h, 2, precision, P, th, o, s, [&](cudaStream_t cs) {
       int n_parts = 0;
@@ -1171,6 +1173,8 @@ srw_status srw_spectrum_batch(srw_handle h, const float* theta, int P, float* ou
   if (precision != SRW_FP32) {
     srw_status st = ensure_coef(h, P);
     if (st != SRW_OK) return st;
+  } else {
+    SRW_CUDA(h, simt_ready(h), "FP32 fold layout");
   }
   if (where == SRW_HOST) {
     if (!all_finite(theta, (size_t)P * 5)) return fail(h, SRW_EINVAL, "theta must be finite");

@@ -321,6 +321,7 @@ inline bool all_finite(const float* x, size_t n) {
 
 cudaError_t gemv_prepare(srw_ctx* h, const std::vector<float>& R);
 cudaError_t simt_prepare(srw_ctx* h, const std::vector<float>& R, cudaStream_t s);
+cudaError_t simt_ready(srw_ctx* h);  // before an FP32 batch (outside a capture)
 void fold_point_init();
 int fold_simt_parts(int n_rec);  // partial sums per point
 cudaError_t launch_fold_point(const srw_ctx* h, const float* W, float* musig_out, float* mu_out, double* out,

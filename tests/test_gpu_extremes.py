@@ -125,6 +125,32 @@ def test_fp32_value_independent_of_the_batch(srw, n_t, n_rec, p):
             np.testing.assert_array_equal(lk.spectrum_batch(theta[:k], srw.SRW_FP32), spec[:k])
 
 
+# No room for the FP32 batch's copy of R: the handle is made all the same, and the
+# batch makes the copy when it is called.
+def test_create_without_room_for_the_fp32_copy(srw):
+    wl = line(64, 130)
+    m, counts = oracle_of(wl)
+    theta = workloads.fit_region_points(4, seed=7)
+    want = m.neg2lnl_batch(theta.astype(np.float64))
+    made = 0
+    for skip in range(100):
+        srw.srw_fault_inject("alloc", skip)
+        try:
+            lk = srw.Likelihood(wl)
+        except srw.SrwError as e:
+            assert e.status == 2  # SRW_ENOMEM
+            continue
+        fired = srw.srw_fault_pending() == 0
+        srw.srw_fault_inject("none")
+        srw.srw_set_data(lk.handle, counts, wl["bkg"])
+        assert np.max(np.abs(lk.loglik(theta, srw.SRW_FP32) - want)) <= 1e-4
+        lk.close()
+        if not fired:  # past the last allocation
+            break
+        made += 1
+    assert made == 2  # either of the two copies
+
+
 # Two million reconstructed bins: more rows than a grid's y dimension holds in tiles of 32.
 def test_fp32_batch_with_very_many_bins(srw):
     from scipy.special import gammaln, xlogy
