@@ -153,9 +153,20 @@ static cudaStream_t pick_stream(srw_ctx* h, void* stream) {
   return stream ? (cudaStream_t)stream : h->own_stream;
 }
 
+constexpr size_t kPinned = 256 * 1024;  // bytes for uploads, as much for downloads
+
 // Grows the staging buffers for host-pointer calls; invalidates graphs that
-// referenced the old buffers.
+// referenced the old buffers.  The pinned buffer comes with the first such call
+// (a handle used with device pointers, or in a group of thousands, needs none);
+// without it copies go straight to the caller's memory.
 static srw_status ensure_staging(srw_ctx* h, int P) {
+  if (!h->pinned && !h->pinned_tried) {
+    h->pinned_tried = true;
+    if (cudaMallocHost(&h->pinned, 2 * kPinned) != cudaSuccess) {
+      cudaGetLastError();
+      h->pinned = nullptr;
+    }
+  }
   if (P <= h->stage_cap && h->d_theta && h->d_out) return SRW_OK;
   int cap = std::max(P, 2 * h->stage_cap);
   destroy_graphs(h);
@@ -198,13 +209,13 @@ static srw_status ensure_bparts(srw_ctx* h, size_t n) {
   return SRW_OK;
 }
 
-// Host-pointer calls copy through a pinned buffer of the handle where it holds
-// the arrays: a copy from or to pageable memory is staged by the driver, and a
-// download waits for the stream each time.  One point on a line's 128 bins,
-// value and status word: 42.9 -> 36.9 us a call; 8191 profiled points 556 -> 553
-// us.  Larger arrays go straight to the caller's memory.  A call ends with a synchronise
-// before the buffer is used again.
-constexpr size_t kPinned = 256 * 1024;  // bytes for uploads, as much for downloads
+// Host-pointer calls of srw_loglik, srw_loglik_points, srw_loglik_linear (points
+// and values) and srw_loglik_profiled copy through a pinned buffer of the handle
+// where it holds the arrays: a copy from or to pageable memory is staged by the
+// driver, and a download waits for the stream each time.  One point on a line's
+// 128 bins, value and status word: 42.9 -> 36.9 us a call; 8191 profiled points
+// 556 -> 553 us.  Larger arrays go straight to the caller's memory.  A call ends
+// with a synchronise before the buffer is used again.
 
 struct Downloads {
   int n = 0;
@@ -735,10 +746,6 @@ static srw_status create_impl(const srw_binning* bin, const srw_source* sources,
   CREATE_CUDA(cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking), "stream create");
   cudaStream_t s = h->own_stream;
   fold_point_init();
-  if (cudaMallocHost(&h->pinned, 2 * kPinned) != cudaSuccess) {  // copies then go straight to the caller's memory
-    cudaGetLastError();
-    h->pinned = nullptr;
-  }
 
   if (!jr) {
     CREATE_CUDA(upload_tables(h, bin, sources, n_sources, s), "node tables");

@@ -162,6 +162,7 @@ struct srw_ctx {
   int2* d_bin_n = nullptr;
   double2* d_bin_q = nullptr;
   unsigned char* pinned = nullptr;  // host: uploads, then status word and downloads of host-pointer calls
+  bool pinned_tried = false;
   double* d_spec = nullptr;  // workspace of the single-point spectrum: chunk totals, prefix sums, clipped terms
   double* d_bin64 = nullptr;
   double* d_basis = nullptr;   // [8][n_t] FP64 coefficient spectra

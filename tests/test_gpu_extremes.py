@@ -151,6 +151,30 @@ def test_create_without_room_for_the_fp32_copy(srw):
     assert made == 2  # either of the two copies
 
 
+# Page-locked host memory serves host-pointer calls: handles that make none hold none.
+def test_handles_pin_no_host_memory_before_a_host_call(srw):
+    def shared_kb():
+        with open("/proc/self/status") as f:
+            return sum(int(x.split()[1]) for x in f if x.startswith("RssShmem"))
+
+    wl = line(64, 130)
+    _, counts = oracle_of(wl)
+    theta = torch.zeros((1, 5), device="cuda")
+    first = srw.Likelihood(wl, counts)  # whatever the process maps once
+    first.loglik(theta, out=torch.zeros(1, dtype=torch.float64, device="cuda"))
+    before = shared_kb()
+    rest = [srw.Likelihood(wl, counts) for _ in range(32)]
+    out = torch.zeros(1, dtype=torch.float64, device="cuda")
+    for lk in rest:
+        lk.loglik(theta, out=out)
+    assert shared_kb() - before < 32 * 64
+    want = first.loglik(np.zeros((1, 5), np.float32))
+    for lk in rest:
+        np.testing.assert_array_equal(lk.loglik(np.zeros((1, 5), np.float32)), want)
+        lk.close()
+    first.close()
+
+
 # Two million reconstructed bins: more rows than a grid's y dimension holds in tiles of 32.
 def test_fp32_batch_with_very_many_bins(srw):
     from scipy.special import gammaln, xlogy
