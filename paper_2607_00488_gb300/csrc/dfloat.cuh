@@ -59,6 +59,19 @@ __device__ __forceinline__ dfloat df_warp_sum(dfloat v) {
   return v;
 }
 
+// Three floats, about 72 bits: a running sum that keeps more than FP64 would
+// without its instructions.
+struct tfloat {
+  float a, b, c;
+};
+
+__device__ __forceinline__ tfloat tf_add(tfloat t, dfloat x) {
+  const dfloat s = two_sum(t.a, x.hi), u = two_sum(t.b, x.lo), v = two_sum(u.hi, s.lo);
+  const dfloat p = fast_two_sum(s.hi, v.hi), q = fast_two_sum(p.lo, t.c + (u.lo + v.lo));
+  return {p.hi, q.hi, q.lo};
+}
+__device__ __forceinline__ double tf_double(tfloat t) { return (double)t.a + ((double)t.b + (double)t.c); }
+
 // Split a double into hi + lo floats (host or device).
 __host__ __device__ __forceinline__ dfloat df_from_double(double x) {
   const float hi = (float)x;

@@ -79,7 +79,7 @@ struct EpiArgs {
   double* loss;          // fit: += sum of squared errors
   // scan: per tile of 128 bins the rows m_j + s_j b_j, s_j, -n_j and n_j ln n_j - n_j (masked bins: 0, 0, 0, -1)
   const float* binc;
-  double* parts;         // scan: partial sums of the deviance (mlp_scan_kernel)
+  double* parts;         // scan: partial sums of the deviance, or its parts (mlp_scan_kernel)
 };
 
 // What one training step differs in from the next (device memory, written by
@@ -371,16 +371,24 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 // Here a CTA keeps the activations of 256 points (128 KB) and streams the
 // weights and the bins' constants past them, 128 bins at a time; a lane owns
 // two points, so the constants serve both, and takes two bins at a time in
-// packed FP32; sixteen warps take a quarter of the lanes and of the bins each,
-// and the sums stay in registers over all of the CTA's bins.
+// packed FP32; sixteen warps take a quarter of the lanes and of the bins each.
 //
 // Unit: 256 points x the bins of one of `groups` equal parts (more parts for
-// small batches).  Partial sums: parts[group * 4 + quarter of the bins][row].
+// small batches).  A point's value does not depend on the cut: FP32 sums over 16
+// bins are added up in double-float over runs of kScanRun tiles (128 bins a
+// warp), the runs of a quarter of the bins in three floats (FP64 there cost
+// latency: 2^20 points took 1828 us, so 1763), then the four quarters in FP64.
+// One unit of all bins (`groups` = 1) writes the quarters' sums,
+// parts[quarter][row] (FP64); several units write the runs',
+// parts[run * 4 + quarter][row] (two floats), or, where they do not hold whole
+// runs (RAW), the FP32 sums, parts[(tile * 4 + quarter) * 2 + half][row], and
+// the reduction adds those up in the same order.
 constexpr int kScanWarps = 16;
 constexpr int kScanThreads = (2 + kScanWarps) * 32;
 constexpr int kScanRows = 2 * kBM, kScanBins = 128, kScanKb = kHidden / kBK, kScanRing = 5;
 constexpr int kScanTile = kBM * kBK * 2;  // bytes of a 128 x 64 operand tile
 constexpr int kScanConsts = 4 * kScanBins * 4;  // bytes of a tile's constants, see EpiArgs::binc
+constexpr int kScanRun = 4;
 constexpr int kScanSmem = (2 * kScanKb + kScanRing) * kScanTile + 2 * kScanConsts + 1024;
 
 // Two bins' terms exp(lm) + w - n lm with lm = x + y v (nz = -n); exp as
@@ -394,6 +402,7 @@ __device__ __forceinline__ float2 scan_terms(uint64_t v, uint64_t x, uint64_t y,
   return unpk(fma2(nz, lm, add2(pk(a, b), w)));
 }
 
+template <bool RAW>
 __global__ void __launch_bounds__(kScanThreads, 1)
 mlp_scan_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M, int N,
                 int groups, const EpiArgs E, unsigned* status) {
@@ -529,7 +538,8 @@ mlp_scan_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     int tc = 0;
     bool ok = true;
     for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-      const int m = (u / groups) * kScanRows + q * 32 + lane, n0 = (u % groups) * tiles * kScanBins;
+      const int m = (u / groups) * kScanRows + q * 32 + lane, t0 = (u % groups) * tiles;
+      tfloat total[2] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
       dfloat dev[2] = {{0.f, 0.f}, {0.f, 0.f}};
       bool infinite[2] = {false, false};
       for (int t = 0; t < tiles; ++t, ++tc) {
@@ -562,8 +572,15 @@ mlp_scan_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           }
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            if (isinf(ts[h])) infinite[h] = true;
-            else dev[h] = df_add(dev[h], ts[h]);
+            if (RAW) {
+              if (m + h * kBM < E.rows_valid)
+                reinterpret_cast<float*>(E.parts)[(size_t)(((t0 + t) * 4 + part) * 2 + c0 / 16) * E.rows_valid + m +
+                                                  h * kBM] = ts[h];
+            } else if (isinf(ts[h])) {
+              infinite[h] = true;
+            } else {
+              dev[h] = df_add(dev[h], ts[h]);
+            }
           }
         }
         tc_fence_before();
@@ -572,13 +589,31 @@ mlp_scan_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           ptx::mbar_arrive(&acc_empty[buf]);
           ptx::mbar_arrive(&c_empty[buf]);
         }
+        if constexpr (!RAW) {
+          if ((t + 1) % kScanRun != 0 && t + 1 != tiles) continue;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {  // a run's end
+            if (groups > 1) {
+              if (m + h * kBM < E.rows_valid)
+                reinterpret_cast<float2*>(
+                    E.parts)[(size_t)((t0 + t) / kScanRun * 4 + part) * E.rows_valid + m + h * kBM] =
+                    infinite[h] ? make_float2(__int_as_float(0x7f800000), 0.f) : make_float2(dev[h].hi, dev[h].lo);
+            } else {
+              total[h] = tf_add(total[h], dev[h]);
+            }
+            dev[h] = {0.f, 0.f};
+          }
+        }
       }
       if (!ok) break;
+      if constexpr (!RAW) {
+        if (groups > 1) continue;
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        if (m + h * kBM < E.rows_valid)
-          E.parts[(size_t)((u % groups) * 4 + part) * E.rows_valid + m + h * kBM] =
-              infinite[h] ? __longlong_as_double(0x7ff0000000000000LL) : (double)dev[h].hi + (double)dev[h].lo;
+        for (int h = 0; h < 2; ++h)
+          if (m + h * kBM < E.rows_valid)
+            E.parts[(size_t)part * E.rows_valid + m + h * kBM] =
+                infinite[h] ? __longlong_as_double(0x7ff0000000000000LL) : tf_double(total[h]);
+      }
     }
   }
 
@@ -817,15 +852,73 @@ __global__ void standardize_kernel(float* __restrict__ t, long long rows, int ld
   }
 }
 
-// -2 ln L = 2 sum of the per-tile deviance partials + the data constant.
+// -2 ln L = 2 sum of the quarters' deviances + the data constant.
 template <class T>
-__global__ void scan_reduce_kernel(const double* __restrict__ parts, int n_parts, int rows,
-                                   const double* __restrict__ c_data, T* __restrict__ out) {
+__device__ __forceinline__ T scan_value(const double* q, const double* c_data) {
+  return (T)(2.0 * (((q[0] + q[1]) + q[2]) + q[3]) + *c_data);
+}
+template <class T>
+__global__ void scan_reduce_kernel(const double* __restrict__ parts, int rows, const double* __restrict__ c_data,
+                                   T* __restrict__ out) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= rows) return;
-  double s = 0.0;
-  for (int t = 0; t < n_parts; ++t) s += parts[(size_t)t * rows + p];
-  out[p] = (T)(2.0 * s + *c_data);
+  double q[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) q[k] = parts[(size_t)k * rows + p];
+  out[p] = scan_value<T>(q, c_data);
+}
+
+// The same from the runs of several units (RAW: from their FP32 sums): 32
+// points a block, a warp for every quarter of two runs at a time.
+template <bool RAW, class T>
+__global__ void __launch_bounds__(256)
+scan_reduce_runs_kernel(const float* __restrict__ parts, int tiles, int rows, const double* __restrict__ c_data,
+                        T* __restrict__ out) {
+  __shared__ float2 run[2][4][32];  // an infinite run: {inf, 0}
+  __shared__ double quarter[4][32];
+  const int p = blockIdx.x * 32 + threadIdx.x, part = threadIdx.y % 4, half = threadIdx.y / 4;
+  tfloat total = {0.f, 0.f, 0.f};
+  bool infinite = false;
+  for (int first = 0; first < tiles; first += 2 * kScanRun) {
+    const int f = first + half * kScanRun;
+    float2 x = make_float2(0.f, 0.f);
+    if (p < rows && f < tiles) {
+      if (RAW) {
+        float v[2 * kScanRun];
+#pragma unroll
+        for (int k = 0; k < 2 * kScanRun; ++k)
+          v[k] = f + k / 2 < tiles ? parts[(size_t)(((f + k / 2) * 4 + part) * 2 + k % 2) * rows + p] : 0.f;
+        dfloat dev = {0.f, 0.f};
+        bool inf = false;
+#pragma unroll
+        for (int k = 0; k < 2 * kScanRun; ++k)
+          if (f + k / 2 < tiles) {
+            if (isinf(v[k])) inf = true;
+            else dev = df_add(dev, v[k]);
+          }
+        x = inf ? make_float2(__int_as_float(0x7f800000), 0.f) : make_float2(dev.hi, dev.lo);
+      } else {
+        x = reinterpret_cast<const float2*>(parts)[(size_t)(f / kScanRun * 4 + part) * rows + p];
+      }
+    }
+    run[half][part][threadIdx.x] = x;
+    __syncthreads();
+    if (half == 0)  // this quarter's runs in order
+      for (int r = 0; r < 2 && first + r * kScanRun < tiles; ++r) {
+        const float2 y = run[r][part][threadIdx.x];
+        if (isinf(y.x)) infinite = true;
+        else total = tf_add(total, dfloat{y.x, y.y});
+      }
+    __syncthreads();
+  }
+  if (half == 0)
+    quarter[part][threadIdx.x] = infinite ? __longlong_as_double(0x7ff0000000000000LL) : tf_double(total);
+  __syncthreads();
+  if (threadIdx.y == 0 && p < rows) {
+    const double q[4] = {quarter[0][threadIdx.x], quarter[1][threadIdx.x], quarter[2][threadIdx.x],
+                         quarter[3][threadIdx.x]};
+    out[p] = scan_value<T>(q, c_data);
+  }
 }
 
 // Sobol points in Gray-code order (Antonov-Saleev): point i is the xor of the
@@ -1039,13 +1132,21 @@ int scan_groups(int M, int N, int sm_count) {
   while ((long long)(M / kScanRows) * groups < 2LL * sm_count && tiles % (2 * groups) == 0) groups *= 2;
   return groups;
 }
+// Units that do not hold whole runs of tiles write FP32 sums (see mlp_scan_kernel).
+bool scan_raw(int N, int groups) { return groups > 1 && N / kScanBins / groups % kScanRun != 0; }
+// Eight-byte partial sums a point.
+int scan_parts(int N, int groups) {
+  const int tiles = N / kScanBins;
+  return 4 * (groups == 1 ? 1 : scan_raw(N, groups) ? tiles : (tiles + kScanRun - 1) / kScanRun);
+}
 
 cudaError_t run_gemm(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s, bool dep = false) {
   if (g.mode == kWgrad) return launch_mode<64, kWgrad>(g, sm_count, status, s, dep);
   if (g.mode == kFwdScan) {
     const int groups = scan_groups(g.M, g.N, sm_count), units = g.M / kScanRows * groups;
-    mlp_scan_kernel<<<units < sm_count ? units : sm_count, kScanThreads, kScanSmem, s>>>(g.ma, g.mb, g.M, g.N, groups,
-                                                                                        g.E, status);
+    const auto kernel = scan_raw(g.N, groups) ? mlp_scan_kernel<true> : mlp_scan_kernel<false>;
+    kernel<<<units < sm_count ? units : sm_count, kScanThreads, kScanSmem, s>>>(g.ma, g.mb, g.M, g.N, groups, g.E,
+                                                                                status);
     return srw::launch_result();
   }
   return g.bn == 256   ? launch_width<256>(g, sm_count, status, s, dep)
@@ -1069,7 +1170,9 @@ cudaError_t gemm_attrs() {
   if (e == cudaSuccess) e = gemm_attrs_width<64>();
   if (e == cudaSuccess) e = gemm_attr<64, kWgrad>();
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(mlp_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kScanSmem);
+    e = cudaFuncSetAttribute(mlp_scan_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kScanSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(mlp_scan_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kScanSmem);
   return e;
 }
 
@@ -1105,7 +1208,7 @@ struct SurrogateBatch {
   __nv_bfloat16* dy = nullptr;
   __nv_bfloat16* dz[3] = {};
   float* y = nullptr;       // FP32 network output (forward hook)
-  double* parts = nullptr;  // scan partials [4 scan_groups][M]
+  double* parts = nullptr;  // scan partials [scan_parts][M]
   double* loss = nullptr;
   Gemm fwd[4], fwd_out, fwd_scan, wgrad[4], bwd[3];
   cudaGraphExec_t step = nullptr;  // captured training step (after its input kernel)
@@ -1271,7 +1374,8 @@ srw_status get_batch(srw_surrogate s, int M, bool train, SurrogateBatch** out) {
   cudaError_t e = salloc(&B->x, (size_t)M * srw::kInPad);
   for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = salloc(&B->h[k], (size_t)M * H);
   const int bn_h = srw::pick_tile(M, H, s->sm_count), bn_o = srw::pick_tile(M, NO, s->sm_count);
-  if (e == cudaSuccess) e = salloc(&B->parts, (size_t)srw::scan_groups(M, NO, s->sm_count) * 4 * M);
+  const int groups = srw::scan_groups(M, NO, s->sm_count);
+  if (e == cudaSuccess) e = salloc(&B->parts, (size_t)srw::scan_parts(NO, groups) * M);
   if (e == cudaSuccess) e = cudaMemset(B->x, 0, sizeof(__nv_bfloat16) * (size_t)M * srw::kInPad);
   if (e == cudaSuccess) e = salloc(&B->loss, 1);
   if (train) {
@@ -1504,10 +1608,14 @@ srw_status loglik_device(srw_surrogate s, const float* theta, long long P, T* ou
       g.E.rows_valid = rows;
       e = srw::run_gemm(g, s->sm_count, s->d_status, st);
     }
-    const int n_parts = 4 * srw::scan_groups(B->M, s->n_out_pad, s->sm_count);
+    const int NO = s->n_out_pad, groups = srw::scan_groups(B->M, NO, s->sm_count);
     if (e == cudaSuccess) {
-      srw::scan_reduce_kernel<T><<<(rows + 255) / 256, 256, 0, st>>>(B->parts, n_parts, rows, s->h->d_cdata,
-                                                                   out + off);
+      if (groups == 1)
+        srw::scan_reduce_kernel<T><<<(rows + 255) / 256, 256, 0, st>>>(B->parts, rows, s->h->d_cdata, out + off);
+      else
+        (srw::scan_raw(NO, groups) ? srw::scan_reduce_runs_kernel<true, T> : srw::scan_reduce_runs_kernel<false, T>)
+            <<<(rows + 31) / 32, dim3(32, 8), 0, st>>>(reinterpret_cast<const float*>(B->parts), NO / srw::kScanBins,
+                                                        rows, s->h->d_cdata, out + off);
       e = srw::launch_result();
     }
     if (e != cudaSuccess) return scuda(s, e, "surrogate likelihood");

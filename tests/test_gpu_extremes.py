@@ -175,6 +175,24 @@ def test_handles_pin_no_host_memory_before_a_host_call(srw):
     first.close()
 
 
+# Surrogate: a full chunk and a small batch cut the bins into different units.
+@pytest.mark.parametrize("n_rec", [100, 257, 600, 1000, 1300, 2048, 4000])
+def test_surrogate_value_independent_of_the_batch(srw, n_rec):
+    from workloads.mlp import BOX_CENTRE, BOX_HALF, init_weights
+    wl = line(64, n_rec)
+    _, counts = oracle_of(wl)
+    params = init_weights(n_rec, seed=5)
+    # neighbouring bins of one size between exp(-25) and exp(18): the sums of 16 bins round where they are added up
+    bias = np.repeat(np.random.default_rng(n_rec).uniform(-25.0, 18.0, n_rec // 16 + 1), 16)[:n_rec].astype(np.float32)
+    params[-1] = (0.1 * params[-1][0], bias)
+    theta = workloads.theta_box(100000, 43)
+    with srw.Likelihood(wl, counts) as lk, srw.Surrogate(lk, params, BOX_CENTRE, BOX_HALF) as s:
+        v = s.loglik(theta)
+        assert np.all(np.isfinite(v))
+        for p in (1, 257, 3000, 20000, 40000):
+            np.testing.assert_array_equal(s.loglik(theta[:p]), v[:p])
+
+
 # Two million reconstructed bins: more rows than a grid's y dimension holds in tiles of 32.
 def test_fp32_batch_with_very_many_bins(srw):
     from scipy.special import gammaln, xlogy
