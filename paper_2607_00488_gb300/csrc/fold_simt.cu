@@ -87,10 +87,11 @@ __device__ __forceinline__ void coefficients(const float* th, dfloat s, const Co
 // 16-byte copies bring in three K tiles ahead (the row-major R went through
 // registers and was transposed by four 4-byte stores per load).  order: {first
 // and end K tile holding nonzero response, rec tile, 0}, longest range first,
-// so that the last wave holds the short ones.  The range is that of the 128
-// bins around a tile in both shapes, which then add the same terms in the same
-// order (a range per 64 bins, with warps that sit out the rest of the large
-// tile's, cost the large tile 7 %).
+// so that the last wave holds the short ones.  K tiles of zeros more or less
+// (128 bins have a longer range than 64) do not change a bin's value: with a
+// sum x of 0 a step of the Kahan sum sends (s, c) to t = fl(s - c) and
+// (t - s) + c, and as |c| is at most a few units in the last place of s, that
+// difference is exact: t minus the new c is s - c, which is all that is read.
 template <int MI, int NI>
 __global__ void __launch_bounds__(THR, MI * NI == 4 ? 2 : 4)
 fold_simt_kernel(const float* __restrict__ theta, int P, dfloat sin2w, CoefRef cref, const float* __restrict__ shk,
@@ -366,34 +367,35 @@ cudaError_t launch_fold_simt(const srw_ctx* h, const float* theta, int P, double
   return launch_result();
 }
 
-// Per 128 rec bins the K tiles [first, end) between their first and last
-// nonzero column of R (FP32, exact zeros outside; an empty range without any
-// nonzero element), for the 128-bin and then for the 64-bin tiles, longest
-// first; and the copies of simt_ready.
+// Per rec tile of 128 and of 64 bins the K tiles [first, end) between its
+// first and last nonzero column of R (FP32, exact zeros outside; a tile
+// without any nonzero element gets an empty range), longest first; and the
+// copies of simt_ready.
 cudaError_t simt_prepare(srw_ctx* h, const std::vector<float>& R, cudaStream_t s) {
   const int n_kt = h->k_pad / BK, cols = std::min(h->ld_r, h->k_pad);
   std::vector<int4> kr;
-  for (int t = 0; t * 128 < h->n_rec; ++t) {
-    int first = cols, last = -1;
-    for (int j = t * 128; j < std::min(h->n_rec, (t + 1) * 128); ++j) {
-      const float* row = R.data() + (size_t)j * h->ld_r;
-      for (int k = 0; k < first; ++k)
-        if (row[k] != 0.f) {
-          first = k;
-          break;
-        }
-      for (int k = cols - 1; k > last; --k)
-        if (row[k] != 0.f) {
-          last = k;
-          break;
-        }
+  for (int bn = 128; bn >= 64; bn -= 64) {
+    const size_t first_of = kr.size();
+    for (int t = 0; t * bn < h->n_rec; ++t) {
+      int first = cols, last = -1;
+      for (int j = t * bn; j < std::min(h->n_rec, (t + 1) * bn); ++j) {
+        const float* row = R.data() + (size_t)j * h->ld_r;
+        for (int k = 0; k < first; ++k)
+          if (row[k] != 0.f) {
+            first = k;
+            break;
+          }
+        for (int k = cols - 1; k > last; --k)
+          if (row[k] != 0.f) {
+            last = k;
+            break;
+          }
+      }
+      kr.push_back(last < 0 ? make_int4(0, 0, t, 0) : make_int4(first / BK, std::min(n_kt, last / BK + 1), t, 0));
     }
-    kr.push_back(last < 0 ? make_int4(0, 0, t, 0) : make_int4(first / BK, std::min(n_kt, last / BK + 1), t, 0));
+    std::stable_sort(kr.begin() + first_of, kr.end(),
+                     [](const int4& a, const int4& b) { return a.y - a.x > b.y - b.x; });
   }
-  std::stable_sort(kr.begin(), kr.end(), [](const int4& a, const int4& b) { return a.y - a.x > b.y - b.x; });
-  for (size_t q = 0, n128 = kr.size(); q < n128; ++q)
-    for (int t = 2 * kr[q].z; t < 2 * kr[q].z + 2; ++t)
-      if (t * 64 < h->n_rec) kr.push_back(make_int4(kr[q].x, kr[q].y, t, 0));
   cudaError_t e = cudaSuccess;
   if (!h->d_simt_kr && (e = dev_malloc(&h->d_simt_kr, sizeof(int4) * kr.size())) != cudaSuccess) return e;
   h->device_bytes += sizeof(int4) * kr.size();
