@@ -599,12 +599,14 @@ srw_status srw_diag_wait_timeout(unsigned limit_us);
  *   SRW_FAULT_LAUNCH  a kernel-launch check reports a launch failure (the
  *                     call returns SRW_ECUDA; a CUDA graph being captured for
  *                     the call is discarded, never cached);
- *   SRW_FAULT_TIMEOUT a fold launch (single-point GEMV or tensor-core fold)
- *                     makes one wait wait on an mbarrier that nothing arrives
- *                     on, with a 1 ms limit; the wait gives up and the kernel
- *                     takes its abort path: the affected points' values are
- *                     NaN, host-pointer calls return SRW_ETIMEOUT, and a
- *                     graph captured with the fault is run once, not cached.
+ *   SRW_FAULT_TIMEOUT a fold launch (single-point GEMV or tensor-core fold) or
+ *                     a matrix product of a surrogate's inference (three
+ *                     hidden layers and the output) makes one wait wait on
+ *                     an mbarrier that nothing arrives on, with a 1 ms limit;
+ *                     the wait gives up and the kernel takes its abort path:
+ *                     the affected points' values are NaN, host-pointer calls
+ *                     return SRW_ETIMEOUT, and a graph captured with the fault
+ *                     is run once, not cached.
  * SRW_FAULT_NONE disarms.  The environment variable SRW_FAULT ("alloc",
  * "launch" or "timeout", optionally ":N" for skip = N) arms a fault once per
  * process, before the first library call that allocates or launches; an

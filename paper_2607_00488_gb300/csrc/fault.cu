@@ -6,7 +6,8 @@
 //            cudaErrorMemoryAllocation (the entry point returns SRW_ENOMEM);
 //   launch:  the selected launch check reports cudaErrorLaunchFailure (the
 //            entry point returns SRW_ECUDA; a graph being captured is dropped);
-//   timeout: the selected fold launch makes one of its waits wait on an
+//   timeout: the selected fold launch (or matrix product of a surrogate's
+//            inference) makes one of its waits wait on an
 //            mbarrier that nothing arrives on, with a 1 ms limit; the wait
 //            gives up and the kernel takes the same abort path as a producer
 //            that never delivers (status bit, NaN results for the affected

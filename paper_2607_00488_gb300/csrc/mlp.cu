@@ -80,6 +80,7 @@ struct EpiArgs {
   // scan: per tile of 128 bins the rows m_j + s_j b_j, s_j, -n_j and n_j ln n_j - n_j (masked bins: 0, 0, 0, -1)
   const float* binc;
   double* parts;         // scan: partial sums of the deviance, or its parts (mlp_scan_kernel)
+  int inject;            // inference: injected timeout (host-side fault injection), CTA 0's epilogue gives up
 };
 
 // What one training step differs in from the next (device memory, written by
@@ -138,7 +139,7 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   // (a round trip through an integer makes them generic loads: slower, and on
   // the long scoreboard)
   unsigned char* smem = dsmem_raw + ((1024u - (ptx::smem_addr(dsmem_raw) & 1023u)) & 1023u);
-  __shared__ __align__(8) uint64_t full[ST], empty[ST], acc_full[2], acc_empty[2], drain;
+  __shared__ __align__(8) uint64_t full[ST], empty[ST], acc_full[2], acc_empty[2], drain, never;
   __shared__ uint32_t tmem_slot;
   __shared__ unsigned abort_flag;
 
@@ -159,6 +160,7 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       ptx::mbar_init(&acc_empty[b], kEpiWarps);
     }
     ptx::mbar_init(&drain, 1);
+    ptx::mbar_init(&never, 1);  // nothing arrives on it (injected timeout)
     abort_flag = 0u;
     ptx::fence_barrier_init();
   }
@@ -255,10 +257,19 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     // ------------------------------------------------------------ epilogue
     const int q = warp & 3;                  // TMEM lanes 32 q .. 32 q + 31
     const int part = (warp - 2) >> 2;        // columns [part kSpan, (part + 1) kSpan)
+    // inference: once this CTA has given up, the outputs that it has not written
+    // become NaN, and with them the values of the affected points, which would
+    // otherwise be formed from an earlier call's (training reports the timeout)
+    constexpr bool kMark = MODE == kFwdHiddenScan || MODE == kFwdOut;
+    bool dead = false;
+    if (kMark && E.inject && blockIdx.x == 0 && warp == 2 &&
+        !__all_sync(0xffffffffu, ptx::mbar_wait(&never, 0, &abort_flag, 1000000ull)))
+      give_up();
     int tc = -1;
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
       ++tc;
-      if (__any_sync(0xffffffffu, aborted(&abort_flag))) break;
+      if (!dead && __any_sync(0xffffffffu, aborted(&abort_flag))) dead = true;
+      if (dead && !kMark) break;
       const int m0 = (t / n_tn) * kBM, n0 = (t % n_tn) * BN;
       const int buf = tc & 1;
       const int m = m0 + q * 32 + lane;
@@ -274,9 +285,20 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         for (int k = 0; k < 4; ++k) ahead[k] = MODE == kBwdData || row_on ? __ldg(p + k) : make_float4(0.f, 0.f, 0.f, 0.f);
       };
       if (MODE == kFwdOutFit || MODE == kBwdData) fetch(part * kSpan);
-      if (!warp_wait(&acc_full[buf], (tc >> 1) & 1, &abort_flag)) {
+      if (!dead && !warp_wait(&acc_full[buf], (tc >> 1) & 1, &abort_flag)) {
         give_up();
-        break;
+        dead = true;
+        if (!kMark) break;
+      }
+      if (kMark && dead) {
+        float nan[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) nan[k] = __int_as_float(0x7fc00000);
+        for (int c0 = part * kSpan; c0 < (part + 1) * kSpan; c0 += 16) {
+          if (MODE == kFwdOut) store_f32x16(E.out_f32 + (size_t)m * N + n0 + c0, nan);
+          else store_bf16x16(E.out_bf + (size_t)m * N + n0 + c0, nan);
+        }
+        continue;
       }
       tc_fence_after();
       const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
@@ -409,7 +431,7 @@ mlp_scan_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   extern __shared__ unsigned char dsmem_raw[];
   unsigned char* smem = dsmem_raw + ((1024u - (ptx::smem_addr(dsmem_raw) & 1023u)) & 1023u);
   __shared__ __align__(8) uint64_t a_full[kScanKb], a_empty[kScanKb], b_full[kScanRing], b_empty[kScanRing];
-  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], c_full[2], c_empty[2], drain;
+  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], c_full[2], c_empty[2], drain, never;
   __shared__ uint32_t tmem_slot;
   __shared__ unsigned abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -434,6 +456,7 @@ mlp_scan_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       ptx::mbar_init(&c_empty[b], kScanWarps);
     }
     ptx::mbar_init(&drain, 1);
+    ptx::mbar_init(&never, 1);  // nothing arrives on it (injected timeout)
     abort_flag = 0u;
     ptx::fence_barrier_init();
   }
@@ -535,14 +558,18 @@ mlp_scan_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
   } else {
     const int q = warp & 3, part = (warp - 2) >> 2;  // lanes 32 q ..; bins 32 part .. of a tile
+    if (E.inject && blockIdx.x == 0 && warp == 2 &&
+        !__all_sync(0xffffffffu, ptx::mbar_wait(&never, 0, &abort_flag, 1000000ull)))
+      give_up();
     int tc = 0;
     bool ok = true;
-    for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+    for (int u = blockIdx.x; u < units; u += gridDim.x) {
       const int m = (u / groups) * kScanRows + q * 32 + lane, t0 = (u % groups) * tiles;
       tfloat total[2] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
       dfloat dev[2] = {{0.f, 0.f}, {0.f, 0.f}};
       bool infinite[2] = {false, false};
-      for (int t = 0; t < tiles; ++t, ++tc) {
+      if (__any_sync(0xffffffffu, aborted(&abort_flag))) ok = false;
+      for (int t = 0; t < tiles && ok; ++t, ++tc) {
         const int buf = tc & 1;
         if (!warp_wait(&c_full[buf], (tc >> 1) & 1, &abort_flag) ||
             !warp_wait(&acc_full[buf], (tc >> 1) & 1, &abort_flag)) {
@@ -605,7 +632,23 @@ mlp_scan_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           }
         }
       }
-      if (!ok) break;
+      if (!ok) {
+        // once this CTA has given up, a partial sum of every point that it has
+        // not finished becomes NaN: no value is formed from an earlier call's sums
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (m + h * kBM < E.rows_valid) {
+            if (RAW)
+              reinterpret_cast<float*>(E.parts)[(size_t)((t0 * 4 + part) * 2) * E.rows_valid + m + h * kBM] =
+                  __int_as_float(0x7fc00000);
+            else if (groups > 1)
+              reinterpret_cast<float2*>(E.parts)[(size_t)(t0 / kScanRun * 4 + part) * E.rows_valid + m + h * kBM] =
+                  make_float2(__int_as_float(0x7fc00000), 0.f);
+            else
+              E.parts[(size_t)part * E.rows_valid + m + h * kBM] = __longlong_as_double(0x7ff8000000000000LL);
+          }
+        continue;
+      }
       if constexpr (!RAW) {
         if (groups > 1) continue;
 #pragma unroll
@@ -1140,7 +1183,9 @@ int scan_parts(int N, int groups) {
   return 4 * (groups == 1 ? 1 : scan_raw(N, groups) ? tiles : (tiles + kScanRun - 1) / kScanRun);
 }
 
-cudaError_t run_gemm(const Gemm& g, int sm_count, unsigned* status, cudaStream_t s, bool dep = false) {
+cudaError_t run_gemm(const Gemm& gemm, int sm_count, unsigned* status, cudaStream_t s, bool dep = false) {
+  Gemm g = gemm;
+  if (g.mode == kFwdHiddenScan || g.mode == kFwdOut || g.mode == kFwdScan) g.E.inject = inject_timeout();
   if (g.mode == kWgrad) return launch_mode<64, kWgrad>(g, sm_count, status, s, dep);
   if (g.mode == kFwdScan) {
     const int groups = scan_groups(g.M, g.N, sm_count), units = g.M / kScanRows * groups;

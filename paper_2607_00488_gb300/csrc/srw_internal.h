@@ -272,7 +272,7 @@ inline cudaError_t launch_result() {
   if (e == cudaSuccess && fault_fire(SRW_FAULT_LAUNCH)) return cudaErrorLaunchFailure;
   return e;
 }
-// 1 when this fold launch is to take an injected timeout (SRW_FAULT_TIMEOUT).
+// 1 when this fold launch (or product of a surrogate's inference) is to take an injected timeout (SRW_FAULT_TIMEOUT).
 inline int inject_timeout() { return fault_fire(SRW_FAULT_TIMEOUT) ? 1 : 0; }
 
 srw_status fail(srw_ctx* h, srw_status s, const std::string& msg);

@@ -214,3 +214,30 @@ def test_fp32_batch_with_very_many_bins(srw):
         want = 2.0 * np.sum(mu - xlogy(counts, mu) + gammaln(counts + 1.0))
         # FP32 products of R with the deviation from the reference: 2^-23 of each
         assert abs(v - want) <= 2.0 * np.sum(np.abs(1.0 - counts / mu) * np.abs(mu - ref)) * 2.0**-23
+
+
+# A device wait that runs out in a surrogate pass: no value, never an earlier call's.
+@pytest.mark.parametrize("skip", [0, 1, 2, 3])
+@pytest.mark.parametrize("p", [300, 3000])
+def test_surrogate_timeout_gives_no_value(srw, p, skip):
+    from workloads.mlp import BOX_CENTRE, BOX_HALF, init_weights
+    wl = line(64, 300)
+    _, counts = oracle_of(wl)
+    with srw.Likelihood(wl, counts) as lk, srw.Surrogate(lk, init_weights(300, seed=5), BOX_CENTRE, BOX_HALF) as s:
+        theta = workloads.theta_box(p, 43)
+        other = workloads.theta_box(p, 44)
+        want = s.loglik(theta)
+        s.loglik(other)  # the buffers hold another call's partial sums
+        dev, out = torch.from_numpy(theta).cuda(), torch.zeros(p, dtype=torch.float64, device="cuda")
+        srw.srw_fault_inject("timeout", skip)  # one of the pass's four kernels
+        s.loglik(dev, out=out)
+        torch.cuda.synchronize()
+        assert srw.srw_fault_pending() == 0
+        got = out.cpu().numpy()
+        bad = np.isnan(got)
+        assert bad.any()
+        np.testing.assert_array_equal(got[~bad], want[~bad])
+        with pytest.raises(srw.SrwError) as ei:  # the next host call reads and clears the status
+            s.loglik(other)
+        assert ei.value.status == 6  # SRW_ETIMEOUT
+        np.testing.assert_array_equal(s.loglik(theta), want)
