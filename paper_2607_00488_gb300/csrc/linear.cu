@@ -112,19 +112,21 @@ __device__ __forceinline__ void deviations(const float* th, dfloat s, const Coef
   g = Couplings{gle.hi + gle.lo, gre.hi + gre.lo, glt.hi + glt.lo, grt.hi + grt.lo, th[4]};
 }
 
-// n / mu of N points in a bin with data; the scaled division where some point
-// of the warp has a tiny mu.
+// n / mu of N points in a bin with data.  A tiny mu takes CUDA's fast division
+// instead, and only that quotient does: which other points and bins share a warp
+// does not touch a value.
 template <int N>
 __device__ __forceinline__ void quotients(float n, const float* mu, float* q) {
   bool fine = true;
 #pragma unroll
-  for (int i = 0; i < N; ++i) fine = fine && !(fabsf(mu[i]) < 1e-30f);
-  if (__all_sync(0xffffffffu, fine)) {
+  for (int i = 0; i < N; ++i) {
+    q[i] = quotient(n, mu[i]);
+    fine = fine && !(fabsf(mu[i]) < 1e-30f);
+  }
+  if (!__all_sync(0xffffffffu, fine)) {
 #pragma unroll
-    for (int i = 0; i < N; ++i) q[i] = quotient(n, mu[i]);
-  } else {
-#pragma unroll
-    for (int i = 0; i < N; ++i) q[i] = __fdividef(n, mu[i]);
+    for (int i = 0; i < N; ++i)
+      if (fabsf(mu[i]) < 1e-30f) q[i] = __fdividef(n, mu[i]);
   }
 }
 
@@ -213,7 +215,8 @@ __device__ __forceinline__ void deviance_bins(const Vf<2>* d, const Vf<2>* s, co
 #pragma unroll
     for (int k = 0; k < K; ++k)
 #pragma unroll
-      for (int i = 0; i < 2; ++i) q[k][i] = __fdividef(n[k], mu[k][i]);
+      for (int i = 0; i < 2; ++i)
+        if (fabsf(mu[k][i]) < 1e-30f) q[k][i] = __fdividef(n[k], mu[k][i]);
   if (!__all_sync(0xffffffffu, all_near))
 #pragma unroll
     for (int k = 0; k < K; ++k) {
@@ -667,7 +670,8 @@ linear_profiled_kernel(const float* __restrict__ theta, int P, dfloat sin2w, Coe
 #pragma unroll
             for (int u = 0; u < K; ++u)
 #pragma unroll
-              for (int k = 0; k < 2; ++k) x[u][k] = __fdividef(n[u], mu[u][k]);
+              for (int k = 0; k < 2; ++k)
+                if (fabsf(mu[u][k]) < 1e-30f) x[u][k] = __fdividef(n[u], mu[u][k]);
 #pragma unroll
           for (int u = 0; u < K; ++u) {
             float *a = split_term<L>(terms, r & 1, 0, S.q, S.i0 + u) + S.pt;
@@ -727,7 +731,7 @@ linear_profiled_kernel(const float* __restrict__ theta, int P, dfloat sin2w, Coe
     const int rounds = (cnt + kSplitRound - 1) / kSplitRound;
     for (int r = 0; r <= rounds; ++r) {
       if (r < rounds) {
-Vf<2> d[K], sm[K];
+        Vf<2> d[K], sm[K];
         float n[K], mu[K][2], m[K][2], q[K][2], t[K][2];
         bool on[K];
 #pragma unroll

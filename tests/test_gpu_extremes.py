@@ -193,6 +193,27 @@ def test_surrogate_value_independent_of_the_batch(srw, n_rec):
             np.testing.assert_array_equal(s.loglik(theta[:p]), v[:p])
 
 
+# Rank 8: an empty bin with a subnormal expectation shares the warps' rounds with
+# ordinary bins; the value of a point does not depend on the path of its batch.
+@pytest.mark.parametrize("n_rec", [65, 257])
+def test_rank8_empty_bins_beside_ordinary_ones(srw, n_rec):
+    wl = line(50, n_rec)
+    r, bkg = wl["R"].copy(), wl["bkg"].copy()
+    _, counts = oracle_of(wl)
+    for j in range(1, n_rec, 9):
+        r[j], bkg[:, j], counts[j] = 0.0, 1e-35, 0.0
+    wl.update(R=r, bkg=bkg)
+    theta = workloads.fit_region_points(19456, seed=5)
+    with srw.Likelihood(wl, counts) as lk:
+        v, g = lk.loglik_linear(theta, grad=True)
+        assert np.all(np.isfinite(v)) and np.all(np.isfinite(g))
+        np.testing.assert_array_equal(lk.loglik_linear(theta), v)
+        for p in (1, 16, 2433, 9728):
+            v1, g1 = lk.loglik_linear(theta[:p], grad=True)
+            np.testing.assert_array_equal(v1, v[:p])
+            np.testing.assert_array_equal(g1, g[:p])
+
+
 # Two million reconstructed bins: more rows than a grid's y dimension holds in tiles of 32.
 def test_fp32_batch_with_very_many_bins(srw):
     from scipy.special import gammaln, xlogy
