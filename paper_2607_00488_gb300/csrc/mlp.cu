@@ -1421,7 +1421,10 @@ srw_status get_batch(srw_surrogate s, int M, bool train, SurrogateBatch** out) {
   const int bn_h = srw::pick_tile(M, H, s->sm_count), bn_o = srw::pick_tile(M, NO, s->sm_count);
   const int groups = srw::scan_groups(M, NO, s->sm_count);
   if (e == cudaSuccess) e = salloc(&B->parts, (size_t)srw::scan_parts(NO, groups) * M);
-  if (e == cudaSuccess) e = cudaMemset(B->x, 0, sizeof(__nv_bfloat16) * (size_t)M * srw::kInPad);
+  // done before the call's first kernel, which may run on any stream (the default
+  // stream's order does not hold the non-blocking ones)
+  if (e == cudaSuccess) e = cudaMemsetAsync(B->x, 0, sizeof(__nv_bfloat16) * (size_t)M * srw::kInPad, s->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e == cudaSuccess) e = salloc(&B->loss, 1);
   if (train) {
     for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = salloc(&B->gz[k], (size_t)M * H);
@@ -1699,10 +1702,10 @@ srw_status upload_weights(srw_surrogate s, const float* const* w) {
       if (!std::isfinite(x)) return sfail(s, SRW_EINVAL, "weights must be finite");
     S_CUDA(s, cudaMemcpy(L.w, W.data(), sizeof(float) * W.size(), cudaMemcpyHostToDevice), "upload weights");
     S_CUDA(s, cudaMemcpy(L.b, b.data(), sizeof(float) * b.size(), cudaMemcpyHostToDevice), "upload biases");
-    S_CUDA(s, cudaMemset(L.mw, 0, sizeof(float) * W.size()), "adam state");
-    S_CUDA(s, cudaMemset(L.vw, 0, sizeof(float) * W.size()), "adam state");
-    S_CUDA(s, cudaMemset(L.mb, 0, sizeof(float) * L.out), "adam state");
-    S_CUDA(s, cudaMemset(L.vb, 0, sizeof(float) * L.out), "adam state");
+    S_CUDA(s, cudaMemsetAsync(L.mw, 0, sizeof(float) * W.size(), s->stream), "adam state");
+    S_CUDA(s, cudaMemsetAsync(L.vw, 0, sizeof(float) * W.size(), s->stream), "adam state");
+    S_CUDA(s, cudaMemsetAsync(L.mb, 0, sizeof(float) * L.out, s->stream), "adam state");
+    S_CUDA(s, cudaMemsetAsync(L.vb, 0, sizeof(float) * L.out, s->stream), "adam state");
     S_CUDA(s, cudaMemsetAsync(L.gw, 0, sizeof(float) * W.size(), s->stream), "gradients");
     srw::cast_weights_kernel<<<(unsigned)((W.size() + 255) / 256), 256, 0, s->stream>>>(L.w, (int)W.size(), L.w_bf);
     S_CUDA(s, srw::launch_result(), "cast weights");

@@ -237,6 +237,24 @@ def test_fp32_batch_with_very_many_bins(srw):
         assert abs(v - want) <= 2.0 * np.sum(np.abs(1.0 - counts / mu) * np.abs(mu - ref)) * 2.0**-23
 
 
+# The first pass at a batch size fills its input buffer's padding and runs at once:
+# its values are those of the second pass (a fill of 256 MB is still on its way
+# when the next launch is made).
+def test_surrogate_first_pass_of_a_large_batch(srw):
+    from workloads.mlp import BOX_CENTRE, BOX_HALF, init_weights
+    wl = line(64, 100)
+    _, counts = oracle_of(wl)
+    theta = torch.from_numpy(workloads.theta_box(1 << 20, 43)).cuda()
+    with srw.Likelihood(wl, counts) as lk:
+        for _ in range(3):
+            with srw.Surrogate(lk, init_weights(100, seed=5), BOX_CENTRE, BOX_HALF) as s:
+                first, second = (torch.zeros(1 << 20, dtype=torch.float64, device="cuda") for _ in range(2))
+                s.loglik(theta, out=first)
+                s.loglik(theta, out=second)
+                torch.cuda.synchronize()
+                assert torch.equal(first, second)
+
+
 # A device wait that runs out in a surrogate pass: no value, never an earlier call's.
 @pytest.mark.parametrize("skip", [0, 1, 2, 3])
 @pytest.mark.parametrize("p", [300, 3000])
