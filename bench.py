@@ -389,7 +389,7 @@ def grouped_measurement(args, srw, workloads, dev, stream, flush, prec, peaks, p
                      "frac": dense / fold_s / 1e12 / peak, "kernel": "fold_tc_kernel (grouped)",
                      "flops_definition": "useful: sum over configurations of 2 N_rec N_T P",
                      "useful_tflop_per_launch": dense / 1e12, "fold_ms": statistics.mean(fold_ms),
-                     "frac_executed": useful * PRODUCTS[prec] / fold_s / 1e12 / peak,
+                     "frac_nonzero_blocks": useful * PRODUCTS[prec] / fold_s / 1e12 / peak,
                      "executed_block_fraction": useful / dense,
                      "peak_source": "%s bf16 dense burst" % peak_src},
         "schedule": {"candidate": cand, "bn_max": sched["bn_max"], "items": sched["n_items"], "ctas": sched["n_cta"],
@@ -429,12 +429,12 @@ def joint_measurement(args, srw, workloads, dev, stream, flush, prec, peaks, pea
            "fold_axis": info["n_t"], "points": args.points,
            "evals_s": args.points * args.steps / (sum(step_ms) * 1e-3), "ms_per_step": statistics.mean(step_ms),
            # the concatenated axis is 79 % exact-zero blocks (each component's band),
-           # so its dense-equivalent rate says little: the executed tensor-core work
-           # (three products on the nonzero blocks) is held to the peak
+           # so its dense-equivalent rate says little: three products on the nonzero
+           # blocks are held to the peak (whole blocks; their all-zero rows are not multiplied)
            "roofline": {"bound": "tensor", "achieved": dense * work * PRODUCTS[prec] / fold_s / 1e12, "peak": peak,
                         "unit": "TFLOP/s", "frac": dense * work * PRODUCTS[prec] / fold_s / 1e12 / peak,
                         "kernel": "fold_tc_kernel",
-                        "flops_definition": "executed: %d products x 2 N_rec K per point on the nonzero blocks"
+                        "flops_definition": "%d products x 2 N_rec K per point on the nonzero blocks, whole blocks"
                                             % PRODUCTS[prec],
                         "dense_equivalent_tflops": dense / fold_s / 1e12,
                         "executed_block_fraction": work, "fold_ms": statistics.mean(fold_ms),
@@ -490,7 +490,7 @@ def surrogate_measurement(args, srw, workloads, lk, peaks, peak_src):
         "same_minimum": bool(r["best_index"] == ex["best_index"] and r["best_value"] == ex["best_value"]),
         "gain": ex["ms"] / t_pre, "gain_vs_rank8": ex8["ms"] / t_pre,
         "roofline": {"bound": "tensor", "achieved": achieved, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
-                     "frac": achieved / peaks["bf16_tflops"], "kernel": "mlp_gemm_kernel (surrogate pass)",
+                     "frac": achieved / peaks["bf16_tflops"], "kernel": "mlp_gemm_kernel, mlp_scan_kernel (surrogate pass)",
                      "flop_per_point": flop_point, "peak_source": "%s (bf16 burst)" % peak_src},
     }
 
@@ -542,9 +542,10 @@ def fold_kernel_ms(srw, h, call, flush, steps):
 def fold_roofline(srw, lk, info, prec, prec_name, P, fold_ms, peaks, peak_src):
     """Roofline of the batched fold: useful flops 2 N_rec N_T per point (the
     dense contraction, whatever the kernel skips or repeats) over the kernel's
-    own device time, against the measured burst peak; beside it the executed
-    tensor-core work (products x executed (rec tile, K block) pairs, whole
-    blocks: their all-zero rows are left out of the MMAs, so this can exceed 1)."""
+    own device time, against the measured burst peak; beside it the rate on the
+    nonzero blocks: products x (rec tile, K block) pairs that are not all zeros,
+    counted whole.  The kernel leaves the all-zero rows of a block out of its
+    MMAs, so that figure is not the executed work and can exceed 1."""
     fold_s = statistics.mean(fold_ms) * 1e-3
     work = lk.fold_work(prec)
     dense = 2.0 * info["n_rec"] * info["n_t"] * P
@@ -557,12 +558,12 @@ def fold_roofline(srw, lk, info, prec, prec_name, P, fold_ms, peaks, peak_src):
         bound, kernel_file, tag = "tensor", "paper_2607_00488_gb300/csrc/fold_tc.cu", "fold_tc_kernel"
         note = "%s bf16 dense burst (fp16 runs at the same rate)" % peak_src
     achieved = dense / fold_s / 1e12
-    executed = dense * work * PRODUCTS[prec]
+    blocks = dense * work * PRODUCTS[prec]
     return {"bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": recorded_traffic(kernel_file, tag + ":" + prec_name), "kernel": tag, "peak_source": note,
             "flops_per_launch": dense, "flops_definition": "useful: 2 N_rec N_T per point",
             "fold_ms": statistics.mean(fold_ms), "fold_ms_sd": statistics.pstdev(fold_ms),
-            "executed_tflops": executed / fold_s / 1e12, "frac_executed": executed / fold_s / 1e12 / peak,
+            "nonzero_block_tflops": blocks / fold_s / 1e12, "frac_nonzero_blocks": blocks / fold_s / 1e12 / peak,
             "executed_block_fraction": work, "products_per_useful_flop": PRODUCTS[prec]}
 
 
@@ -673,7 +674,7 @@ def main():
         alt_name = {v: k for k, v in srw.PRECISIONS.items()}[alt_prec]
         a_roof = fold_roofline(srw, lk, info, alt_prec, alt_name, P, a_fold, peaks, peak_src)
         alt = {"precision": alt_name, "value": P * args.steps / (sum(a_ms) * 1e-3), "ms_per_step": statistics.mean(a_ms),
-               "fold_ms": a_roof["fold_ms"], "frac": a_roof["frac"], "frac_executed": a_roof["frac_executed"],
+               "fold_ms": a_roof["fold_ms"], "frac": a_roof["frac"], "frac_nonzero_blocks": a_roof["frac_nonzero_blocks"],
                "executed_block_fraction": a_roof["executed_block_fraction"],
                "autotune": autotune_record(srw, h, alt_prec)}
 

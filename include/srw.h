@@ -296,7 +296,8 @@ srw_status srw_get_fold_config(srw_handle h, srw_precision precision, int* index
  * runs only the range of true-bin blocks in which the split response has a
  * nonzero element; the skipped blocks hold zeros in both split operands, so
  * their products are exact zeros and skipping them changes no bit of the
- * result.  1 for SRW_FP32 (the SIMT fold runs every block). */
+ * result.  Inside a block the rows without nonzero elements are not multiplied
+ * either; the fraction counts whole blocks.  1 for SRW_FP32 (the SIMT fold runs every block). */
 srw_status srw_fold_work(srw_handle h, srw_precision precision, int tile, double* executed_fraction);
 
 /* Bytes of R the single-point fold (the GEMV of srw_loglik with P = 1 and

@@ -38,7 +38,7 @@ constexpr int kLinThreads = 128;              // a warp per residue of the rec b
 constexpr int kLinChunk = 256;                // rec bins per shared-memory chunk
 constexpr int kSplitThreads = 512;            // split kernels (few points): sixteen warps on a round of
 constexpr int kSplitRound = 64;               // 64 rec bins
-constexpr int kSplitChunk = 1024;             // 48 KB of constants beside 16 KB of terms
+constexpr int kSplitChunk = 1024;             // 48 KB of constants beside 16 KB of terms (L = 8; 32 KB at L = 16)
 constexpr int kProfChunk = 2048;              // 96 KB of constants, staged once up to this many bins
 
 // M_jb = sum_i R_ji shat_b,i with shat_b,i = B_b,i E_SM,i / S_SM,i (FP64); one
@@ -810,9 +810,17 @@ void launch_warps(const srw_ctx* h, const float* theta, int P, double* out, doub
 
 template <bool GRAD>
 void launch_linear(const srw_ctx* h, const float* theta, int P, double* out, double* grad, cudaStream_t s) {
-  if (P <= 16 * h->sm_count) launch_split<GRAD, 8>(h, theta, P, out, grad, s);  // at most one block an SM
-  // value only / with gradient, us, at 5000, 12,000 and 19,000 points: L = 16 68 / 108, 43 / 68, 90 / 143;
-  // a warp per residue with one point a lane 140 / 160, 57 / 66, 96 / 112, with two points 100 / 133 at 19,000
+  // The lines lie where the one side becomes the faster; the first two are also
+  // whole waves, one block of 16 points an SM (L = 8), then two of 32 (L = 16).
+  // us on 2048 bins, value only / with gradient, back to back:
+  //   points      L = 8      L = 16   one a lane   two a lane
+  //    2432     21 / 29     31 / 48     88 / 95     91 / 117
+  //    9727     54 / 107    48 / 75     91 / 98     92 / 118
+  //   12,000    66 / 132    71 / 111    93 / 103    98 / 128
+  //   19,000   101 / 208    91 / 144    99 / 111    99 / 129
+  //   40,000   207 / 437   195 / 311   194 / 220   140 / 189
+  // (Values alone from 2433 to about 7000 points would be 2 to 4 us faster at L = 8.)
+  if (P <= 16 * h->sm_count) launch_split<GRAD, 8>(h, theta, P, out, grad, s);
   else if (P < (GRAD ? 64 : 128) * h->sm_count) launch_split<GRAD, 16>(h, theta, P, out, grad, s);
   else if (GRAD && P < 128 * h->sm_count) launch_warps<true, 1>(h, theta, P, out, grad, s);
   else launch_warps<GRAD, 2>(h, theta, P, out, grad, s);
