@@ -1405,7 +1405,8 @@ cudaError_t prep(Gemm& g, const __nv_bfloat16* A, const __nv_bfloat16* B, int M,
 }
 
 // Buffers and prepared products for batch size M (multiple of 128).
-srw_status get_batch(srw_surrogate s, int M, bool train, SurrogateBatch** out) {
+// st: the stream of the call that asks for it.
+srw_status get_batch(srw_surrogate s, int M, bool train, cudaStream_t st, SurrogateBatch** out) {
   for (SurrogateBatch* B : s->batches)
     if (B->M == M && (B->train || !train)) {
       *out = B;
@@ -1421,10 +1422,8 @@ srw_status get_batch(srw_surrogate s, int M, bool train, SurrogateBatch** out) {
   const int bn_h = srw::pick_tile(M, H, s->sm_count), bn_o = srw::pick_tile(M, NO, s->sm_count);
   const int groups = srw::scan_groups(M, NO, s->sm_count);
   if (e == cudaSuccess) e = salloc(&B->parts, (size_t)srw::scan_parts(NO, groups) * M);
-  // done before the call's first kernel, which may run on any stream (the default
-  // stream's order does not hold the non-blocking ones)
-  if (e == cudaSuccess) e = cudaMemsetAsync(B->x, 0, sizeof(__nv_bfloat16) * (size_t)M * srw::kInPad, s->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+  // on the call's stream: the default stream's order does not hold the non-blocking ones
+  if (e == cudaSuccess) e = cudaMemsetAsync(B->x, 0, sizeof(__nv_bfloat16) * (size_t)M * srw::kInPad, st);
   if (e == cudaSuccess) e = salloc(&B->loss, 1);
   if (train) {
     for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = salloc(&B->gz[k], (size_t)M * H);
@@ -1648,7 +1647,7 @@ srw_status loglik_device(srw_surrogate s, const float* theta, long long P, T* ou
     const int rows = (int)std::min<long long>(kScanChunk, P - off);
     SurrogateBatch* B = nullptr;
     const int M = round_up(rows, srw::kScanRows);
-    srw_status r = get_batch(s, M < 65536 ? M : round_up(rows, 65536), false, &B);
+    srw_status r = get_batch(s, M < 65536 ? M : round_up(rows, 65536), false, st, &B);
     if (r != SRW_OK) return r;
     cudaError_t e = forward_hidden(s, theta + off * 5, rows, B, st);
     if (e == cudaSuccess) {
@@ -1820,7 +1819,7 @@ srw_status srw_surrogate_forward(srw_surrogate s, const float* theta, int P, flo
   if (!s || !theta || !y || P < 1) return SRW_EINVAL;
   const int M = round_up(P, srw::kBM);
   SurrogateBatch* B = nullptr;
-  srw_status st = get_batch(s, M, false, &B);
+  srw_status st = get_batch(s, M, false, s->stream, &B);
   if (st != SRW_OK) return st;
   CallBuf<float> th;
   S_CUDA(s, salloc_async(&th, (size_t)5 * P, s->stream), "alloc");
@@ -1849,7 +1848,7 @@ srw_status srw_surrogate_gradients(srw_surrogate s, const float* theta, const fl
   if (!s || !theta || !targets || !grads || P < 1) return SRW_EINVAL;
   const int M = round_up(P, srw::kBM);
   SurrogateBatch* B = nullptr;
-  srw_status st = get_batch(s, M, true, &B);
+  srw_status st = get_batch(s, M, true, s->stream, &B);
   if (st != SRW_OK) return st;
   CallBuf<float> th, tg;
   S_CUDA(s, salloc_async(&th, (size_t)5 * P, s->stream), "alloc");
@@ -1890,7 +1889,7 @@ srw_status srw_surrogate_train_step(srw_surrogate s, const float* theta, const f
   if (!s || !theta || !targets || P < 1 || !(lr > 0.f)) return SRW_EINVAL;
   const int M = round_up(P, srw::kBM);
   SurrogateBatch* B = nullptr;
-  srw_status st = get_batch(s, M, true, &B);
+  srw_status st = get_batch(s, M, true, s->stream, &B);
   if (st != SRW_OK) return st;
   CallBuf<float> th, tg;
   S_CUDA(s, salloc_async(&th, (size_t)5 * P, s->stream), "alloc");
@@ -1972,7 +1971,7 @@ static srw_status fit_impl(srw_surrogate s, const float* theta, long long n, con
     return scuda(s, e, "targets");
   }
   SurrogateBatch* B = nullptr;
-  srw_status r = get_batch(s, M, true, &B);
+  srw_status r = get_batch(s, M, true, st, &B);
   if (r != SRW_OK) {
     cleanup();
     return r;
