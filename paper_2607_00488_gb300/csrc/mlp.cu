@@ -7,8 +7,8 @@
 //   y  = W4 h3 + b4,   log mu_j = m_j + s_j y_j             (n_rec outputs, padded to 256)
 //
 // gelu(z) = z Phi(z) (erf form).  Training: mean squared error of y against
-// standardized targets, Adam with FP32 master weights and BF16 copies of W and
-// W^T for the tensor cores.
+// standardized targets, Adam with FP32 master weights and BF16 copies for the
+// tensor cores.
 //
 // Every matrix product is one persistent tcgen05 GEMM (BF16, 128-byte swizzle,
 // TMA-fed, FP32 accumulation in double-buffered TMEM) with an epilogue fused
@@ -817,8 +817,9 @@ __device__ __forceinline__ double widen(float x) {
 // sum and sum of squares of this block's kStatRows rows, in row order, in the
 // block's own slot (no atomics: the statistics, and so every resumed fit, are
 // the same bit for bit whatever the order in which the blocks run).  A thread
-// is a column.  Bound by the FP64 unit: two operations an element, 0.45 ms for
-// 65,536 x 2048 (a pass for the logarithm and one for the sums: 0.45 + 0.99 ms).
+// is a column.  The FP64 unit's two operations an element alone take 0.43 ms for
+// 65,536 x 2048; 0.89 ms in all (a pass for the logarithm and one for the sums:
+// 0.45 + 0.98 ms; cold, one launch at a time).
 constexpr int kStatRows = 4096;
 __global__ void __launch_bounds__(64, 8)
 log_stats_kernel(const float* src, long long rows, int n, int ld, const double* __restrict__ b64, float* dst,
