@@ -314,7 +314,8 @@ typedef struct {
   int n_t, n_rec, n_nodes, k_pad;
   int device, sm_count, tensor_path;   /* tensor_path: 1 if the tcgen05 fold can run */
   double lambda;                        /* E_SM = lambda * S_SM normalisation (0 if e_true_sm given) */
-  size_t device_bytes;                  /* persistent device memory held by the context */
+  size_t device_bytes;                  /* persistent device memory held by the context (beside it, from the
+                                         * first host-pointer call on, 512 KB of page-locked host memory) */
 } srw_info_t;
 srw_status srw_info(srw_handle h, srw_info_t* info);
 

@@ -256,13 +256,14 @@ def test_surrogate_first_pass_of_a_large_batch(srw):
 
 
 # A device wait that runs out in a surrogate pass: no value, never an earlier call's.
+# The sizes give each form of the partial sums: of short units, of runs, of quarters.
 @pytest.mark.parametrize("skip", [0, 1, 2, 3])
-@pytest.mark.parametrize("p", [300, 3000])
-def test_surrogate_timeout_gives_no_value(srw, p, skip):
+@pytest.mark.parametrize("n_rec,p", [(300, 300), (300, 3000), (2048, 20000), (100, 100000)])
+def test_surrogate_timeout_gives_no_value(srw, n_rec, p, skip):
     from workloads.mlp import BOX_CENTRE, BOX_HALF, init_weights
-    wl = line(64, 300)
+    wl = line(64, n_rec)
     _, counts = oracle_of(wl)
-    with srw.Likelihood(wl, counts) as lk, srw.Surrogate(lk, init_weights(300, seed=5), BOX_CENTRE, BOX_HALF) as s:
+    with srw.Likelihood(wl, counts) as lk, srw.Surrogate(lk, init_weights(n_rec, seed=5), BOX_CENTRE, BOX_HALF) as s:
         theta = workloads.theta_box(p, 43)
         other = workloads.theta_box(p, 44)
         want = s.loglik(theta)
