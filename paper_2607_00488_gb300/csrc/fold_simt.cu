@@ -8,7 +8,7 @@
 // block produces its W tile on chip from shat and the 8 coefficients of its
 // points, so W is never written to memory.  The epilogue adds the summed
 // background, applies the mask, evaluates the Poisson terms and reduces over
-// its rec bins per point into FP64 partials (one per rec tile).  The fold is
+// its rec bins per point into FP64 partials (one per 64 bins).  The fold is
 // taken of W(theta) - W_ref; the FP64 reference fold R W_ref enters with the
 // background (b64 argument = background + reference fold).
 //
@@ -43,7 +43,7 @@ constexpr int kNC = kNB - 1;  // monomials of a point's deviation (the constant 
 //   <2, 2>: 64 points x 128 bins.  A thread's 8 x 8 outputs take four 128-bit
 //           shared loads per 64 FMAs, half of the 4 x 8 outputs' six, which
 //           kept the kernel at the shared-memory limit (26 % of the FP32 rate);
-//           with 240 registers two blocks of four warps share an SM, and the
+//           with 255 registers two blocks of four warps share an SM, and the
 //           one's epilogue and W production run beside the other's FMAs.
 //   <1, 1>: 32 points x 64 bins, for grids of fewer large tiles than SMs.
 template <int MI, int NI>
